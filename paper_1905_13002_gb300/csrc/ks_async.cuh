@@ -38,6 +38,12 @@ KS_DEV void bulk_wait_read_all() { asm volatile("cp.async.bulk.wait_group.read 0
 // Wait until every committed bulk store has completed.
 KS_DEV void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
+// 4-byte asynchronous copies of single words (any 4-byte alignment).
+KS_DEV void cp_async4(void* sdst, const void* gsrc) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(smem_addr(sdst)), "l"(gsrc) : "memory");
+}
+KS_DEV void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 KS_DEV void mbar_init(uint64_t* m, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(smem_addr(m)), "r"(count) : "memory");
 }

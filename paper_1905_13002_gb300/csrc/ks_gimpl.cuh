@@ -14,6 +14,7 @@ struct GImpl {
     using SM = grp::GSmem<N, M, NW>;
     static constexpr int NG = SM::NG;                      // chains per tile (one lane group each)
     static constexpr int64_t TILE = (int64_t)NG * CH;
+    static constexpr bool kSettled = N <= 8;   // ks_steady.cuh is compiled for this size
 
     static size_t prep_smem() { return sizeof(PrepSmem<N, M>) + sizeof(ModelConst<N, M>) + 16; }
 
@@ -27,6 +28,8 @@ struct GImpl {
         size_t off = 256;
         L.off_const = off;
         off = align_up(off + sizeof(ModelConst<N, M>) * (size_t)B, 256);
+        L.off_plan = off;                                   // one SteadyPlan per segment
+        if (kSettled) off = align_up(off + sizeof(SteadyPlan<N, M>) * (size_t)B, 256);
         L.off_flags = off;                                  // zeroed by the preparation kernel
         L.flags_bytes = 16;
         off = align_up(off + L.flags_bytes, 256);
@@ -52,6 +55,9 @@ struct GImpl {
 
     static ModelConst<N, M>* mconst(void* ws, const Layout& L) {
         return reinterpret_cast<ModelConst<N, M>*>(static_cast<char*>(ws) + L.off_const);
+    }
+    static SteadyPlan<N, M>* plan(void* ws, const Layout& L) {
+        return reinterpret_cast<SteadyPlan<N, M>*>(static_cast<char*>(ws) + L.off_plan);
     }
     static uint32_t* status(void* ws) { return static_cast<uint32_t*>(ws); }
 
@@ -88,9 +94,12 @@ struct GImpl {
     }
 
     // Per scan: a reduce launch, log2(tiles) spine launches, an apply launch.
+    // gate: null, or the workspace header when the scans stand behind the
+    // settled path.
     template <bool SEG, bool TV = false>
     static int scans(void* ws, const Layout& L, const float* y, float* fm, float* fc, float* sm, float* sc,
-                     Segs<N, M> segs, cudaStream_t st, void* const* ev, bool filter, bool smoother) {
+                     Segs<N, M> segs, cudaStream_t st, void* const* ev, bool filter, bool smoother,
+                     const uint32_t* gate = nullptr) {
         grp::GBuf fb, sb;
         buffers(ws, L, fb, sb);
         constexpr int smem = SM::BYTES;
@@ -105,19 +114,22 @@ struct GImpl {
             auto ka = grp::gfilter_apply_kernel<N, M, NW, CH, SEG, TV>;
             static const bool ok = allow_smem(kr, smem) && allow_smem(ks, ssmem) && allow_smem(ka, smem);
             if (!ok) return KS_ECUDA;
-            kr<<<L.ntf, NW * 32, smem, st>>>(mconst(ws, L), y, L.T, fb, stat, segs);
-            if ((rc = launch_status())) return rc;
+            rc = launch_gated(kr, L.ntf, NW * 32, smem, st, gate,
+                              mconst(ws, L), y, L.T, fb, stat, segs);
+            if (rc) return rc;
             const float* src = fb.spine0;
             float* dst = fb.spine1;
             for (int s = 1; s < L.ntf; s <<= 1) {
-                ks<<<(L.ntf + SG - 1) / SG, SW * 32, ssmem, st>>>(src, dst, L.ntf, s, stat);
-                if ((rc = launch_status())) return rc;
+                rc = launch_gated(ks, (L.ntf + SG - 1) / SG, SW * 32, ssmem, st, gate,
+                                  src, dst, L.ntf, s, stat);
+                if (rc) return rc;
                 float* t = const_cast<float*>(src);
                 src = dst;
                 dst = t;
             }
-            ka<<<L.ntf, NW * 32, smem, st>>>(mconst(ws, L), y, L.T, fm, fc, fb, src, stat, segs);
-            if ((rc = launch_status())) return rc;
+            rc = launch_gated(ka, L.ntf, NW * 32, smem, st, gate,
+                              mconst(ws, L), y, L.T, fm, fc, fb, src, stat, segs);
+            if (rc) return rc;
         }
         if (ev && ev[2] && record_event(ev[2], st) != cudaSuccess) return KS_ECUDA;
         if (smoother) {
@@ -126,21 +138,63 @@ struct GImpl {
             auto ka = grp::gsmoother_apply_kernel<N, M, NW, CH>;
             static const bool ok = allow_smem(kr, smem) && allow_smem(ks, ssmem) && allow_smem(ka, smem);
             if (!ok) return KS_ECUDA;
-            kr<<<L.nts, NW * 32, smem, st>>>(mconst(ws, L), fm, fc, L.T, sb, stat, segs);
-            if ((rc = launch_status())) return rc;
+            rc = launch_gated(kr, L.nts, NW * 32, smem, st, gate,
+                              mconst(ws, L), fm, fc, L.T, sb, stat, segs);
+            if (rc) return rc;
             const float* src = sb.spine0;
             float* dst = sb.spine1;
             for (int s = 1; s < L.nts; s <<= 1) {
-                ks<<<(L.nts + SG - 1) / SG, SW * 32, ssmem, st>>>(src, dst, L.nts, s, stat);
-                if ((rc = launch_status())) return rc;
+                rc = launch_gated(ks, (L.nts + SG - 1) / SG, SW * 32, ssmem, st, gate,
+                                  src, dst, L.nts, s, stat);
+                if (rc) return rc;
                 float* t = const_cast<float*>(src);
                 src = dst;
                 dst = t;
             }
-            ka<<<L.nts, NW * 32, smem, st>>>(L.T, sm, sc, sb, src, stat);
-            if ((rc = launch_status())) return rc;
+            if ((rc = launch_gated(ka, L.nts, NW * 32, smem, st, gate, L.T, sm, sc, sb, src, stat))) return rc;
         }
         return KS_OK;
+    }
+
+    // The fused call's kernels: the preparation, then the settled path with
+    // the scans gated behind it where its 16-byte row copies can be used, else
+    // the scans.
+    template <bool SEG>
+    static int fused(const float* F, const float* u, const float* Q, const float* H, const float* d, const float* R,
+                     const double* m0, const double* P0, const float* y, int B, const int64_t* off, void* ws,
+                     const Layout& L, float* fm, float* fc, float* sm, float* sc, bool keep, cudaStream_t st,
+                     void* const* ev) {
+        const bool smoother = sm != nullptr;
+        const uint32_t* gate = nullptr;
+        int rc;
+        if constexpr (kSettled) {
+            if (aligned16(fm) && aligned16(fc) && (!smoother || (aligned16(sm) && aligned16(sc)))) gate = status(ws);
+        }
+        if (gate == nullptr) {
+            rc = prep(F, u, Q, H, d, R, m0, P0, y, B, off, ws, L, st);
+            if (rc) return rc;
+        }
+        if constexpr (kSettled) {
+            if (gate != nullptr) {
+                PlanArgs<N, M> p{F, u, Q, H, d, R, m0, P0, y, mconst(ws, L), status(ws)};
+                p.zero = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + L.off_flags);
+                p.nzero = (int)(L.flags_bytes / 4);
+                p.off = off;
+                p.B = B;
+                p.T = L.T;
+                p.plan = plan(ws, L);
+                if ((rc = launch_plan_kernel(p, st))) return rc;
+            }
+        }
+        if (ev && ev[1] && record_event(ev[1], st) != cudaSuccess) return KS_ECUDA;
+        if constexpr (kSettled) {
+            if (gate != nullptr) {
+                const SteadyArgs<N, M> g{plan(ws, L), off, B, L.T, y, fm, fc, sm, sc, keep ? 1 : 0, status(ws)};
+                if ((rc = launch_steady_kernel(g, st))) return rc;
+            }
+        }
+        const Segs<N, M> segs{SEG ? mconst(ws, L) : nullptr, off, B};
+        return scans<SEG>(ws, L, y, fm, fc, sm, sc, segs, st, ev, true, smoother, gate);
     }
 
     static int check(const ks_model* m, int64_t T, void* ws, size_t ws_bytes, size_t need) {
@@ -234,10 +288,8 @@ struct GImpl {
             fc = reinterpret_cast<float*>(static_cast<char*>(ws) + L.off_fcov);
         }
         if (ev && ev[0] && record_event(ev[0], st) != cudaSuccess) return KS_ECUDA;
-        if ((rc = prep(m->F, m->u, m->Q, m->H, m->d, m->R, m->m0, m->P0, y, 1, nullptr, ws, L, st))) return rc;
-        if (ev && ev[1] && record_event(ev[1], st) != cudaSuccess) return KS_ECUDA;
-        if ((rc = scans<false>(ws, L, y, fm, fc, sm, sc, Segs<N, M>{nullptr, nullptr, 1}, st, ev, true,
-                               !filter_only)))
+        if ((rc = fused<false>(m->F, m->u, m->Q, m->H, m->d, m->R, m->m0, m->P0, y, 1, nullptr, ws, L, fm, fc,
+                               filter_only ? nullptr : sm, filter_only ? nullptr : sc, !own, st, ev)))
             return rc;
         if (ev && ev[3] && record_event(ev[3], st) != cudaSuccess) return KS_ECUDA;
         return KS_OK;
@@ -251,10 +303,8 @@ struct GImpl {
         const Layout L = layout(T, mb->B);
         if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0 || ws_bytes < L.bytes_smooth) return KS_EINVAL;
         if (!y || !fm || !fc || !sm || !sc) return KS_EINVAL;
-        int rc = prep(mb->F, mb->u, mb->Q, mb->H, mb->d, mb->R, mb->m0, mb->P0, y, mb->B, mb->offsets, ws, L, st);
-        if (rc) return rc;
-        return scans<true>(ws, L, y, fm, fc, sm, sc, Segs<N, M>{mconst(ws, L), mb->offsets, mb->B}, st, nullptr,
-                           true, true);
+        return fused<true>(mb->F, mb->u, mb->Q, mb->H, mb->d, mb->R, mb->m0, mb->P0, y, mb->B, mb->offsets, ws, L,
+                           fm, fc, sm, sc, true, st, nullptr);
     }
 
     static int no_comb(int64_t, const float*, const float*, float*, void*, cudaStream_t) { return KS_EUNSUPPORTED; }

@@ -101,7 +101,8 @@ constexpr int gspine_warps() {
 template <int N, int M, int NW, int CH, bool SEG, bool TV = false>
 __global__ void __launch_bounds__(NW * 32) gfilter_reduce_kernel(const ModelConst<N, M>* __restrict__ mcg,
                                                                  const float* __restrict__ y, int64_t T, GBuf gb,
-                                                                 uint32_t* status, Segs<N, M> segs) {
+                                                                 uint32_t* status, Segs<N, M> segs, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = GSmem<N, M, NW>;
     constexpr int FS = Dim<N>::FSLOT, NG = SM::NG;
     extern __shared__ __align__(16) char gsm[];
@@ -177,7 +178,8 @@ __global__ void __launch_bounds__(NW * 32) gfilter_reduce_kernel(const ModelCons
 // and C of the result are formed.
 template <int N, int NWS>
 __global__ void __launch_bounds__(NWS * 32) gspine_filter_kernel(const float* __restrict__ src, float* __restrict__ dst,
-                                                                 int ntiles, int s, uint32_t* status) {
+                                                                 int ntiles, int s, uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = GSpineSmem<N, NWS>;
     constexpr int FS = Dim<N>::FSLOT;
     constexpr int SLOT = GChain<N>::SLOT;
@@ -208,7 +210,8 @@ __global__ void __launch_bounds__(NW * 32) gfilter_apply_kernel(const ModelConst
                                                                 const float* __restrict__ y, int64_t T,
                                                                 float* __restrict__ fmean, float* __restrict__ fcov,
                                                                 GBuf gb, const float* __restrict__ pre,
-                                                                uint32_t* status, Segs<N, M> segs) {
+                                                                uint32_t* status, Segs<N, M> segs, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = GSmem<N, M, NW>;
     constexpr int FS = Dim<N>::FSLOT, NG = SM::NG;
     extern __shared__ __align__(16) char gsm[];
@@ -280,7 +283,8 @@ template <int N, int M, int NW, int CH, bool SEG, bool TV = false>
 __global__ void __launch_bounds__(NW * 32) gsmoother_reduce_kernel(const ModelConst<N, M>* __restrict__ mcg,
                                                                    const float* __restrict__ fmean,
                                                                    const float* __restrict__ fcov, int64_t T, GBuf gb,
-                                                                   uint32_t* status, Segs<N, M> segs) {
+                                                                   uint32_t* status, Segs<N, M> segs, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = GSmem<N, M, NW>;
     constexpr int SS = Dim<N>::SSLOT, NG = SM::NG;
     extern __shared__ __align__(16) char gsm[];
@@ -358,7 +362,8 @@ __global__ void __launch_bounds__(NW * 32) gsmoother_reduce_kernel(const ModelCo
 template <int N, int NWS>
 __global__ void __launch_bounds__(NWS * 32) gspine_smoother_kernel(const float* __restrict__ src,
                                                                    float* __restrict__ dst, int ntiles, int s,
-                                                                   uint32_t* status) {
+                                                                   uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = GSpineSmem<N, NWS>;
     constexpr int SS = Dim<N>::SSLOT;
     constexpr int SLOT = GChain<N>::SLOT;
@@ -387,7 +392,8 @@ __global__ void __launch_bounds__(NWS * 32) gspine_smoother_kernel(const float* 
 template <int N, int M, int NW, int CH>
 __global__ void __launch_bounds__(NW * 32) gsmoother_apply_kernel(int64_t T, float* __restrict__ smean,
                                                                   float* __restrict__ scov, GBuf gb,
-                                                                  const float* __restrict__ pre, uint32_t* status) {
+                                                                  const float* __restrict__ pre, uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = GSmem<N, M, NW>;
     constexpr int SS = Dim<N>::SSLOT, NG = SM::NG;
     extern __shared__ __align__(16) char gsm[];

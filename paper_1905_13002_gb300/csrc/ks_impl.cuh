@@ -9,6 +9,7 @@
 #include "../../include/ks.h"
 #include "ks_scan.cuh"
 #include "ks_shard.cuh"
+#include "ks_steady.cuh"
 
 namespace ks {
 
@@ -22,7 +23,7 @@ struct Layout {
     int64_t T = 0, ld = 0;
     int B = 1;
     int ntf = 0, nts = 0;
-    size_t off_const = 0, off_coef = 0, off_flags = 0, flags_bytes = 0;
+    size_t off_const = 0, off_coef = 0, off_plan = 0, off_flags = 0, flags_bytes = 0;
     size_t off_fagg = 0, off_fpre = 0, off_sagg = 0, off_spre = 0, off_sblk = 0;
     size_t off_elems = 0, off_fmean = 0, off_fcov = 0;
     size_t bytes_smooth = 0, bytes_elements = 0;
@@ -84,6 +85,17 @@ inline int launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem
     return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? KS_OK : KS_ECUDA;
 }
 
+// Launch of a scan kernel that takes a gate as its last argument: a plain
+// launch when it is null, else one chained behind the settled path (26 closed
+// kernels behind an nx = 8 batch: 272 us a call chained, 346 us plain).
+template <class... KArgs, class... Args>
+inline int launch_gated(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
+                        const uint32_t* gate, Args... args) {
+    if (gate != nullptr) return launch_pdl(kernel, grid, block, smem, st, args..., gate);
+    kernel<<<grid, block, smem, st>>>(args..., gate);
+    return launch_status();
+}
+
 // FCH_ = steps per thread of the block scans (one tile = 128 * FCH_ steps).
 template <int N, int M, int FCH_ = 32>
 struct Impl {
@@ -106,6 +118,8 @@ struct Impl {
         off = align_up(off + sizeof(ModelConst<N, M>) * (size_t)B, 256);
         L.off_coef = off;                                   // one BlockCoef per segment
         off = align_up(off + sizeof(BlockCoef<N, M>) * (size_t)B, 256);
+        L.off_plan = off;                                   // one SteadyPlan per segment
+        off = align_up(off + sizeof(SteadyPlan<N, M>) * (size_t)B, 256);
         L.off_flags = off;   // [fcounter, scounter, retry counter, pad][fflags][sflags][retry fflags]
         L.flags_bytes = 16 + 4 * (size_t)(2 * L.ntf + L.nts);
         off = align_up(off + L.flags_bytes, 256);
@@ -136,11 +150,15 @@ struct Impl {
     static BlockCoef<N, M>* coef(void* ws, const Layout& L) {
         return reinterpret_cast<BlockCoef<N, M>*>(static_cast<char*>(ws) + L.off_coef);
     }
+    static SteadyPlan<N, M>* plan(void* ws, const Layout& L) {
+        return reinterpret_cast<SteadyPlan<N, M>*>(static_cast<char*>(ws) + L.off_plan);
+    }
     static uint32_t* status(void* ws) { return static_cast<uint32_t*>(ws); }
 
-    static ScanState fstate(void* ws, const Layout& L) {
+    static ScanState fstate(void* ws, const Layout& L, bool gated = false) {
         char* b = static_cast<char*>(ws);
         ScanState s;
+        s.gated = gated ? 1u : 0u;
         s.counter = reinterpret_cast<uint32_t*>(b + L.off_flags);
         s.flags = reinterpret_cast<uint32_t*>(b + L.off_flags + 16);
         s.agg = reinterpret_cast<float*>(b + L.off_fagg);
@@ -150,16 +168,17 @@ struct Impl {
         return s;
     }
     // The forward scan's retry with refinement: its own counter and flags.
-    static ScanState fstate_retry(void* ws, const Layout& L) {
-        ScanState s = fstate(ws, L);
+    static ScanState fstate_retry(void* ws, const Layout& L, bool gated = false) {
+        ScanState s = fstate(ws, L, gated);
         char* b = static_cast<char*>(ws);
         s.counter = reinterpret_cast<uint32_t*>(b + L.off_flags + 8);
         s.flags = reinterpret_cast<uint32_t*>(b + L.off_flags + 16 + 4 * (size_t)(L.ntf + L.nts));
         return s;
     }
-    static ScanState sstate(void* ws, const Layout& L) {
+    static ScanState sstate(void* ws, const Layout& L, bool gated = false) {
         char* b = static_cast<char*>(ws);
         ScanState s;
+        s.gated = gated ? 1u : 0u;
         s.counter = reinterpret_cast<uint32_t*>(b + L.off_flags + 4);
         s.flags = reinterpret_cast<uint32_t*>(b + L.off_flags + 16 + 4 * (size_t)L.ntf);
         s.agg = reinterpret_cast<float*>(b + L.off_sagg);
@@ -224,12 +243,13 @@ struct Impl {
         static const bool ok = allow_smem(k, smem) && allow_smem(kr, smem);
         if (!ok) return KS_ECUDA;
         const ModelConst<N, M>* mc = mconst(ws, L);
+        // both gated: the settled path ran first (launch_steady)
         const float* none = nullptr;
         float* sb = sblk(ws, L);
-        int rc = launch_pdl(k, L.ntf, FNT, smem, st, mc, y, none, L.ld, L.T, fm, fc, fstate(ws, L), sb, segs,
+        int rc = launch_pdl(k, L.ntf, FNT, smem, st, mc, y, none, L.ld, L.T, fm, fc, fstate(ws, L, true), sb, segs,
                             TVArgs{});
         if (rc) return rc;
-        return launch_pdl(kr, L.ntf, FNT, smem, st, mc, y, none, L.ld, L.T, fm, fc, fstate_retry(ws, L), sb, segs,
+        return launch_pdl(kr, L.ntf, FNT, smem, st, mc, y, none, L.ld, L.T, fm, fc, fstate_retry(ws, L, true), sb, segs,
                           TVArgs{});
     }
 
@@ -272,7 +292,30 @@ struct Impl {
         if (!ok) return KS_ECUDA;
         const float* sb = FROM_AGG ? sblk(ws, L) : nullptr;
         return launch_pdl(k, L.nts, SNT, smem, st, (const ModelConst<N, M>*)mconst(ws, L), (const float*)fm,
-                          (const float*)fc, L.T, sm, sc, sstate(ws, L), sb, segs, tv);
+                          (const float*)fc, L.T, sm, sc, sstate(ws, L, FROM_AGG && !TV), sb, segs, tv);
+    }
+
+    // Preparation with the settled path's plan, and the settled path itself
+    // (ks_steady.cuh), which the gated general scans follow.
+    static int launch_plan(const float* F, const float* u, const float* Q, const float* H, const float* d,
+                           const float* R, const double* m0, const double* P0, const float* y, int B,
+                           const int64_t* off, void* ws, const Layout& L, bool fold, cudaStream_t st) {
+        PlanArgs<N, M> g{F, u, Q, H, d, R, m0, P0, y, mconst(ws, L), status(ws)};
+        g.zero = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + L.off_flags);
+        g.nzero = (int)(L.flags_bytes / 4);
+        g.off = off;
+        g.B = B;
+        g.T = L.T;
+        g.first_tile = status(ws) + HDR_FIRST_TILE;
+        g.coef = fold ? coef(ws, L) : nullptr;
+        g.ch = FCH;
+        g.plan = plan(ws, L);
+        return launch_plan_kernel(g, st);
+    }
+    static int launch_steady(void* ws, const Layout& L, const float* y, float* fm, float* fc, float* sm, float* sc,
+                             bool keep, const int64_t* off, cudaStream_t st) {
+        const SteadyArgs<N, M> g{plan(ws, L), off, L.B, L.T, y, fm, fc, sm, sc, keep ? 1 : 0, status(ws)};
+        return launch_steady_kernel(g, st);
     }
 
     static int build_elements(const ks_model* m, const float* y, int64_t T, void* ws, size_t ws_bytes,
@@ -383,9 +426,12 @@ struct Impl {
             return KS_EINVAL;
         }
         if ((rc = record(ev, 0, st))) return rc;
-        if ((rc = prep(m, y, ws, L, st, fold))) return rc;
+        if ((rc = launch_plan(m->F, m->u, m->Q, m->H, m->d, m->R, m->m0, m->P0, y, 1, nullptr, ws, L, fold, st)))
+            return rc;
         if ((rc = record(ev, 1, st))) return rc;
-        const Segs<N, M> segs{nullptr, nullptr, 1, fold ? coef(ws, L) : nullptr};
+        if ((rc = launch_steady(ws, L, y, fm, fc, sm, sc, !own, nullptr, st))) return rc;
+        const Segs<N, M> segs{nullptr, nullptr, 1, fold ? coef(ws, L) : nullptr,
+                               &plan(ws, L)->ok};
         if ((rc = launch_filter_fused<false>(ws, L, y, fm, fc, segs, st))) return rc;
         if ((rc = record(ev, 2, st))) return rc;
         if (!filter_only && (rc = launch_smoother<true, false>(ws, L, fm, fc, sm, sc, no_segs(), st))) return rc;
@@ -407,14 +453,10 @@ struct Impl {
         if (!y || !fm || !fc || !sm || !sc) return KS_EINVAL;
         if (!aligned16(y) || !aligned16(fm) || !aligned16(fc) || !aligned16(sm) || !aligned16(sc))
             return KS_EINVAL;
-        uint32_t* z = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + L.off_flags);
-        auto k = fold ? prep_kernel<N, M, true> : prep_kernel<N, M, false>;
-        k<<<mb->B, kPrepThreads, prep_smem(), st>>>(mb->F, mb->u, mb->Q, mb->H, mb->d, mb->R, mb->m0, mb->P0, y,
-                                                    mconst(ws, L), status(ws), z, (int)(L.flags_bytes / 4),
-                                                    mb->offsets, T, status(ws) + HDR_FIRST_TILE,
-                                                    fold ? coef(ws, L) : nullptr, FCH);
-        int rc = launch_status();
+        int rc = launch_plan(mb->F, mb->u, mb->Q, mb->H, mb->d, mb->R, mb->m0, mb->P0, y, mb->B, mb->offsets, ws, L,
+                             fold, st);
         if (rc) return rc;
+        if ((rc = launch_steady(ws, L, y, fm, fc, sm, sc, true, mb->offsets, st))) return rc;
         const Segs<N, M> segs{mconst(ws, L), mb->offsets, mb->B, fold ? coef(ws, L) : nullptr};
         if ((rc = launch_filter_fused<true>(ws, L, y, fm, fc, segs, st))) return rc;
         return launch_smoother<true, true>(ws, L, fm, fc, sm, sc, segs, st);

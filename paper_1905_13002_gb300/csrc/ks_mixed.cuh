@@ -1,4 +1,5 @@
-// ks_mixed.cuh -- one preparation, one forward and one reverse launch over a
+// ks_mixed.cuh -- one preparation, one settled-path launch (ks_steady.cuh) and,
+// when a sequence needs them, one forward and one reverse scan launch over a
 // batch whose sequences have different state sizes (nx in {2, 4, 6}).
 //
 // The sequences come in up to three groups, one per state size, each laid
@@ -39,6 +40,7 @@ struct MixedGroup {
     uint32_t* zero = nullptr;   // the group's flags region
     int nzero = 0;
     int ch = 0;                 // steps per thread of the launch (block-fold coefficients)
+    SteadyPlan<N, M>* plan = nullptr;   // settled path: one plan per sequence
 };
 
 using MG6 = MixedGroup<6, 3>;
@@ -55,37 +57,11 @@ struct MixedQueue {
 
 constexpr int kMixedThreads = 128;
 
-template <int N, int M, bool FOLD>
-KS_DEV void mixed_prep_one(char* dsm, int sg, const MixedGroup<N, M>& g) {
-    prep_body<N, M, FOLD>(dsm, sg, g.B, g.F, g.u, g.Q, g.H, g.d, g.R, g.m0, g.P0, g.y,
-                    const_cast<ModelConst<N, M>*>(g.segs.mcg), g.fs.status, g.zero, g.nzero, g.segs.off, g.T,
-                    nullptr, const_cast<BlockCoef<N, M>*>(g.segs.coef), g.ch);
-}
-
-// One block per sequence of all groups (nx = 6 sequences first); block 0 also
-// zeroes the two work-queue counters.  (CH only makes one copy per
-// instantiation unit; FOLD: build the block-fold coefficients.)
-template <int CH, bool FOLD>
-__global__ void __launch_bounds__(kPrepThreads) mixed_prep_kernel(MG6 g6, MG4 g4, MG2 g2, MixedQueue q) {
-    extern __shared__ __align__(16) char prep_dsm[];
-    int b = (int)blockIdx.x;
-    if (b == 0 && threadIdx.x == 0) {
-        *q.fcounter = 0u;
-        *q.scounter = 0u;
-        *q.fcounter2 = 0u;
-    }
-    if (b < g6.B) { mixed_prep_one<6, 3, FOLD>(prep_dsm, b, g6); return; }
-    b -= g6.B;
-    if (b < g4.B) { mixed_prep_one<4, 2, FOLD>(prep_dsm, b, g4); return; }
-    b -= g4.B;
-    if (b < g2.B) mixed_prep_one<2, 1, FOLD>(prep_dsm, b, g2);
-}
-
-template <int N, int M>
-constexpr size_t mixed_prep_smem_of() { return prep_dyn_smem<N, M>(); }
-constexpr size_t mixed_prep_smem() {
-    return cmax(cmax(mixed_prep_smem_of<6, 3>(), mixed_prep_smem_of<4, 2>()), mixed_prep_smem_of<2, 1>());
-}
+// The preparation with the settled path's plans, one block per sequence of all
+// groups (nx = 6 sequences first; it also zeroes the queue counters), and the
+// settled path, one launch over the windows of all groups (ks_steady_mixed.cu).
+int launch_mixed_plan(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, bool fold, cudaStream_t st);
+int launch_mixed_steady(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, cudaStream_t st);
 
 template <int CH, int REF, bool RETRY>
 KS_DEV void mixed_filter_tile(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q);
@@ -95,15 +71,13 @@ KS_DEV void mixed_filter_tile(const MG6& g6, const MG4& g4, const MG2& g2, const
 // when the first met one.
 template <int CH, int REF, bool RETRY>
 __global__ void __launch_bounds__(kMixedThreads) mixed_filter_kernel(MG6 g6, MG4 g4, MG2 g2, MixedQueue q) {
+    pdl_trigger();
     pdl_wait();
+    if (!general_wanted(q.status)) return;   // the settled path took every sequence
     if constexpr (RETRY) {
-        if (*(volatile uint32_t*)(q.status + HDR_NEED) == 0u) {
-            pdl_trigger();
-            return;
-        }
+        if (*(volatile uint32_t*)(q.status + HDR_NEED) == 0u) return;
     }
     mixed_filter_tile<CH, REF, RETRY>(g6, g4, g2, q);
-    pdl_trigger();
 }
 
 // Dynamic shared memory of one size's body: its block-scan state first, its
@@ -171,6 +145,7 @@ __global__ void __launch_bounds__(kMixedThreads, kRevMinBlocks<4>) mixed_smoothe
     __shared__ int s_tile;
     extern __shared__ __align__(16) char dsm[];
     pdl_wait();
+    if (!general_wanted(q.status)) return;
     if (threadIdx.x == 0) s_tile = (int)atomicAdd(q.scounter, 1u);
     __syncthreads();
     int t = s_tile;
@@ -248,6 +223,7 @@ struct Mixed {
         o.sagg = reinterpret_cast<float*>(b + L.off_sblk);
         o.zero = reinterpret_cast<uint32_t*>(b + L.off_flags);
         o.nzero = (int)(L.flags_bytes / 4);
+        o.plan = reinterpret_cast<SteadyPlan<N, M>*>(b + L.off_plan);
         return o;
     }
 
@@ -267,20 +243,14 @@ struct Mixed {
         const MixedQueue q{reinterpret_cast<uint32_t*>(w + kMixedQueueOff),
                            reinterpret_cast<uint32_t*>(w + kMixedQueueOff + 4),
                            reinterpret_cast<uint32_t*>(w + kMixedQueueOff + 8), reinterpret_cast<uint32_t*>(w)};
-        const int nseq = g6.B + g4.B + g2.B;
         const int ntiles = g6.ntiles + g4.ntiles + g2.ntiles;
-        static const bool ok = allow_smem(mixed_prep_kernel<CH, true>, (int)mixed_prep_smem()) &&
-                               allow_smem(mixed_prep_kernel<CH, false>, (int)mixed_prep_smem()) &&
-                               allow_smem(mixed_filter_kernel<CH, REF_DETECT, false>, mixed_filter_smem()) &&
+        static const bool ok = allow_smem(mixed_filter_kernel<CH, REF_DETECT, false>, mixed_filter_smem()) &&
                                allow_smem(mixed_filter_kernel<CH, REF_FP64, true>, mixed_filter_smem()) &&
                                allow_smem(mixed_smoother_kernel<CH>, mixed_smoother_smem());
         if (!ok) return KS_ECUDA;
-        if (fold)
-            mixed_prep_kernel<CH, true><<<nseq, kPrepThreads, mixed_prep_smem(), st>>>(g6, g4, g2, q);
-        else
-            mixed_prep_kernel<CH, false><<<nseq, kPrepThreads, mixed_prep_smem(), st>>>(g6, g4, g2, q);
-        int rc = launch_status();
+        int rc = launch_mixed_plan(g6, g4, g2, q, fold, st);
         if (rc) return rc;
+        if ((rc = launch_mixed_steady(g6, g4, g2, q, st))) return rc;
         if ((rc = launch_pdl(mixed_filter_kernel<CH, REF_DETECT, false>, ntiles, kMixedThreads, mixed_filter_smem(),
                              st, g6, g4, g2, q)))
             return rc;

@@ -46,8 +46,18 @@ constexpr float kRefineCond = 1.0e3f;
 // wait limit in polls (0: the scan's default), [3] the forward scans' first
 // tile number (0; 1 only when a test leaves tile 0 unclaimed to make the
 // look-back waits run out), [4] set when a scan without refinement met an
-// ill-conditioned inverse (cleared by the preparation kernel).
-enum : int { HDR_STATUS = 0, HDR_REFINED = 1, HDR_WAIT = 2, HDR_FIRST_TILE = 3, HDR_NEED = 4 };
+// ill-conditioned inverse (cleared by the preparation kernel), [5] set when a
+// sequence of a fused call does not take the settled path (ks_steady.cuh) and
+// the call's general scans must run (cleared by the preparation kernel).
+enum : int { HDR_STATUS = 0, HDR_REFINED = 1, HDR_WAIT = 2, HDR_FIRST_TILE = 3, HDR_NEED = 4, HDR_GENERAL = 5 };
+
+// Whether the general scans of a fused call have work: some sequence asked
+// for them, or the offsets table is inconsistent (the scans define what such
+// a call writes).
+KS_DEV bool general_wanted(const uint32_t* status) {
+    const volatile uint32_t* w = status;
+    return w[HDR_GENERAL] != 0u || (w[HDR_STATUS] & ST_BADARG) != 0u;
+}
 
 // End-of-kernel report of one warp or lane group (`mask`), by its `leader`
 // lane: a numeric failure sets ST_NUMERIC in the status word, a group in

@@ -45,7 +45,18 @@ struct ScanState {
     float* pre;          // per-tile inclusive prefixes
     uint32_t* status;    // device status word (workspace header, see below)
     uint32_t spin_limit; // look-back polls before giving up (~1 s)
+    uint32_t gated = 0;  // run only when general_wanted(status) (behind the settled path of a fused call)
 };
+
+// Start of a kernel that may stand behind the settled path of a fused call
+// (gate: the workspace header, null when it does not): whether it has nothing
+// to do.
+KS_DEV bool gate_closed(const uint32_t* gate) {
+    if (gate == nullptr) return false;
+    pdl_trigger();   // what follows waits too
+    pdl_wait();
+    return !general_wanted(gate);
+}
 
 KS_DEV uint32_t wait_limit(const ScanState& ss) {
     const uint32_t o = ss.status[HDR_WAIT];
@@ -253,6 +264,7 @@ struct Segs {
     const int64_t* off;            // [B+1] (batched), else nullptr
     int B;
     const BlockCoef<N, M>* coef = nullptr;   // block-fold coefficients per segment (null: none)
+    const int* settled = nullptr;   // single sequence: non-zero when its plan passed, so that coef was not built
 };
 
 // With TV the constants are per step (g.mcg[k] for step k of one sequence of
@@ -623,27 +635,18 @@ KS_DEV void first_element_fp64(PS& p, MC& mc, int i) {
     }
 }
 
-// One block per model (segment).  After one round of loads, warp 0 builds the
-// FP32 constants of Lemma 3 for k > 1 (and the block-fold coefficients), and
-// warps 1-3, at the same time, the k = 1 element (prediction of N(m0, P0) and
-// update with y_1) in FP64; the two chains only meet for the final store.
-// Body of the preparation of segment sg of nseg (one thread block); dyn:
-// its dynamic shared memory (PrepSmem and a ModelConst).
-// FOLD = false leaves the block-fold coefficient code out (fewer registers
-// for launches that never fold).
-template <int N, int M, bool FOLD = true>
-KS_DEV void prep_body(char* prep_dsm, int sg, int nseg, const float* __restrict__ F, const float* __restrict__ u,
-                      const float* __restrict__ Q, const float* __restrict__ H, const float* __restrict__ d,
-                      const float* __restrict__ R, const double* __restrict__ m0, const double* __restrict__ P0,
-                      const float* __restrict__ y, ModelConst<N, M>* __restrict__ out, uint32_t* __restrict__ status,
-                      uint32_t* __restrict__ zero, int nzero, const int64_t* __restrict__ off, int64_t T,
-                      const uint32_t* __restrict__ first_tile, BlockCoef<N, M>* __restrict__ coef = nullptr,
-                      int ch = 0) {
-    PrepSmem<N, M>& p = *reinterpret_cast<PrepSmem<N, M>*>(prep_dsm);
-    ModelConst<N, M>& mc =
-        *reinterpret_cast<ModelConst<N, M>*>(prep_dsm + ((sizeof(PrepSmem<N, M>) + 15) / 16) * 16);
+// Inputs of segment sg of nseg into shared memory (one round of independent
+// loads), the scans' words zeroed and the segment table checked by the way.
+// Returns the segment's first measurement, null when it has none.
+template <int N, int M>
+KS_DEV const float* prep_inputs(PrepSmem<N, M>& p, int sg, int nseg, const float* __restrict__ F,
+                                const float* __restrict__ u, const float* __restrict__ Q,
+                                const float* __restrict__ H, const float* __restrict__ d,
+                                const float* __restrict__ R, const double* __restrict__ m0,
+                                const double* __restrict__ P0, const float* __restrict__ y,
+                                uint32_t* __restrict__ status, uint32_t* __restrict__ zero, int nzero,
+                                const int64_t* __restrict__ off, int64_t T, const uint32_t* __restrict__ first_tile) {
     const int t = threadIdx.x, nt = blockDim.x;
-    const int warp = t >> 5, l = t & 31;
     if (sg == 0) {   // zero[0] is the forward tile counter of the nx <= 6 scans (first_tile: its start)
         for (int i = t; i < nzero; i += nt) zero[i] = (i == 0 && first_tile != nullptr) ? *first_tile : 0u;
         if (t == 0) status[HDR_NEED] = 0u;
@@ -665,7 +668,6 @@ KS_DEV void prep_body(char* prep_dsm, int sg, int nseg, const float* __restrict_
         const int64_t a = off[sg], b = off[sg + 1];
         y = (a >= 0 && a < b && a < T) ? y + a * M : nullptr;
     }
-    out += sg;
     // ---- every input in one round of independent loads
     constexpr int nF = N * N, nQ = N * N, nP = N * N, nH = M * N, nR = M * M;
     constexpr int nAll = nF + nQ + nP + nH + nR + N + N + M + M;
@@ -691,90 +693,134 @@ KS_DEV void prep_body(char* prep_dsm, int sg, int nseg, const float* __restrict_
     }
     if (t == 0) { p.ok0 = 1; p.ok1 = 1; }
     __syncthreads();
+    return y;
+}
 
+// FP32 constants of Lemma 3 for k > 1, by one warp (lane l).
+template <int N, int M>
+KS_DEV void prep_consts(PrepSmem<N, M>& p, ModelConst<N, M>& mc, int l) {
+    // ---- FP32 constants for k > 1: S = H Q H^T + R = L_S L_S^T, U = L_S^{-1} H F,
+    // K = Q H^T S^{-1}, A = F - K H F, C = Q - K S K^T (Q, R symmetrised)
+    for (int e = l; e < M * N; e += 32) {
+        const int q = e / N, a = e % N;
+        float s = 0.f, h = 0.f;
+        for (int c = 0; c < N; ++c) {
+            s = fmaf(p.H[q][c], 0.5f * (p.Q[c][a] + p.Q[a][c]), s);
+            h = fmaf(p.H[q][c], p.F[c][a], h);
+        }
+        p.HQ[q][a] = s;
+        p.HF[q][a] = h;
+    }
+    __syncwarp();
+    for (int e = l; e < M * M; e += 32) {
+        const int q = e / M, r = e % M;
+        float s = 0.5f * (p.R[q][r] + p.R[r][q]);
+        for (int c = 0; c < N; ++c) s = fmaf(p.HQ[q][c], p.H[r][c], s);
+        p.S[q][r] = s;
+    }
+    __syncwarp();
+    if (l == 0) {                              // Cholesky of S, L_S^{-1}
+        float Ls[M][M];
+        bool ok = true;
+        for (int j = 0; j < M; ++j) {
+            float s = p.S[j][j];
+            for (int k = 0; k < j; ++k) s -= Ls[j][k] * Ls[j][k];
+            ok = ok && (s > 0.f);
+            Ls[j][j] = sqrtf(fmaxf(s, 1e-37f));
+            for (int i = j + 1; i < M; ++i) {
+                float q = p.S[i][j];
+                for (int k = 0; k < j; ++k) q -= Ls[i][k] * Ls[j][k];
+                Ls[i][j] = q / Ls[j][j];
+            }
+        }
+        for (int c = 0; c < M; ++c)
+            for (int i = 0; i < M; ++i) {
+                if (i < c) { p.Lsi[i][c] = 0.f; continue; }
+                float q = (i == c) ? 1.f : 0.f;
+                for (int k = c; k < i; ++k) q -= Ls[i][k] * p.Lsi[k][c];
+                p.Lsi[i][c] = q / Ls[i][i];
+            }
+        if (!ok) p.ok0 = 0;
+    }
+    __syncwarp();
+    for (int e = l; e < M * N; e += 32) {      // tmp = L_S^{-1} H Q, U = L_S^{-1} H F
+        const int q = e / N, a = e % N;
+        float s = 0.f, v = 0.f;
+        for (int r = 0; r <= q; ++r) { s = fmaf(p.Lsi[q][r], p.HQ[r][a], s); v = fmaf(p.Lsi[q][r], p.HF[r][a], v); }
+        p.tmp[q][a] = s;
+        mc.U[q * N + a] = v;
+    }
+    for (int e = l; e < M; e += 32) {
+        float s = p.d[e];
+        for (int c = 0; c < N; ++c) s = fmaf(p.H[e][c], p.u[c], s);
+        mc.hud[e] = s;
+        for (int r = 0; r < M; ++r) mc.Lsi[e * M + r] = p.Lsi[e][r];
+    }
+    __syncwarp();
+    for (int e = l; e < N * M; e += 32) {      // K = tmp^T L_S^{-1}
+        const int a = e / M, q = e % M;
+        float s = 0.f;
+        for (int r = q; r < M; ++r) s = fmaf(p.tmp[r][a], p.Lsi[r][q], s);
+        p.K[a][q] = s;
+        mc.K[a * M + q] = s;
+    }
+    __syncwarp();
+    for (int e = l; e < N * N; e += 32) {      // A = F - K H F ; C = Q - tmp^T tmp ; copies
+        const int a = e / N, b = e % N;
+        float s = p.F[a][b];
+        for (int q = 0; q < M; ++q) s = fmaf(-p.K[a][q], p.HF[q][b], s);
+        mc.A[a * N + b] = s;
+        mc.F[a * N + b] = p.F[a][b];
+        if (b <= a) {
+            const float qs = 0.5f * (p.Q[a][b] + p.Q[b][a]);
+            float c = qs;
+            for (int q = 0; q < M; ++q) c = fmaf(-p.tmp[q][a], p.tmp[q][b], c);
+            mc.C[sidx(a, b)] = c;
+            mc.Q[sidx(a, b)] = qs;
+        }
+    }
+    for (int e = l; e < N; e += 32) mc.u[e] = p.u[e];
+    if (l < 4) mc.pad[l] = 0.f;
+}
+
+// The constants to global memory (all threads), a failed factorisation to the
+// status word.
+template <int N, int M>
+KS_DEV void prep_store(const PrepSmem<N, M>& p, const ModelConst<N, M>& mc, ModelConst<N, M>* __restrict__ out,
+                       uint32_t* __restrict__ status) {
+    const int t = threadIdx.x, nt = blockDim.x;
+    {
+        const float* src = reinterpret_cast<const float*>(&mc);
+        float* dst = reinterpret_cast<float*>(out);
+        for (int i = t; i < (int)(sizeof(ModelConst<N, M>) / 4); i += nt) dst[i] = src[i];
+    }
+    if (t == 0 && !(p.ok0 && p.ok1)) atomicOr(status, ST_NUMERIC);
+}
+
+// One block per model (segment).  After one round of loads, warp 0 builds the
+// FP32 constants of Lemma 3 for k > 1 (and the block-fold coefficients), and
+// warps 1-3, at the same time, the k = 1 element (prediction of N(m0, P0) and
+// update with y_1) in FP64; the two chains only meet for the final store.
+// Body of the preparation of segment sg of nseg (one thread block); dyn:
+// its dynamic shared memory (PrepSmem and a ModelConst).
+// FOLD = false leaves the block-fold coefficient code out (fewer registers
+// for launches that never fold).
+template <int N, int M, bool FOLD = true>
+KS_DEV void prep_body(char* prep_dsm, int sg, int nseg, const float* __restrict__ F, const float* __restrict__ u,
+                      const float* __restrict__ Q, const float* __restrict__ H, const float* __restrict__ d,
+                      const float* __restrict__ R, const double* __restrict__ m0, const double* __restrict__ P0,
+                      const float* __restrict__ y, ModelConst<N, M>* __restrict__ out, uint32_t* __restrict__ status,
+                      uint32_t* __restrict__ zero, int nzero, const int64_t* __restrict__ off, int64_t T,
+                      const uint32_t* __restrict__ first_tile, BlockCoef<N, M>* __restrict__ coef = nullptr,
+                      int ch = 0) {
+    PrepSmem<N, M>& p = *reinterpret_cast<PrepSmem<N, M>*>(prep_dsm);
+    ModelConst<N, M>& mc =
+        *reinterpret_cast<ModelConst<N, M>*>(prep_dsm + ((sizeof(PrepSmem<N, M>) + 15) / 16) * 16);
+    const int t = threadIdx.x, warp = t >> 5, l = t & 31;
+    const float* y1 =
+        prep_inputs<N, M>(p, sg, nseg, F, u, Q, H, d, R, m0, P0, y, status, zero, nzero, off, T, first_tile);
     if (warp == 0) {
-        // ---- FP32 constants for k > 1: S = H Q H^T + R = L_S L_S^T, U = L_S^{-1} H F,
-        // K = Q H^T S^{-1}, A = F - K H F, C = Q - K S K^T (Q, R symmetrised)
-        for (int e = l; e < M * N; e += 32) {
-            const int q = e / N, a = e % N;
-            float s = 0.f, h = 0.f;
-            for (int c = 0; c < N; ++c) {
-                s = fmaf(p.H[q][c], 0.5f * (p.Q[c][a] + p.Q[a][c]), s);
-                h = fmaf(p.H[q][c], p.F[c][a], h);
-            }
-            p.HQ[q][a] = s;
-            p.HF[q][a] = h;
-        }
-        __syncwarp();
-        for (int e = l; e < M * M; e += 32) {
-            const int q = e / M, r = e % M;
-            float s = 0.5f * (p.R[q][r] + p.R[r][q]);
-            for (int c = 0; c < N; ++c) s = fmaf(p.HQ[q][c], p.H[r][c], s);
-            p.S[q][r] = s;
-        }
-        __syncwarp();
-        if (l == 0) {                              // Cholesky of S, L_S^{-1}
-            float Ls[M][M];
-            bool ok = true;
-            for (int j = 0; j < M; ++j) {
-                float s = p.S[j][j];
-                for (int k = 0; k < j; ++k) s -= Ls[j][k] * Ls[j][k];
-                ok = ok && (s > 0.f);
-                Ls[j][j] = sqrtf(fmaxf(s, 1e-37f));
-                for (int i = j + 1; i < M; ++i) {
-                    float q = p.S[i][j];
-                    for (int k = 0; k < j; ++k) q -= Ls[i][k] * Ls[j][k];
-                    Ls[i][j] = q / Ls[j][j];
-                }
-            }
-            for (int c = 0; c < M; ++c)
-                for (int i = 0; i < M; ++i) {
-                    if (i < c) { p.Lsi[i][c] = 0.f; continue; }
-                    float q = (i == c) ? 1.f : 0.f;
-                    for (int k = c; k < i; ++k) q -= Ls[i][k] * p.Lsi[k][c];
-                    p.Lsi[i][c] = q / Ls[i][i];
-                }
-            if (!ok) p.ok0 = 0;
-        }
-        __syncwarp();
-        for (int e = l; e < M * N; e += 32) {      // tmp = L_S^{-1} H Q, U = L_S^{-1} H F
-            const int q = e / N, a = e % N;
-            float s = 0.f, v = 0.f;
-            for (int r = 0; r <= q; ++r) { s = fmaf(p.Lsi[q][r], p.HQ[r][a], s); v = fmaf(p.Lsi[q][r], p.HF[r][a], v); }
-            p.tmp[q][a] = s;
-            mc.U[q * N + a] = v;
-        }
-        for (int e = l; e < M; e += 32) {
-            float s = p.d[e];
-            for (int c = 0; c < N; ++c) s = fmaf(p.H[e][c], p.u[c], s);
-            mc.hud[e] = s;
-            for (int r = 0; r < M; ++r) mc.Lsi[e * M + r] = p.Lsi[e][r];
-        }
-        __syncwarp();
-        for (int e = l; e < N * M; e += 32) {      // K = tmp^T L_S^{-1}
-            const int a = e / M, q = e % M;
-            float s = 0.f;
-            for (int r = q; r < M; ++r) s = fmaf(p.tmp[r][a], p.Lsi[r][q], s);
-            p.K[a][q] = s;
-            mc.K[a * M + q] = s;
-        }
-        __syncwarp();
-        for (int e = l; e < N * N; e += 32) {      // A = F - K H F ; C = Q - tmp^T tmp ; copies
-            const int a = e / N, b = e % N;
-            float s = p.F[a][b];
-            for (int q = 0; q < M; ++q) s = fmaf(-p.K[a][q], p.HF[q][b], s);
-            mc.A[a * N + b] = s;
-            mc.F[a * N + b] = p.F[a][b];
-            if (b <= a) {
-                const float qs = 0.5f * (p.Q[a][b] + p.Q[b][a]);
-                float c = qs;
-                for (int q = 0; q < M; ++q) c = fmaf(-p.tmp[q][a], p.tmp[q][b], c);
-                mc.C[sidx(a, b)] = c;
-                mc.Q[sidx(a, b)] = qs;
-            }
-        }
-        for (int e = l; e < N; e += 32) mc.u[e] = p.u[e];
-        if (l < 4) mc.pad[l] = 0.f;
+        prep_consts<N, M>(p, mc, l);
         if constexpr (N <= 6 && FOLD) {   // register-path sizes only
             if (coef != nullptr) {   // the block-fold coefficients, while warps 1-3 build the k = 1 element
                 __syncwarp();
@@ -782,7 +828,7 @@ KS_DEV void prep_body(char* prep_dsm, int sg, int nseg, const float* __restrict_
             }
         }
     } else {   // warps 1-3
-        if (y != nullptr) {
+        if (y1 != nullptr) {
             first_element_fp64<N, M>(p, mc, t - 32);
         } else {
             for (int e = t - 32; e < N; e += kFirstThreads) mc.b1[e] = 0.f;
@@ -790,12 +836,7 @@ KS_DEV void prep_body(char* prep_dsm, int sg, int nseg, const float* __restrict_
         }
     }
     __syncthreads();
-    {
-        const float* src = reinterpret_cast<const float*>(&mc);
-        float* dst = reinterpret_cast<float*>(out);
-        for (int i = t; i < (int)(sizeof(ModelConst<N, M>) / 4); i += nt) dst[i] = src[i];
-    }
-    if (t == 0 && !(p.ok0 && p.ok1)) atomicOr(status, ST_NUMERIC);
+    prep_store<N, M>(p, mc, out + sg, status);
 }
 
 // Dynamic shared memory of prep_body.
@@ -1753,7 +1794,9 @@ __global__ void __launch_bounds__(NT) filter_scan_kernel(const ModelConst<N, M>*
                                                          float* __restrict__ fcov, ScanState ss,
                                                          float* __restrict__ sagg, Segs<N, M> segs,
                                                          TVArgs tv) {
+    if (ss.gated) pdl_trigger();   // what follows waits too, and mostly has nothing to do
     pdl_wait();   // the preparation (or the first run) has completed
+    if (ss.gated && !general_wanted(ss.status)) return;
     if constexpr (RETRY) {
         if (*(volatile uint32_t*)(ss.status + HDR_NEED) == 0u) {   // the first run needed no refinement
             pdl_trigger();
@@ -1765,6 +1808,7 @@ __global__ void __launch_bounds__(NT) filter_scan_kernel(const ModelConst<N, M>*
     extern __shared__ __align__(16) char dsm[];
     const int tid = threadIdx.x;
     load_const<N, M>(mcg, sm.mc, tid, NT);
+    if (!SEG && segs.settled != nullptr && *segs.settled != 0) segs.coef = nullptr;
     if (!SEG && segs.coef != nullptr) load_coef<N, M>(segs.coef, sm.bc, tid, NT);
     if (tid == 0) s_tile = (int)atomicAdd(ss.counter, 1u);
     __syncthreads();
@@ -2023,7 +2067,9 @@ __global__ void __launch_bounds__(NT, kRevMinBlocks<N>) smoother_scan_kernel(con
     __shared__ int s_tile;
     extern __shared__ __align__(16) char dsm[];
     const int tid = threadIdx.x;
+    if (ss.gated) pdl_trigger();
     pdl_wait();   // the forward scan has completed
+    if (ss.gated && !general_wanted(ss.status)) return;
     load_const<N, M>(mcg, sm.mc, tid, NT);
     if (tid == 0) s_tile = (int)atomicAdd(ss.counter, 1u);
     if constexpr (Stage<N>::kOn) {

@@ -69,7 +69,8 @@ struct TImpl {
     }
 
     static int scans(void* ws, const Layout& L, const float* y, float* fm, float* fc, float* sm, float* sc,
-                     cudaStream_t st, void* const* ev, bool filter, bool smoother) {
+                     cudaStream_t st, void* const* ev, bool filter, bool smoother,
+                     const uint32_t* gate = nullptr) {
         using FSP = tc::SpineSmem<N, tc::kSpineWarps, tc::kSpineBufF>;
         using SSP = tc::SpineSmem<N, tc::kSpineWarps, tc::kSpineBufS>;
         constexpr int SW = tc::kSpineWarps;
@@ -86,19 +87,20 @@ struct TImpl {
             static const bool ok = allow_smem(kr, (int)sizeof(FSM)) && allow_smem(ks, (int)sizeof(FSP)) &&
                                    allow_smem(ka, (int)sizeof(FSM));
             if (!ok) return KS_ECUDA;
-            kr<<<L.ntf, NW * 32, sizeof(FSM), st>>>(mc, y, L.T, fb, status);
-            if ((rc = launch_status())) return rc;
+            if ((rc = launch_gated(kr, L.ntf, NW * 32, sizeof(FSM), st, gate, mc, y, L.T, fb, status))) return rc;
             const float* src = fb.spine0;
             float* dst = fb.spine1;
             for (int s = 1; s < L.ntf; s <<= 1) {
-                ks<<<(L.ntf + SW - 1) / SW, SW * 32, sizeof(FSP), st>>>(src, dst, L.ntf, s, status);
-                if ((rc = launch_status())) return rc;
+                rc = launch_gated(ks, (L.ntf + SW - 1) / SW, SW * 32, sizeof(FSP), st, gate,
+                                  src, dst, L.ntf, s, status);
+                if (rc) return rc;
                 float* t = const_cast<float*>(src);
                 src = dst;
                 dst = t;
             }
-            ka<<<L.ntf, NW * 32, sizeof(FSM), st>>>(mc, y, L.T, fm, fc, fb, src, status);
-            if ((rc = launch_status())) return rc;
+            rc = launch_gated(ka, L.ntf, NW * 32, sizeof(FSM), st, gate,
+                              mc, y, L.T, fm, fc, fb, src, status);
+            if (rc) return rc;
         }
         if (ev && ev[2] && record_event(ev[2], st) != cudaSuccess) return KS_ECUDA;
         if (smoother) {
@@ -108,19 +110,22 @@ struct TImpl {
             static const bool ok = allow_smem(kr, (int)sizeof(SSM)) && allow_smem(ks, (int)sizeof(SSP)) &&
                                    allow_smem(ka, (int)sizeof(SSM));
             if (!ok) return KS_ECUDA;
-            kr<<<L.nts, NW * 32, sizeof(SSM), st>>>(mc, fm, fc, L.T, sb, status);
-            if ((rc = launch_status())) return rc;
+            rc = launch_gated(kr, L.nts, NW * 32, sizeof(SSM), st, gate,
+                              mc, fm, fc, L.T, sb, status);
+            if (rc) return rc;
             const float* src = sb.spine0;
             float* dst = sb.spine1;
             for (int s = 1; s < L.nts; s <<= 1) {
-                ks<<<(L.nts + SW - 1) / SW, SW * 32, sizeof(SSP), st>>>(src, dst, L.nts, s, status);
-                if ((rc = launch_status())) return rc;
+                rc = launch_gated(ks, (L.nts + SW - 1) / SW, SW * 32, sizeof(SSP), st, gate,
+                                  src, dst, L.nts, s, status);
+                if (rc) return rc;
                 float* t = const_cast<float*>(src);
                 src = dst;
                 dst = t;
             }
-            ka<<<L.nts, NW * 32, sizeof(SSM), st>>>(L.T, sm, sc, sb, src, status);
-            if ((rc = launch_status())) return rc;
+            rc = launch_gated(ka, L.nts, NW * 32, sizeof(SSM), st, gate,
+                              L.T, sm, sc, sb, src, status);
+            if (rc) return rc;
         }
         return KS_OK;
     }

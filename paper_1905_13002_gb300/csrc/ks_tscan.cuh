@@ -73,7 +73,8 @@ KS_DEV void copy_record(float* dst, const float* src, int n) {
 template <int N, int M, int NW, int CH>
 __global__ void __launch_bounds__(NW * 32) tfilter_reduce_kernel(const ModelConst<N, M>* __restrict__ mcg,
                                                                  const float* __restrict__ y, int64_t T, TBuf tb,
-                                                                 uint32_t* status) {
+                                                                 uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = TSmem<N, M, NW, FConst<N, M>>;
     constexpr int MAT = TD<N>::MAT, KW = SM::KW, FR = Rec<N>::F;
     extern __shared__ __align__(16) char tsm[];
@@ -140,7 +141,8 @@ __global__ void __launch_bounds__(NW * 32) tfilter_reduce_kernel(const ModelCons
 // result is one too (only b and C are formed and stored).
 template <int N, int NWS>
 __global__ void __launch_bounds__(NWS * 32) tspine_filter_kernel(const float* __restrict__ src, float* __restrict__ dst,
-                                                                 int ntiles, int s, uint32_t* status) {
+                                                                 int ntiles, int s, uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = SpineSmem<N, NWS, kSpineBufF>;
     constexpr int FR = Rec<N>::F;
     extern __shared__ __align__(16) char tsm[];
@@ -179,7 +181,8 @@ __global__ void __launch_bounds__(NW * 32) tfilter_apply_kernel(const ModelConst
                                                                 const float* __restrict__ y, int64_t T,
                                                                 float* __restrict__ fmean, float* __restrict__ fcov,
                                                                 TBuf tb, const float* __restrict__ pre,
-                                                                uint32_t* status) {
+                                                                uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = TSmem<N, M, NW, FConst<N, M>>;
     constexpr int MAT = TD<N>::MAT, KW = SM::KW, FR = Rec<N>::F;
     extern __shared__ __align__(16) char tsm[];
@@ -237,7 +240,8 @@ template <int N, int M, int NW, int CH>
 __global__ void __launch_bounds__(NW * 32) tsmoother_reduce_kernel(const ModelConst<N, M>* __restrict__ mcg,
                                                                    const float* __restrict__ fmean,
                                                                    const float* __restrict__ fcov, int64_t T, TBuf tb,
-                                                                   uint32_t* status) {
+                                                                   uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = TSmem<N, M, NW, SConst<N, M>>;
     constexpr int MAT = TD<N>::MAT, KW = SM::KW, SR = Rec<N>::S;
     extern __shared__ __align__(16) char tsm[];
@@ -308,7 +312,8 @@ __global__ void __launch_bounds__(NW * 32) tsmoother_reduce_kernel(const ModelCo
 // u - s < s: then it is a suffix state (E = 0) and so is the result.
 template <int N, int NWS>
 __global__ void __launch_bounds__(NWS * 32) tspine_smoother_kernel(const float* __restrict__ src, float* __restrict__ dst,
-                                                                   int ntiles, int s, uint32_t* status) {
+                                                                   int ntiles, int s, uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = SpineSmem<N, NWS, kSpineBufS>;
     constexpr int SR = Rec<N>::S;
     extern __shared__ __align__(16) char tsm[];
@@ -342,7 +347,8 @@ __global__ void __launch_bounds__(NWS * 32) tspine_smoother_kernel(const float* 
 template <int N, int M, int NW, int CH>
 __global__ void __launch_bounds__(NW * 32) tsmoother_apply_kernel(int64_t T, float* __restrict__ smean,
                                                                   float* __restrict__ scov, TBuf tb,
-                                                                  const float* __restrict__ pre, uint32_t* status) {
+                                                                  const float* __restrict__ pre, uint32_t* status, const uint32_t* gate) {
+    if (gate_closed(gate)) return;
     using SM = TSmem<N, M, NW, SConst<N, M>>;
     constexpr int MAT = TD<N>::MAT, KW = SM::KW, SR = Rec<N>::S;
     extern __shared__ __align__(16) char tsm[];
