@@ -58,6 +58,10 @@ struct ChunkVariant {
                   cudaStream_t, void* const*, bool);
     int (*smooth_batch)(const ks_model_batch*, const float*, int64_t, void*, size_t, float*, float*, float*,
                         float*, cudaStream_t, bool);
+    // the scan-only entry points; the element arrays start at byte `off_elems`
+    int (*filter_scan)(const ks_model*, int64_t, void*, size_t, float*, float*, size_t off_elems, cudaStream_t);
+    int (*smooth_scan)(const ks_model*, int64_t, const float*, const float*, void*, size_t, float*, float*,
+                       cudaStream_t);
 };
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -320,7 +324,10 @@ struct Impl {
 
     static int build_elements(const ks_model* m, const float* y, int64_t T, void* ws, size_t ws_bytes,
                               cudaStream_t st) {
-        const Layout L = layout(T);
+        return build_elements_at(m, y, T, ws, ws_bytes, layout(T), st);
+    }
+    static int build_elements_at(const ks_model* m, const float* y, int64_t T, void* ws, size_t ws_bytes,
+                                 const Layout& L, cudaStream_t st) {
         int rc = check_common(m, T, ws, ws_bytes, L.bytes_elements);
         if (rc) return rc;
         if (!y || !aligned16(y)) return KS_EINVAL;
@@ -333,12 +340,16 @@ struct Impl {
 
     static int filter_scan(const ks_model* m, int64_t T, void* ws, size_t ws_bytes, float* fm, float* fc,
                            cudaStream_t st) {
+        return filter_scan_at(m, T, ws, ws_bytes, fm, fc, layout(T).off_elems, st);
+    }
+    static int filter_scan_at(const ks_model* m, int64_t T, void* ws, size_t ws_bytes, float* fm, float* fc,
+                              size_t off_elems, cudaStream_t st) {
         const Layout L = layout(T);
-        int rc = check_common(m, T, ws, ws_bytes, L.bytes_elements);
+        int rc = check_common(m, T, ws, ws_bytes, off_elems + 4 * (size_t)NCOMP * (size_t)L.ld);
         if (rc) return rc;
         if (!fm || !fc || !aligned16(fm) || !aligned16(fc)) return KS_EINVAL;
         if ((rc = reset_flags(ws, L, st))) return rc;
-        const float* el = reinterpret_cast<const float*>(static_cast<char*>(ws) + L.off_elems);
+        const float* el = reinterpret_cast<const float*>(static_cast<char*>(ws) + off_elems);
         return launch_filter_soa(ws, L, el, fm, fc, st);
     }
 
@@ -531,7 +542,7 @@ struct Impl {
         return VTable{N, M, &layout, &build_elements, &filter_scan, &smooth_scan, &smooth, &smooth_batch,
                       &fcomb_batch, &scomb_batch, &agg_bytes, &faggregate, &saggregate, &tv_bytes};
     }
-    static constexpr ChunkVariant chunk_variant() { return ChunkVariant{&layout, &smooth_v, &smooth_batch_v}; }
+    static constexpr ChunkVariant chunk_variant() { return ChunkVariant{&layout, &smooth_v, &smooth_batch_v, &filter_scan_at, &smooth_scan}; }
 };
 
 // Steps per thread of the fused smooth / smooth_batch scans, picked from
@@ -566,10 +577,12 @@ struct ChunkTable {
     static const ChunkVariant* const v[4];
 };
 
-// The registered function table: every entry of the 32-step Impl, except that
-// smooth and smooth_batch go to the chunk variant chosen by T, and the
-// workspace sizes cover every variant (offsets stay the 32-step layout's,
-// which the element-building and scan-only entry points use).
+// The registered function table: the entry points that scan go to the chunk
+// variant chosen by T (the scan-only ones by the built-in rule: their tiles
+// idle the chip at short T just as the fused ones do; at nx = 4, T = 262147
+// the three-call form takes 383 us at 32 steps per thread), and the workspace
+// covers every variant.  The element arrays start behind the largest variant's
+// scratch, at the offset that ks_elements_layout_get reports.
 template <int N, int M>
 struct Tuned {
     using Base = Impl<N, M, 32>;
@@ -580,7 +593,28 @@ struct Tuned {
             L.bytes_smooth = std::max(L.bytes_smooth, Li.bytes_smooth);
             L.bytes_elements = std::max(L.bytes_elements, Li.bytes_elements);
         }
+        const size_t elems = 4 * (size_t)Base::NCOMP * (size_t)L.ld;
+        L.off_elems = L.bytes_smooth;
+        L.bytes_elements = std::max(L.bytes_elements, align_up(L.off_elems + elems, 256));
         return L;
+    }
+    static int build_elements(const ks_model* m, const float* y, int64_t T, void* ws, size_t ws_bytes,
+                              cudaStream_t st) {
+        if (T < 1 || T > 0x7fffffffLL) return KS_EINVAL;
+        return Base::build_elements_at(m, y, T, ws, ws_bytes, layout(T, 1), st);
+    }
+    static int filter_scan(const ks_model* m, int64_t T, void* ws, size_t ws_bytes, float* fm, float* fc,
+                           cudaStream_t st) {
+        if (T < 1 || T > 0x7fffffffLL) return KS_EINVAL;
+        const Layout L = layout(T, 1);
+        if (ws_bytes < L.bytes_elements) return Base::check_common(m, T, ws, ws_bytes, L.bytes_elements);
+        return ChunkTable<N, M>::v[builtin_chunk_index(T)]->filter_scan(m, T, ws, ws_bytes, fm, fc, L.off_elems, st);
+    }
+    static int smooth_scan(const ks_model* m, int64_t T, const float* fm, const float* fc, void* ws,
+                           size_t ws_bytes, float* sm, float* sc, cudaStream_t st) {
+        if (T < 1 || T > 0x7fffffffLL) return KS_EINVAL;
+        if (ws_bytes < layout(T, 1).bytes_smooth) return Base::check_common(m, T, ws, ws_bytes, (size_t)-1);
+        return ChunkTable<N, M>::v[builtin_chunk_index(T)]->smooth_scan(m, T, fm, fc, ws, ws_bytes, sm, sc, st);
     }
     static int smooth(const ks_model* m, const float* y, int64_t T, void* ws, size_t ws_bytes, float* fm,
                       float* fc, float* sm, float* sc, cudaStream_t st, void* const* ev) {
@@ -600,6 +634,9 @@ struct Tuned {
         VTable t = Base::vtable();
         t.layout = &layout;
         t.tv_bytes = &tv_bytes;
+        t.build_elements = &build_elements;
+        t.filter_scan = &filter_scan;
+        t.smooth_scan = &smooth_scan;
         t.smooth = &smooth;
         t.smooth_batch = &smooth_batch;
         return t;
