@@ -593,11 +593,13 @@ KS_DEV float in_sd(const float (&x)[N], const float* __restrict__ rsd) {
     return m;
 }
 
+// Whether every component is a number below 1e30: beyond that the scans decide
+// (their products overflow earlier than a matrix-vector recursion's).
 template <int N>
 KS_DEV bool all_finite(const float (&x)[N]) {
     float s = 0.f;
 #pragma unroll
-    for (int a = 0; a < N; ++a) s = fmaf(x[a], 0.f, s);
+    for (int a = 0; a < N; ++a) s = fabsf(x[a]) < 1e30f ? s : 1.f;
     return s == 0.f;
 }
 

@@ -5,6 +5,7 @@
 #pragma once
 
 #include "ks_gimpl.cuh"
+#include "ks_steady32.cuh"
 #include "ks_tscan.cuh"
 
 namespace ks {
@@ -26,6 +27,8 @@ struct TImpl {
         size_t off = 256;
         L.off_const = off;
         off = align_up(off + sizeof(ModelConst<N, M>), 256);
+        L.off_plan = off;                                   // the settled path's plan and scratch
+        off = align_up(off + s32_bytes(T), 256);
         L.off_flags = off;                                  // zeroed by the preparation kernel
         L.flags_bytes = 16;
         off = align_up(off + L.flags_bytes, 256);
@@ -171,11 +174,24 @@ struct TImpl {
         }
         if (!vec_ok(fm, fc, filter_only ? fm : sm, filter_only ? fc : sc)) return KS_EINVAL;
         if (ev && ev[0] && record_event(ev[0], st) != cudaSuccess) return KS_ECUDA;
-        if ((rc = GImpl<N, M, NW, CH>::prep(m->F, m->u, m->Q, m->H, m->d, m->R, m->m0, m->P0, y, 1, nullptr, ws,
-                                            L, st)))
-            return rc;
+        const uint32_t* gate = nullptr;
+        Args32 g{};
+        if (T >= kS32MinT) {   // the settled path, with the scans gated behind it
+            static_assert(N == 32 && M == 8, "ks_steady32.cu is this size's");
+            gate = static_cast<uint32_t*>(ws);
+            char* w = static_cast<char*>(ws);
+            g = Args32{m->F, m->u, m->Q, m->H, m->d, m->R, m->m0, m->P0, y, T,
+                       reinterpret_cast<ModelConst<32, 8>*>(w + L.off_const), static_cast<uint32_t*>(ws),
+                       reinterpret_cast<uint32_t*>(w + L.off_flags), (int)(L.flags_bytes / 4), fm, fc,
+                       filter_only ? nullptr : sm, filter_only ? nullptr : sc, own ? 0 : 1, s32_at(w + L.off_plan, T)};
+            rc = launch_steady32_plan(g, st);
+        } else {
+            rc = GImpl<N, M, NW, CH>::prep(m->F, m->u, m->Q, m->H, m->d, m->R, m->m0, m->P0, y, 1, nullptr, ws, L, st);
+        }
+        if (rc) return rc;
         if (ev && ev[1] && record_event(ev[1], st) != cudaSuccess) return KS_ECUDA;
-        if ((rc = scans(ws, L, y, fm, fc, sm, sc, st, ev, true, !filter_only))) return rc;
+        if (gate != nullptr && (rc = launch_steady32(g, st))) return rc;
+        if ((rc = scans(ws, L, y, fm, fc, sm, sc, st, ev, true, !filter_only, gate))) return rc;
         if (ev && ev[3] && record_event(ev[3], st) != cudaSuccess) return KS_ECUDA;
         return KS_OK;
     }

@@ -127,6 +127,42 @@ def test_non_finite_measurement_takes_the_scans(ks, nx, value, at):
         assert general == 1
 
 
+# nx = 32 takes the settled path from 768 rows on: edges of its chunks of 32,
+# of the eight chunks behind a chunk, and of a block's eight chunks
+@pytest.mark.parametrize("T", [767, 768, 769, 799, 800, 801, 1151, 1152, 1153, 2000, 5000])
+def test_edges_nx32(ks, T):
+    rng = np.random.default_rng(9000 + T)
+    m = model_of(32, rng)
+    _, y = workloads.simulate(m, T, rng)
+    out, ws, general = call(ks, m, y)
+    assert ks.status(ws) == ks.KS_OK and general == 0
+    parity.check_all(out, oracle.kf_rts(m, np.asarray(y, dtype=np.float64)), parity.TOL_NX32)
+    f, ws, general = call(ks, m, y, filter_only=True)
+    assert general == 0 and torch.equal(f[0], out[0]) and torch.equal(f[1], out[1])
+    s, ws, general = call(ks, m, y, keep_filtered=False)
+    assert general == 0 and torch.equal(s[2], out[2]) and torch.equal(s[3], out[3])
+
+
+@pytest.mark.parametrize("at", [0, 100, 1500, 2999])
+def test_nx32_leaves_for_the_scans(ks, at):
+    rng = np.random.default_rng(95)
+    m = workloads.random_stable(32, 8, rng)
+    _, y = workloads.simulate(m, 3000, rng)
+    y = y.copy()
+    y[at, 0] = np.nan
+    out, ws, general = call(ks, m, y)
+    ref, wr = scans(ks, m, y)
+    assert general == 1 and ks.status(ws) == ks.status(wr)
+    assert all(torch.equal(torch.isfinite(a), torch.isfinite(b)) for a, b in zip(out, ref))
+    slow = workloads.random_stable(32, 8, rng, q=1e-8)      # does not settle
+    _, y = workloads.simulate(slow, 3000, rng)
+    out, ws, general = call(ks, slow, y)
+    ref, wr = scans(ks, slow, y)
+    assert general == 1
+    for a, b in zip(out, ref):
+        assert torch.allclose(a, b, rtol=1e-4, atol=1e-5 * float(b.abs().max()))
+
+
 def test_unaligned_outputs_nx8(ks):
     """nx = 8 takes any 4-byte aligned posterior buffer (the settled path's row
     copies need 16 bytes, so these go through the scans)."""
