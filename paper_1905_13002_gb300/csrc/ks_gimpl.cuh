@@ -323,4 +323,23 @@ struct GImpl {
     }
 };
 
+// Steps per chain of the nx = 8 scans by length: a chain is one 8-lane group
+// and folds its steps one after another, so that at 32 steps a 20000-step call
+// is 157 warps on 152 SMs.  Shorter chains give more of them; long calls keep
+// 32 (fewer tiles for the spine's levels).
+struct GVariant {
+    Layout (*layout)(int64_t T, int B);
+    int (*smooth_scan)(const ks_model*, int64_t, const float*, const float*, void*, size_t, float*, float*,
+                       cudaStream_t);
+    int (*smooth)(const ks_model*, const float*, int64_t, void*, size_t, float*, float*, float*, float*,
+                  cudaStream_t, void* const*);
+    int (*smooth_batch)(const ks_model_batch*, const float*, int64_t, void*, size_t, float*, float*, float*, float*,
+                        cudaStream_t);
+    size_t (*tv_bytes)(int64_t T);
+};
+template <class G>
+constexpr GVariant gvariant() {
+    return GVariant{&G::layout, &G::smooth_scan, &G::smooth, &G::smooth_batch, &G::tv_bytes};
+}
+
 }  // namespace ks

@@ -89,15 +89,13 @@ inline int launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem
     return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? KS_OK : KS_ECUDA;
 }
 
-// Launch of a scan kernel that takes a gate as its last argument: a plain
-// launch when it is null, else one chained behind the settled path (26 closed
-// kernels behind an nx = 8 batch: 272 us a call chained, 346 us plain).
+// Chained launch of a scan kernel that takes a gate (may be null) as its last
+// argument (26 closed kernels behind an nx = 8 batch: 272 us a call chained,
+// 346 us plain).
 template <class... KArgs, class... Args>
 inline int launch_gated(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st,
                         const uint32_t* gate, Args... args) {
-    if (gate != nullptr) return launch_pdl(kernel, grid, block, smem, st, args..., gate);
-    kernel<<<grid, block, smem, st>>>(args..., gate);
-    return launch_status();
+    return launch_pdl(kernel, grid, block, smem, st, args..., gate);
 }
 
 // FCH_ = steps per thread of the block scans (one tile = 128 * FCH_ steps).

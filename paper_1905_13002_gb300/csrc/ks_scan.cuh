@@ -48,14 +48,13 @@ struct ScanState {
     uint32_t gated = 0;  // run only when general_wanted(status) (behind the settled path of a fused call)
 };
 
-// Start of a kernel that may stand behind the settled path of a fused call
-// (gate: the workspace header, null when it does not): whether it has nothing
-// to do.
+// Start of a scan kernel chained to the one before it.  It may stand behind the
+// settled path of a fused call (gate: the workspace header, null when it does
+// not): returns whether it has nothing to do.
 KS_DEV bool gate_closed(const uint32_t* gate) {
-    if (gate == nullptr) return false;
     pdl_trigger();   // what follows waits too
     pdl_wait();
-    return !general_wanted(gate);
+    return gate != nullptr && !general_wanted(gate);
 }
 
 KS_DEV uint32_t wait_limit(const ScanState& ss) {
