@@ -43,11 +43,11 @@ struct HImpl {
         L.off_fpre = off;
         off = align_up(off + sizeof(FS<K>) * (size_t)L.ntiles, 256);
         L.off_sagg = off;
-        off = align_up(off + sizeof(SE<K>) * (size_t)L.ntiles, 256);
+        off = align_up(off + sizeof(FE<K>) * (size_t)L.ntiles, 256);
         L.off_spre = off;
         off = align_up(off + sizeof(SS<K>) * (size_t)L.ntiles, 256);
-        L.off_sblk = off;                                   // one smoothing aggregate per CH steps
-        off = align_up(off + sizeof(SE<K>) * (size_t)L.nblk, 256);
+        L.off_sblk = off;                                   // one block element per CH steps
+        off = align_up(off + sizeof(FE<K>) * (size_t)L.nblk, 256);
         L.bytes = off;
         return L;
     }
@@ -82,11 +82,13 @@ struct HImpl {
                                              reinterpret_cast<uint32_t*>(b + L.off_flags), (int)(L.flags_bytes / 4));
         if ((rc = launch_status())) return rc;
         if ((rc = rec(1))) return rc;
-        hmm_filter_kernel<K, NT, CH><<<L.ntiles, NT, 0, st>>>(cg, lik, T, filt, loglik, state(ws, L, true), sblk);
+        hmm_filter_kernel<K, NT, CH><<<L.ntiles, NT, 0, st>>>(cg, lik, T, filt, loglik, state(ws, L, true),
+                                                               smooth ? sblk : nullptr);
         if ((rc = launch_status())) return rc;
         if ((rc = rec(2))) return rc;
         if (smooth) {
-            hmm_smoother_kernel<K, NT, CH><<<L.ntiles, NT, 0, st>>>(cg, filt, T, smooth, state(ws, L, false), sblk);
+            hmm_smoother_kernel<K, NT, CH><<<L.ntiles, NT, 0, st>>>(cg, lik, filt, T, smooth, state(ws, L, false),
+                                                                     sblk);
             if ((rc = launch_status())) return rc;
         }
         return rec(3);
@@ -121,8 +123,8 @@ struct WImpl {
     struct WLayout {
         int64_t nch = 0;
         int ntiles = 0;
-        size_t off_const = 0, off_fexcl = 0, off_fsp0 = 0, off_fsp1 = 0, off_schain = 0, off_sexcl = 0,
-               off_ssp0 = 0, off_ssp1 = 0, bytes = 0;
+        size_t off_const = 0, off_fexcl = 0, off_fsp0 = 0, off_fsp1 = 0, off_chain = 0, off_ssp0 = 0, off_ssp1 = 0,
+               bytes = 0;
     };
     static WLayout layout(int64_t T) {
         using D = hmmw::Dims<K>;
@@ -138,14 +140,12 @@ struct WImpl {
         off = align_up(off + 4 * (size_t)D::FREC * L.ntiles, 256);
         L.off_fsp1 = off;
         off = align_up(off + 4 * (size_t)D::FREC * L.ntiles, 256);
-        L.off_schain = off;
-        off = align_up(off + 4 * (size_t)D::SREC * L.nch, 256);
-        L.off_sexcl = off;
-        off = align_up(off + 4 * (size_t)D::SREC * L.nch, 256);
+        L.off_chain = off;
+        off = align_up(off + 4 * (size_t)D::FREC * L.nch, 256);
         L.off_ssp0 = off;
-        off = align_up(off + 4 * (size_t)D::SREC * L.ntiles, 256);
+        off = align_up(off + 4 * (size_t)D::FREC * L.ntiles, 256);
         L.off_ssp1 = off;
-        off = align_up(off + 4 * (size_t)D::SREC * L.ntiles, 256);
+        off = align_up(off + 4 * (size_t)D::FREC * L.ntiles, 256);
         L.bytes = off;
         return L;
     }
@@ -164,8 +164,7 @@ struct WImpl {
         bf.fexcl = reinterpret_cast<float*>(b + L.off_fexcl);
         bf.fspine0 = reinterpret_cast<float*>(b + L.off_fsp0);
         bf.fspine1 = reinterpret_cast<float*>(b + L.off_fsp1);
-        bf.schain = reinterpret_cast<float*>(b + L.off_schain);
-        bf.sexcl = reinterpret_cast<float*>(b + L.off_sexcl);
+        bf.chain = smooth ? reinterpret_cast<float*>(b + L.off_chain) : nullptr;
         bf.sspine0 = reinterpret_cast<float*>(b + L.off_ssp0);
         bf.sspine1 = reinterpret_cast<float*>(b + L.off_ssp1);
         auto rec = [&](int i) {
@@ -193,8 +192,6 @@ struct WImpl {
         if ((rc = launch_status())) return rc;
         if ((rc = rec(2))) return rc;
         if (smooth) {
-            smoother_reduce_kernel<K, NW><<<L.ntiles, NW * 32, 0, st>>>(L.nch, bf, stat);
-            if ((rc = launch_status())) return rc;
             const float* ssrc = bf.sspine0;
             float* sdst = bf.sspine1;
             for (int s = 1; s < L.ntiles; s <<= 1) {
@@ -204,7 +201,8 @@ struct WImpl {
                 ssrc = sdst;
                 sdst = t;
             }
-            smoother_apply_kernel<K, NW, CH><<<L.ntiles, NW * 32, 0, st>>>(cg, filt, T, smooth, bf, ssrc, stat);
+            smoother_apply_kernel<K, NW, CH><<<L.ntiles, NW * 32, 0, st>>>(cg, lik, filt, T, smooth, bf, ssrc, L.ntiles,
+                                                                           stat);
             if ((rc = launch_status())) return rc;
         }
         return rec(3);

@@ -49,11 +49,6 @@ struct FS {
     float pad[(K + 1) % 2 == 0 ? 1 : 0];
 };
 template <int K>
-struct SE {
-    float a[K * K];
-    float pad[(K * K) % 2 == 0 ? 1 : 0];
-};
-template <int K>
 struct SS {
     float s[K];
     float pad[K % 2 == 0 ? 1 : 0];
@@ -96,14 +91,6 @@ KS_DEV void set_identity(FE<K>& e) {
         for (int x = 0; x < K; ++x) e.f[z * K + x] = (z == x) ? 1.f : 0.f;
         e.lg[z] = 0.f;
     }
-}
-
-template <int K>
-KS_DEV void set_identity(SE<K>& e) {
-#pragma unroll
-    for (int z = 0; z < K; ++z)
-#pragma unroll
-        for (int x = 0; x < K; ++x) e.a[z * K + x] = (z == x) ? 1.f : 0.f;
 }
 
 // Likelihood row of step k scaled to a maximum of 1; returns log of the
@@ -193,10 +180,37 @@ KS_DEV void fadvance(FS<K>& st, const FE<K>& e, Flags& bad) {
     st.L += mx + __logf(d);
 }
 
-// Aggregate (x) step element, with l the scaled likelihood row and lm the log
-// of its scale (see the header).  Pi is read from shared memory.
+// 2^-e and e for the exponent e of a positive finite r (r 2^-e in [1, 2); a
+// subnormal r keeps e = -127).
+KS_DEV float pow2_of(float r, int& e) {
+    e = (int)(__float_as_uint(r) >> 23) - 127;
+    return __uint_as_float((uint32_t)(127 - e) << 23);
+}
+
+// Likelihood row scaled by a power of two to a maximum in [1, 2); returns the
+// exponent taken out.
 template <int K>
-KS_DEV void ffold_step(FE<K>& acc, const float* __restrict__ Pi, const float (&l)[K], float lm, Flags& bad) {
+KS_DEV int scale_lik2(float (&l)[K], Flags& bad) {
+    float m = 0.f;
+#pragma unroll
+    for (int x = 0; x < K; ++x) m = fmaxf(m, l[x]);
+    const bool ok = m > 0.f && m <= 3.0e38f;
+    bad |= !ok;
+    int e;
+    const float s = pow2_of(ok ? m : 1.f, e);
+#pragma unroll
+    for (int x = 0; x < K; ++x) l[x] *= s;
+    return e;
+}
+
+// Aggregate (x) step element, with l the scaled likelihood row.  A row is
+// kept at a sum in [1, 2) by a power of two, whose exponents are added up in
+// ex: the fold needs no division and no logarithm (they were K of each per
+// step beside the K^3 products) and the scaling is exact.  Pi is read from
+// shared memory.
+template <int K>
+KS_DEV void ffold_step(FE<K>& acc, int (&ex)[K], const float* __restrict__ Pi, const float (&l)[K], int le,
+                       Flags& bad) {
     float row[K][K];   // row[z][x] accumulates (f Pi)[z][x], one Pi row at a time
 #pragma unroll
     for (int z = 0; z < K; ++z)
@@ -220,30 +234,37 @@ KS_DEV void ffold_step(FE<K>& acc, const float* __restrict__ Pi, const float (&l
             r += row[z][x];
         }
         bad |= !(r > 0.f);
-        const float rr = 1.f / r;
+        int e;
+        const float s = pow2_of(r, e);
 #pragma unroll
-        for (int x = 0; x < K; ++x) acc.f[z * K + x] = row[z][x] * rr;
-        acc.lg[z] += lm + __logf(r);
+        for (int x = 0; x < K; ++x) acc.f[z * K + x] = row[z][x] * s;
+        ex[z] += e + le;
     }
 }
 
-// The step element itself (fold of the identity).
+// End of a fold: rows of sum one, log g from the exponents and the last sums.
 template <int K>
-KS_DEV void step_element(FE<K>& e, const float* __restrict__ Pi, const float (&l)[K], float lm, Flags& bad) {
+KS_DEV void ffold_end(FE<K>& acc, const int (&ex)[K], Flags& bad) {
 #pragma unroll
     for (int z = 0; z < K; ++z) {
         float r = 0.f;
 #pragma unroll
-        for (int x = 0; x < K; ++x) {
-            e.f[z * K + x] = Pi[z * K + x] * l[x];
-            r += e.f[z * K + x];
-        }
+        for (int x = 0; x < K; ++x) r += acc.f[z * K + x];
         bad |= !(r > 0.f);
         const float rr = 1.f / r;
 #pragma unroll
-        for (int x = 0; x < K; ++x) e.f[z * K + x] *= rr;
-        e.lg[z] = lm + __logf(r);
+        for (int x = 0; x < K; ++x) acc.f[z * K + x] *= rr;
+        acc.lg[z] = fmaf((float)ex[z], 0.693147180559945f, logf(r));
     }
+}
+
+// The step element itself, rows of sum below 2 (the start of a fold).
+template <int K>
+KS_DEV void step_element(FE<K>& e, const float* __restrict__ Pi, const float (&l)[K]) {
+#pragma unroll
+    for (int z = 0; z < K; ++z)
+#pragma unroll
+        for (int x = 0; x < K; ++x) e.f[z * K + x] = Pi[z * K + x] * l[x];
 }
 
 // Step 1's element as a prefix state: p(x_1 | y_1) and log p(y_1).
@@ -292,61 +313,6 @@ KS_DEV void fadvance_step(FS<K>& st, const float* __restrict__ Pi, const float (
     st.L = L;
 }
 
-// Smoothing element of step k from its filtered marginal p (k < n):
-// a(x | z) = p(x) Pi[x][z] / sum_x' p(x') Pi[x'][z].
-template <int K>
-KS_DEV void selem(SE<K>& e, const float* __restrict__ PiT, const float (&p)[K], Flags& bad) {
-#pragma unroll
-    for (int z = 0; z < K; ++z) {
-        float pc[K], d = 0.f;
-        load_row<K>(PiT, z, pc);   // column z of Pi
-#pragma unroll
-        for (int x = 0; x < K; ++x) {
-            e.a[z * K + x] = p[x] * pc[x];
-            d += e.a[z * K + x];
-        }
-        bad |= !(d > 0.f);
-        const float rd = 1.f / d;
-#pragma unroll
-        for (int x = 0; x < K; ++x) e.a[z * K + x] *= rd;
-    }
-}
-
-// Smoothing element of the last step: a(x | z) = p_n(x) for every z.
-template <int K>
-KS_DEV void selem_last(SE<K>& e, const float (&p)[K]) {
-#pragma unroll
-    for (int z = 0; z < K; ++z)
-#pragma unroll
-        for (int x = 0; x < K; ++x) e.a[z * K + x] = p[x];
-}
-
-// Definition 2 in matrix form: (a_i (x) a_j)[z][x] = sum_y a_j[z][y] a_i[y][x]
-// (i earlier), i.e. the product a_j a_i.
-// The rows of a product of row-stochastic matrices sum to one in exact
-// arithmetic; each row is rescaled to that sum, so that the rounding of the
-// total probability does not build up along the look-back's chain of tile
-// prefixes (one product per tile).
-template <int K>
-KS_DEV SE<K> smatmul(SE<K> l, const SE<K>& r) {   // l r, l overwritten row by row
-#pragma unroll
-    for (int z = 0; z < K; ++z) {
-        float o[K], t = 0.f;
-#pragma unroll
-        for (int x = 0; x < K; ++x) {
-            float s = 0.f;
-#pragma unroll
-            for (int y = 0; y < K; ++y) s = fmaf(l.a[z * K + y], r.a[y * K + x], s);
-            o[x] = s;
-            t += s;
-        }
-        const float rt = 1.f / t;
-#pragma unroll
-        for (int x = 0; x < K; ++x) l.a[z * K + x] = o[x] * rt;
-    }
-    return l;
-}
-
 template <int K>
 struct FilterOp {
     using Elem = FE<K>;
@@ -368,39 +334,88 @@ struct FilterOp {
     }
 };
 
-// Reverse scan in scan (reversed-time) order: x (x)_r y = y (x) x, which in
-// matrix form is x.a y.a.
+// beta(z) = p(measurements of an element and what follows | state z before it),
+// up to a factor: exp(lg(z) - max) (f v)(z) for the following v, rescaled by a
+// power of two to a maximum in [1, 2).
 template <int K>
-struct SmootherOp {
-    using Elem = SE<K>;
+KS_DEV void beta_of(float (&v)[K], const float (&lg)[K]) {
+    float mx = lg[0];
+#pragma unroll
+    for (int z = 1; z < K; ++z) mx = fmaxf(mx, lg[z]);
+    float m = 0.f;
+#pragma unroll
+    for (int z = 0; z < K; ++z) {
+        v[z] *= __expf(lg[z] - mx);
+        m = fmaxf(m, v[z]);
+    }
+    int e;
+    const float s = pow2_of(m, e);
+#pragma unroll
+    for (int z = 0; z < K; ++z) v[z] *= s;
+}
+
+// Reverse scan over the forward scan's own block elements, in reversed time
+// order (x (x)_r y = y (x) x); a suffix that reaches the last measurement only
+// needs beta.
+template <int K>
+struct BetaOp {
+    using Elem = FE<K>;
     using State = SS<K>;
-    KS_DEV static Elem combine(const Elem& a, const Elem& b, Flags&) { return smatmul<K>(a, b); }
-    KS_DEV static void advance(State& s, const Elem& e, Flags&) {   // s <- s e.a, rescaled to sum 1
-        float o[K], t = 0.f;
+    // log g relative to its largest: the sum over a long suffix would leave no
+    // bits for the differences between states
+    KS_DEV static Elem combine(const Elem& a, const Elem& b, Flags& bad) {
+        Elem r = fcombine<K>(b, a, bad);
+        float mx = r.lg[0];
 #pragma unroll
-        for (int x = 0; x < K; ++x) {
-            float v = 0.f;
+        for (int z = 1; z < K; ++z) mx = fmaxf(mx, r.lg[z]);
 #pragma unroll
-            for (int z = 0; z < K; ++z) v = fmaf(s.s[z], e.a[z * K + x], v);
-            o[x] = v;
-            t += v;
+        for (int z = 0; z < K; ++z) r.lg[z] -= mx;
+        return r;
+    }
+    KS_DEV static void advance(State& s, const Elem& e, Flags&) {
+        float v[K];
+#pragma unroll
+        for (int z = 0; z < K; ++z) {
+            float o = 0.f;
+#pragma unroll
+            for (int x = 0; x < K; ++x) o = fmaf(e.f[z * K + x], s.s[x], o);
+            v[z] = o;
         }
-        const float rt = 1.f / t;
+        beta_of<K>(v, e.lg);
 #pragma unroll
-        for (int x = 0; x < K; ++x) s.s[x] = o[x] * rt;
+        for (int z = 0; z < K; ++z) s.s[z] = v[z];
     }
     KS_DEV static void identity(Elem& e) { set_identity<K>(e); }
     KS_DEV static void zero_state(State& s) {
 #pragma unroll
         for (int x = 0; x < K; ++x) s.s[x] = 0.f;
     }
-    KS_DEV static State state_of(const Elem& e) {
+    KS_DEV static State state_of(const Elem& e) {   // rows of sum one
         State s;
 #pragma unroll
-        for (int x = 0; x < K; ++x) s.s[x] = e.a[x];
+        for (int x = 0; x < K; ++x) s.s[x] = 1.f;
+        beta_of<K>(s.s, e.lg);
         return s;
     }
 };
+
+// Smoothed marginal p beta / sum.  The factors are scaled up before the
+// product so that a very unlikely sequence (p and beta far apart) does not
+// underflow: p <= 1 and beta < 2, so the sum stays below 2^127.
+template <int K>
+KS_DEV void smoothed(const float (&p)[K], const float (&b)[K], float (&o)[K], Flags& bad) {
+    constexpr float kUp = 1.152921504606847e18f;   // 2^60
+    float t = 0.f;
+#pragma unroll
+    for (int x = 0; x < K; ++x) {
+        o[x] = (p[x] * kUp) * (b[x] * kUp);
+        t += o[x];
+    }
+    bad |= !(t > 0.f);
+    const float r = 1.f / t;
+#pragma unroll
+    for (int x = 0; x < K; ++x) o[x] *= r;
+}
 
 // ---------------------------------------------------------------- kernels
 // Model constants (q1 = pi Pi) and the scans' counters and flags.
@@ -435,13 +450,15 @@ KS_DEV void load_const(const Const<K>* __restrict__ g, Const<K>& s, int tid, int
 }
 
 // Forward scan: filtered marginals filt [T][K], running log-likelihoods
-// loglik [T] (may be null), and each thread's smoothing aggregate (its CH
-// steps' Definition 2 elements folded forward) in sagg.
+// loglik [T] (may be null), and each thread's block element in blk (may be
+// null), which the reverse scan starts from: smoothing as p_k beta_k / sum
+// (two filters) needs no Definition 2 elements, whose fold cost another K^3
+// and K divisions per step (2.1 times the products of this scan at K = 8).
 template <int K, int NT, int CH>
 __global__ void __launch_bounds__(NT) hmm_filter_kernel(const Const<K>* __restrict__ cg,
                                                         const float* __restrict__ lik, int64_t T,
                                                         float* __restrict__ filt, float* __restrict__ loglik,
-                                                        ScanState ss, float* __restrict__ sagg) {
+                                                        ScanState ss, float* __restrict__ blk) {
     using BS = BlockScan<FilterOp<K>, NT>;
     constexpr int64_t TILE = (int64_t)NT * CH;
     __shared__ __align__(16) Const<K> mc;
@@ -463,18 +480,20 @@ __global__ void __launch_bounds__(NT) hmm_filter_kernel(const Const<K>* __restri
         set_identity<K>(acc);
     } else {
         float l[K];
-        const float lm = load_lik<K>(lik, k0, l, bad);
+        int ex[K];
+        load_raw<K>(lik, k0, l);
+        {
+            const int le = scale_lik2<K>(l, bad);
+#pragma unroll
+            for (int z = 0; z < K; ++z) ex[z] = le;
+        }
         if (k0 == 0) {        // step 1: rows p(x_1 | y_1), g = p(y_1)
-            FS<K> s1;
-            first_state<K>(s1, mc.q1, l, lm, bad);
 #pragma unroll
-            for (int z = 0; z < K; ++z) {
+            for (int z = 0; z < K; ++z)
 #pragma unroll
-                for (int x = 0; x < K; ++x) acc.f[z * K + x] = s1.p[x];
-                acc.lg[z] = s1.L;
-            }
+                for (int x = 0; x < K; ++x) acc.f[z * K + x] = mc.q1[x] * l[x];
         } else {
-            step_element<K>(acc, mc.Pi, l, lm, bad);
+            step_element<K>(acc, mc.Pi, l);
         }
         // the next step's likelihood row is loaded while the current one folds
         float ln[K];
@@ -485,9 +504,20 @@ __global__ void __launch_bounds__(NT) hmm_filter_kernel(const Const<K>* __restri
 #pragma unroll
             for (int x = 0; x < K; ++x) l[x] = ln[x];
             if (i + 1 < last) load_raw<K>(lik, k0 + i + 1, ln);
-            const float lmk = scale_lik<K>(l, bad);
-            ffold_step<K>(acc, mc.Pi, l, lmk, bad);
+            const int le = scale_lik2<K>(l, bad);
+            ffold_step<K>(acc, ex, mc.Pi, l, le, bad);
         }
+        if (blk != nullptr) {   // for beta only the differences of log g count: the common exponent stays out
+            int top = ex[0], rel[K];
+#pragma unroll
+            for (int z = 1; z < K; ++z) top = max(top, ex[z]);
+#pragma unroll
+            for (int z = 0; z < K; ++z) rel[z] = ex[z] - top;
+            FE<K> e = acc;
+            ffold_end<K>(e, rel, bad);
+            store_plain(blk + (k0 / CH) * (int64_t)(sizeof(FE<K>) / 4), e);
+        }
+        ffold_end<K>(acc, ex, bad);
     }
 
     // ---- phase 2
@@ -497,7 +527,6 @@ __global__ void __launch_bounds__(NT) hmm_filter_kernel(const Const<K>* __restri
 
     // ---- phase 3: step through the block from the incoming prefix
     if (valid) {
-        SE<K> sacc;
         float comp = 0.f, probe = 0.f;
         const int last = (int)((k0 + CH <= T ? k0 + CH : T) - k0);
         float ln[K];
@@ -523,26 +552,22 @@ __global__ void __launch_bounds__(NT) hmm_filter_kernel(const Const<K>* __restri
             }
             if (loglik) loglik[k] = st.L;
             probe += st.L;
-            SE<K> e;
-            if (k == T - 1) selem_last<K>(e, st.p);
-            else selem<K>(e, mc.PiT, st.p, bad);
-            sacc = (i == 0) ? e : smatmul<K>(e, sacc);   // a_k0 (x) ... (x) a_k = a_k ... a_k0
         }
-        store_plain(sagg + (k0 / CH) * (int64_t)(sizeof(SE<K>) / 4), sacc);
         bad |= !isfinite(probe);
     }
     report_flags(ss.status, bad, kFull, (tid & 31) == 0);
 }
 
-// Reverse scan over the forward scan's per-thread smoothing aggregates; each
-// thread then walks its steps backwards from the suffix after them, writing
-// smooth [T][K].
+// Reverse scan over the forward scan's block elements; each thread then walks
+// its steps backwards with beta_{k-1} = Pi (l_k . beta_k), writing
+// smooth [T][K] = filt . beta / sum.
 template <int K, int NT, int CH>
 __global__ void __launch_bounds__(NT) hmm_smoother_kernel(const Const<K>* __restrict__ cg,
+                                                          const float* __restrict__ lik,
                                                           const float* __restrict__ filt, int64_t T,
                                                           float* __restrict__ smooth, ScanState ss,
-                                                          const float* __restrict__ sagg) {
-    using BS = BlockScan<SmootherOp<K>, NT>;
+                                                          const float* __restrict__ blk) {
+    using BS = BlockScan<BetaOp<K>, NT>;
     __shared__ __align__(16) Const<K> mc;
     __shared__ typename BS::Smem bsm;
     __shared__ int s_tile;
@@ -559,8 +584,8 @@ __global__ void __launch_bounds__(NT) hmm_smoother_kernel(const Const<K>* __rest
     const int64_t khi = valid ? ((klo + CH < T ? klo + CH : T) - 1) : -1;
     Flags bad = 0u;
 
-    SE<K> acc;
-    if (valid) acc = load_cg<SE<K>>(sagg + c * (int64_t)(sizeof(SE<K>) / 4));
+    FE<K> acc;
+    if (valid) acc = load_cg<FE<K>>(blk + c * (int64_t)(sizeof(FE<K>) / 4));
     else set_identity<K>(acc);
 
     SS<K> st;
@@ -569,24 +594,46 @@ __global__ void __launch_bounds__(NT) hmm_smoother_kernel(const Const<K>* __rest
 
     if (valid) {
         float probe = 0.f;
-        float pn[K];
+        float pn[K], ln[K], b[K];
+#pragma unroll
+        for (int x = 0; x < K; ++x) b[x] = has ? st.s[x] : 1.f;   // nothing after the last step
         load_raw<K>(filt, khi, pn);
+        load_raw<K>(lik, khi, ln);
 #pragma unroll 1
         for (int64_t k = khi; k >= klo; --k) {
-            float p[K];
-#pragma unroll
-            for (int x = 0; x < K; ++x) p[x] = pn[x];
-            if (k > klo) load_raw<K>(filt, k - 1, pn);
-            SE<K> e;
-            if (k == T - 1) selem_last<K>(e, p);
-            else selem<K>(e, mc.PiT, p, bad);
-            if (!has) { st = SmootherOp<K>::state_of(e); has = true; }   // only k = T - 1
-            else SmootherOp<K>::advance(st, e, bad);
+            float p[K], l[K], o[K];
 #pragma unroll
             for (int x = 0; x < K; ++x) {
-                smooth[k * K + x] = st.s[x];
-                probe += st.s[x];
+                p[x] = pn[x];
+                l[x] = ln[x];
             }
+            if (k > klo) {
+                load_raw<K>(filt, k - 1, pn);
+                load_raw<K>(lik, k - 1, ln);
+            }
+            smoothed<K>(p, b, o, bad);
+#pragma unroll
+            for (int x = 0; x < K; ++x) {
+                smooth[k * K + x] = o[x];
+                probe += o[x];
+            }
+            scale_lik2<K>(l, bad);
+#pragma unroll
+            for (int x = 0; x < K; ++x) l[x] *= b[x];
+            float m = 0.f;
+#pragma unroll
+            for (int z = 0; z < K; ++z) {
+                float pr[K], s = 0.f;
+                load_row<K>(mc.Pi, z, pr);
+#pragma unroll
+                for (int x = 0; x < K; ++x) s = fmaf(pr[x], l[x], s);
+                b[z] = s;
+                m = fmaxf(m, s);
+            }
+            int e;
+            const float s2 = pow2_of(m, e);
+#pragma unroll
+            for (int z = 0; z < K; ++z) b[z] *= s2;
         }
         bad |= !isfinite(probe);
     }

@@ -11,14 +11,16 @@
 //    storing each chain's exclusive in-tile prefix and the tile aggregate;
 //  * spine: Kogge-Stone over the tile aggregates (one launch per level);
 //  * forward apply: each chain starts from its prefix (all rows equal:
-//    p(x | y_1:k) and log p(y_1:k)), steps through its measurements writing
-//    filt and loglik, and folds its Definition 2 elements into one chain
-//    smoothing aggregate;
-//  * reverse reduce / spine / apply over those aggregates in reversed order,
-//    the apply walking each chain backwards from its suffix.
-// Likelihood rows are scaled to a maximum of 1 and g is kept as log g, so
-// that p(y_1:k) survives long prefixes in FP32; products of row-stochastic
-// matrices are rescaled to unit row sums.
+//    p(x | y_1:k) and log p(y_1:k)) and steps through its measurements writing
+//    filt and loglik;
+//  * reverse: smoothing as filt . beta / sum with beta(z) = p(what follows | z).
+//    A spine over the same tile aggregates in reversed order, then an apply:
+//    beta enters a chain through the elements of the tile's later chains, one
+//    matrix-vector product each, and walks the chain backwards.  (Definition 2
+//    elements folded beside the forward apply cost another K^2 products per
+//    lane and step, half of the forward scan.)
+// Likelihood rows are scaled to a maximum near 1 and g is kept as log g, so
+// that p(y_1:k) survives long prefixes in FP32.
 #pragma once
 
 #include "ks_scan.cuh"
@@ -27,17 +29,14 @@ namespace ks {
 namespace hmmw {
 
 // Shared-memory pitches: Pi rows are read by all lanes of a chain at once
-// (broadcast) or a column per lane, so pitch K with float4 rows; Pi^T is read a
-// row per lane, so an odd pitch; element slots are written a row per lane with
-// float4 stores and read by broadcast, so pitch Q (a multiple of 4, rows in
-// distinct banks per quarter-warp).
+// (broadcast), so pitch K with float4 rows; element slots are written a row per
+// lane with float4 stores and read by broadcast, so pitch Q (a multiple of 4,
+// rows in distinct banks per quarter-warp).
 template <int K>
 struct Dims {
-    static constexpr int PT = K + 1;
     static constexpr int Q = K + 4;
     static constexpr int SLOT = K * Q + K;       // rows, then log g
     static constexpr int FREC = K * K + K;       // global filtering record: rows, then log g
-    static constexpr int SREC = K * K;           // global smoothing record: rows
 };
 
 // A chain is K lanes of one warp (lane z = row z); 32 / K chains per warp.
@@ -70,14 +69,29 @@ KS_DEV float group_sum(float v) {
     return v;
 }
 
-// Pi (pitch K) and its transpose (pitch PT) into shared memory.
 template <int K>
-KS_DEV void load_pi(const Const<K>* __restrict__ cg, float* __restrict__ Pi, float* __restrict__ PiT, float* q1) {
-    for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
-        const float v = __ldg(cg->Pi + e);
-        Pi[e] = v;
-        PiT[(e % K) * Dims<K>::PT + e / K] = v;
-    }
+KS_DEV float group_max(float v) {
+#pragma unroll
+    for (int o = K / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(gmask<K>(), v, o, K));
+    return v;
+}
+
+template <int K>
+KS_DEV int group_max_i(int v) {
+#pragma unroll
+    for (int o = K / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(gmask<K>(), v, o, K));
+    return v;
+}
+
+// log g relative to its largest, all that beta needs: over a long suffix the
+// sum itself would leave no bits for the differences between states.
+template <int K>
+KS_DEV void relative_lg(FRow<K>& r) { r.lg -= group_max<K>(r.lg); }
+
+// Pi (pitch K) into shared memory.
+template <int K>
+KS_DEV void load_pi(const Const<K>* __restrict__ cg, float* __restrict__ Pi, float* q1) {
+    for (int e = threadIdx.x; e < K * K; e += blockDim.x) Pi[e] = __ldg(cg->Pi + e);
     for (int e = threadIdx.x; e < K; e += blockDim.x) q1[e] = __ldg(cg->q1 + e);
 }
 
@@ -103,26 +117,6 @@ KS_DEV void store_frow(float* __restrict__ dst, const FRow<K>& r) {
 #pragma unroll
     for (int i = 0; i < K / 4; ++i) p[i] = make_float4(r.f[4 * i], r.f[4 * i + 1], r.f[4 * i + 2], r.f[4 * i + 3]);
     dst[K * K + z] = r.lg;
-}
-
-template <int K>
-KS_DEV void load_srow(const float* __restrict__ src, float (&a)[K]) {
-    const float4* p = reinterpret_cast<const float4*>(src + glane<K>() * K);
-#pragma unroll
-    for (int i = 0; i < K / 4; ++i) {
-        const float4 q = __ldcg(p + i);
-        a[4 * i] = q.x;
-        a[4 * i + 1] = q.y;
-        a[4 * i + 2] = q.z;
-        a[4 * i + 3] = q.w;
-    }
-}
-
-template <int K>
-KS_DEV void store_srow(float* __restrict__ dst, const float (&a)[K]) {
-    float4* p = reinterpret_cast<float4*>(dst + glane<K>() * K);
-#pragma unroll
-    for (int i = 0; i < K / 4; ++i) p[i] = make_float4(a[4 * i], a[4 * i + 1], a[4 * i + 2], a[4 * i + 3]);
 }
 
 // A chain's element in a shared-memory slot (pitch Q rows, then lg).
@@ -153,10 +147,16 @@ KS_DEV void smem_row(const float* __restrict__ M, int y, float (&v)[K]) {
     }
 }
 
-// Likelihood row of step k, the same for every lane, scaled to a maximum of
-// 1; returns the log of the maximum.
+// 2^-e and e for the exponent e of a positive finite r.
+KS_DEV float pow2_of(float r, int& e) {
+    e = (int)(__float_as_uint(r) >> 23) - 127;
+    return __uint_as_float((uint32_t)(127 - e) << 23);
+}
+
+// Likelihood row of step k (the same for every lane) scaled by a power of two
+// to a maximum in [1, 2); returns the exponent taken out.
 template <int K>
-KS_DEV float lik_row(const float* __restrict__ lik, int64_t k, float (&l)[K], Flags& bad) {
+KS_DEV int lik_row2(const float* __restrict__ lik, int64_t k, float (&l)[K], Flags& bad) {
     const float4* p = reinterpret_cast<const float4*>(lik + k * K);
     float m = 0.f;
 #pragma unroll
@@ -169,50 +169,19 @@ KS_DEV float lik_row(const float* __restrict__ lik, int64_t k, float (&l)[K], Fl
     }
 #pragma unroll
     for (int x = 0; x < K; ++x) m = fmaxf(m, l[x]);
-    bad |= !(m > 0.f) || !(m <= 3.0e38f);
-    const float r = 1.f / m;
+    const bool ok = m > 0.f && m <= 3.0e38f;
+    bad |= !ok;
+    int e;
+    const float s = pow2_of(ok ? m : 1.f, e);
 #pragma unroll
-    for (int x = 0; x < K; ++x) l[x] *= r;
-    return __logf(m);
+    for (int x = 0; x < K; ++x) l[x] *= s;
+    return e;
 }
 
-// Row z of the step element: Pi[z][x] l(x) normalised, lg = lm + log(row sum).
+// Fold of a step element into row z: (f Pi)[z] . l, kept at a sum in [1, 2) by
+// a power of two (exponents added up in ex: no division, no logarithm).
 template <int K>
-KS_DEV void step_row(FRow<K>& r, const float* __restrict__ Pi, const float (&l)[K], float lm, Flags& bad) {
-    const int z = glane<K>();
-    float s = 0.f;
-    smem_row<K>(Pi, z, r.f);
-#pragma unroll
-    for (int x = 0; x < K; ++x) {
-        r.f[x] *= l[x];
-        s += r.f[x];
-    }
-    bad |= !(s > 0.f);
-    const float rs = 1.f / s;
-#pragma unroll
-    for (int x = 0; x < K; ++x) r.f[x] *= rs;
-    r.lg = lm + __logf(s);
-}
-
-// The k = 1 element: every row p(x_1 | y_1), lg = log p(y_1).
-template <int K>
-KS_DEV void first_row(FRow<K>& r, const float* __restrict__ q1, const float (&l)[K], float lm, Flags& bad) {
-    float s = 0.f;
-#pragma unroll
-    for (int x = 0; x < K; ++x) {
-        r.f[x] = q1[x] * l[x];
-        s += r.f[x];
-    }
-    bad |= !(s > 0.f);
-    const float rs = 1.f / s;
-#pragma unroll
-    for (int x = 0; x < K; ++x) r.f[x] *= rs;
-    r.lg = lm + __logf(s);
-}
-
-// Fold of a step element into row z: (f Pi)[z] . l, normalised.
-template <int K>
-KS_DEV void fold_row(FRow<K>& r, const float* __restrict__ Pi, const float (&l)[K], float lm, Flags& bad) {
+KS_DEV void fold_row(FRow<K>& r, int& ex, const float* __restrict__ Pi, const float (&l)[K], int le, Flags& bad) {
     float o[K];
 #pragma unroll
     for (int x = 0; x < K; ++x) o[x] = 0.f;
@@ -230,10 +199,24 @@ KS_DEV void fold_row(FRow<K>& r, const float* __restrict__ Pi, const float (&l)[
         s += o[x];
     }
     bad |= !(s > 0.f);
-    const float rs = 1.f / s;
+    int e;
+    const float rs = pow2_of(s, e);
 #pragma unroll
     for (int x = 0; x < K; ++x) r.f[x] = o[x] * rs;
-    r.lg += lm + __logf(s);
+    ex += e + le;
+}
+
+// End of a fold: row of sum one, log g from the exponents and the last sum.
+template <int K>
+KS_DEV void fold_end(FRow<K>& r, int ex, Flags& bad) {
+    float s = 0.f;
+#pragma unroll
+    for (int x = 0; x < K; ++x) s += r.f[x];
+    bad |= !(s > 0.f);
+    const float rs = 1.f / s;
+#pragma unroll
+    for (int x = 0; x < K; ++x) r.f[x] *= rs;
+    r.lg = fmaf((float)ex, 0.693147180559945f, logf(s));
 }
 
 // Definition 1, (row z of a_i, in registers) (x) a_j (in shared memory).
@@ -261,27 +244,6 @@ KS_DEV void combine_row(FRow<K>& r, const float* __restrict__ ej, Flags& bad) {
     r.lg += mx + __logf(d);
 }
 
-// Row z of (a in registers) times (b in shared memory), rescaled to sum 1.
-template <int K>
-KS_DEV void matmul_row(float (&a)[K], const float* __restrict__ b) {
-    float o[K];
-#pragma unroll
-    for (int x = 0; x < K; ++x) o[x] = 0.f;
-#pragma unroll
-    for (int y = 0; y < K; ++y) {
-        float br[K];
-        smem_row<Dims<K>::Q>(b, y, br);
-#pragma unroll
-        for (int x = 0; x < K; ++x) o[x] = fmaf(a[y], br[x], o[x]);
-    }
-    float s = 0.f;
-#pragma unroll
-    for (int x = 0; x < K; ++x) s += o[x];
-    const float rs = 1.f / s;
-#pragma unroll
-    for (int x = 0; x < K; ++x) a[x] = o[x] * rs;
-}
-
 // The prefix (all rows equal) as a state: lane x takes p(x) from row 0.
 template <int K>
 KS_DEV void row0_state(const FRow<K>& r, float& p, float& L) {
@@ -295,27 +257,32 @@ KS_DEV void row0_state(const FRow<K>& r, float& p, float& L) {
     L = __shfl_sync(gmask<K>(), r.lg, 0, K);
 }
 
+// sum_x m[x] v(x) for a vector with v(x) on lane x, through the group's buffer
+// (K floats of shared memory): one store and K / 4 broadcast loads in place of K
+// shuffles.
 template <int K>
-KS_DEV float row0_vec(const float (&a)[K]) {
-    const int lane = glane<K>();
-    float s = 0.f;
+KS_DEV float row_dot(const float (&m)[K], float v, float* __restrict__ buf) {
+    __syncwarp(gmask<K>());
+    buf[glane<K>()] = v;
+    __syncwarp(gmask<K>());
+    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
-    for (int x = 0; x < K; ++x) {
-        const float v = __shfl_sync(gmask<K>(), a[x], 0, K);
-        if (lane == x) s = v;
+    for (int x = 0; x < K; x += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(buf + x);
+        a0 = fmaf(m[x], t.x, a0);
+        a1 = fmaf(m[x + 1], t.y, a1);
+        a2 = fmaf(m[x + 2], t.z, a2);
+        a3 = fmaf(m[x + 3], t.w, a3);
     }
-    return s;
+    return (a0 + a1) + (a2 + a3);
 }
 
-// Filtering state (lane x: p(x)) (x) step: p'(x) = (p Pi)(x) l(x) / c.
+// Filtering state (lane x: p(x)) (x) step: p'(x) = (p Pi)(x) l(x) / c, with the
+// lane's column of Pi in registers.
 template <int K>
-KS_DEV void advance_step(float& p, float& L, float& comp, const float* __restrict__ Pi, float lx, float lm,
+KS_DEV void advance_step(float& p, float& L, float& comp, const float (&col)[K], float lx, float lm, float* buf,
                          Flags& bad) {
-    const int x = glane<K>();
-    float o = 0.f;
-#pragma unroll
-    for (int y = 0; y < K; ++y) o = fmaf(__shfl_sync(gmask<K>(), p, y, K), Pi[y * K + x], o);
-    const float v = o * lx;
+    const float v = row_dot<K>(col, p, buf) * lx;
     const float c = group_sum<K>(v);
     bad |= !(c > 0.f);
     p = v / c;
@@ -325,45 +292,13 @@ KS_DEV void advance_step(float& p, float& L, float& comp, const float* __restric
     L = Ln;
 }
 
-// Row z of the step's Definition 2 element from its filtered marginal
-// (lane x: p(x)): a(x | z) = p(x) Pi[x][z] / sum_x' p(x') Pi[x'][z].
+// beta(z) of an element with log weights lg followed by v(z) = (f beta')(z):
+// exp(lg - max) v, rescaled by a power of two to a maximum in [1, 2).
 template <int K>
-KS_DEV void selem_row(float (&a)[K], float p, const float* __restrict__ PiT, Flags& bad) {
-    const int z = glane<K>();
-    float d = 0.f;
-#pragma unroll
-    for (int x = 0; x < K; ++x) {
-        a[x] = __shfl_sync(gmask<K>(), p, x, K) * PiT[z * Dims<K>::PT + x];
-        d += a[x];
-    }
-    bad |= !(d > 0.f);
-    const float rd = 1.f / d;
-#pragma unroll
-    for (int x = 0; x < K; ++x) a[x] *= rd;
-}
-
-template <int K>
-KS_DEV void selem_last_row(float (&a)[K], float p) {
-#pragma unroll
-    for (int x = 0; x < K; ++x) a[x] = __shfl_sync(gmask<K>(), p, x, K);
-}
-
-// Smoothing state (lane x: s(x)) advanced through the step's element built
-// from p (lane x: p(x)):  s'(x) = p(x) sum_z (s(z) / d(z)) Pi[x][z],
-// d(z) = sum_x p(x) Pi[x][z]; rescaled to sum 1.
-template <int K>
-KS_DEV void sadvance_step(float& s, float p, const float* __restrict__ PiT, Flags& bad) {
-    const int lane = glane<K>();
-    float d = 0.f;   // lane z: d(z)
-#pragma unroll
-    for (int x = 0; x < K; ++x) d = fmaf(__shfl_sync(gmask<K>(), p, x, K), PiT[lane * Dims<K>::PT + x], d);
-    bad |= !(d > 0.f);
-    const float v = s / d;
-    float o = 0.f;   // lane x
-#pragma unroll
-    for (int z = 0; z < K; ++z) o = fmaf(__shfl_sync(gmask<K>(), v, z, K), PiT[z * Dims<K>::PT + lane], o);
-    const float sn = p * o;
-    s = sn / group_sum<K>(sn);
+KS_DEV float beta_of(float v, float lg) {
+    v *= __expf(lg - group_max<K>(lg));
+    int e;
+    return v * pow2_of(group_max<K>(v), e);
 }
 
 // ---------------------------------------------------------------- kernels
@@ -371,9 +306,8 @@ struct Bufs {
     float* fexcl;     // [nchains][FREC] exclusive in-tile prefixes of the forward scan
     float* fspine0;   // [ntiles][FREC]
     float* fspine1;
-    float* schain;    // [nchains][SREC] chain smoothing aggregates (forward apply)
-    float* sexcl;     // [nchains][SREC]
-    float* sspine0;   // [ntiles][SREC]
+    float* chain;     // [nchains][FREC] chain elements, for the reverse scan (null: not wanted)
+    float* sspine0;   // [ntiles][FREC] tile aggregates again, for the reversed spine
     float* sspine1;
 };
 
@@ -382,9 +316,8 @@ template <int K, int NW>
 struct alignas(16) Smem {
     static constexpr int NG = NW * 32 / K;
     float Pi[K * K];
-    float PiT[K * Dims<K>::PT];
     float q1[K];
-    float pad[(4 - (K * Dims<K>::PT + K) % 4) % 4];
+    int top[(NG + 3) / 4 * 4];
     float slot[NG][Dims<K>::SLOT];   // one element per chain (pitch Q rows + lg)
 };
 
@@ -394,7 +327,7 @@ __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* 
                                                                 uint32_t* status) {
     __shared__ Smem<K, NW> sm;
     constexpr int NG = Smem<K, NW>::NG;
-    load_pi(cg, sm.Pi, sm.PiT, sm.q1);
+    load_pi(cg, sm.Pi, sm.q1);
     __syncthreads();
     const int w = threadIdx.x / K;
     const int64_t nch = (T + CH - 1) / CH;
@@ -406,62 +339,70 @@ __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* 
         const int64_t k0 = c * CH, k1 = (k0 + CH < T) ? k0 + CH : T;
         FRow<K> r;
         float l[K];
-        float lm = lik_row(lik, k0, l, bad);
-        if (k0 == 0) first_row(r, sm.q1, l, lm, bad);
-        else step_row(r, sm.Pi, l, lm, bad);
+        int ex = lik_row2(lik, k0, l, bad);
+        const float* first = k0 == 0 ? sm.q1 : sm.Pi + glane<K>() * K;   // k = 1: every row p(x_1, y_1)
+#pragma unroll
+        for (int x = 0; x < K; ++x) r.f[x] = first[x] * l[x];
 #pragma unroll 1
         for (int64_t k = k0 + 1; k < k1; ++k) {
-            lm = lik_row(lik, k, l, bad);
-            fold_row(r, sm.Pi, l, lm, bad);
+            const int le = lik_row2(lik, k, l, bad);
+            fold_row(r, ex, sm.Pi, l, le, bad);
         }
+        // log g relative to the chain's largest exponent, which is kept beside it
+        const int top = group_max_i<K>(ex);
+        fold_end(r, ex - top, bad);
         put_frow(sm.slot[w], r);
+        if (glane<K>() == 0) sm.top[w] = top;
+        if (b.chain != nullptr) store_frow(b.chain + c * Dims<K>::FREC, r);
     }
     __syncthreads();
     if (w == 0) {   // in-tile combine, chain order
         FRow<K> acc;
         smem_row<Dims<K>::Q>(sm.slot[0], glane<K>(), acc.f);
         acc.lg = sm.slot[0][K * Dims<K>::Q + glane<K>()];
+        int top = sm.top[0];
+        auto absolute = [&](float* dst) {   // log g itself, for the prefixes
+            FRow<K> q = acc;
+            q.lg = fmaf((float)top, 0.693147180559945f, q.lg);
+            store_frow(dst, q);
+        };
 #pragma unroll 1
         for (int t = 1; t < nvalid; ++t) {
-            store_frow(b.fexcl + ((int64_t)blockIdx.x * NG + t) * Dims<K>::FREC, acc);
+            absolute(b.fexcl + ((int64_t)blockIdx.x * NG + t) * Dims<K>::FREC);
             combine_row(acc, sm.slot[t], bad);
+            top += sm.top[t];
         }
-        store_frow(b.fspine0 + (int64_t)blockIdx.x * Dims<K>::FREC, acc);
+        absolute(b.fspine0 + (int64_t)blockIdx.x * Dims<K>::FREC);
+        if (b.chain != nullptr) {
+            relative_lg<K>(acc);
+            store_frow(b.sspine0 + (int64_t)blockIdx.x * Dims<K>::FREC, acc);
+        }
     }
     report_flags(status, bad, kFull, (threadIdx.x & 31) == 0);
 }
 
-// Kogge-Stone level s over tile aggregates: dst[t] = src[t - s] (x) src[t].
-// FILTER: Definition 1 records; else smoothing records in scan (reversed
-// time) order, combined as the matrix product src[t - s] src[t].
-template <bool FILTER, int K, int NW>
+// Kogge-Stone level s over tile aggregates: dst[t] = src[t - s] (x) src[t]
+// (prefixes), or src[t] (x) src[t + s] (suffixes).
+template <bool PREFIX, int K, int NW>
 __global__ void __launch_bounds__(NW * 32) spine_kernel(const float* __restrict__ src, float* __restrict__ dst,
                                                         int ntiles, int s, uint32_t* status) {
     constexpr int NG = NW * 32 / K;
     __shared__ __align__(16) float slot[NG][Dims<K>::SLOT];
-    constexpr int REC = FILTER ? Dims<K>::FREC : Dims<K>::SREC;
+    constexpr int REC = Dims<K>::FREC;
     const int w = threadIdx.x / K;
     const int t = blockIdx.x * NG + w;
     Flags bad = 0u;
     if (t < ntiles) {
-        if (t >= s) {
-            if constexpr (FILTER) {
-                FRow<K> r;
-                load_frow(src + (int64_t)t * REC, r);
-                put_frow(slot[w], r);
-                __syncwarp(gmask<K>());
-                load_frow(src + (int64_t)(t - s) * REC, r);
-                combine_row(r, slot[w], bad);
-                store_frow(dst + (int64_t)t * REC, r);
-            } else {
-                float a[K];
-                load_srow(src + (int64_t)t * REC, a);
-                put_srow(slot[w], a);
-                __syncwarp(gmask<K>());
-                load_srow(src + (int64_t)(t - s) * REC, a);
-                matmul_row(a, slot[w]);
-                store_srow(dst + (int64_t)t * REC, a);
-            }
+        const int left = PREFIX ? t - s : t, right = PREFIX ? t : t + s;
+        if (left >= 0 && right < ntiles) {
+            FRow<K> r;
+            load_frow(src + (int64_t)right * REC, r);
+            put_frow(slot[w], r);
+            __syncwarp(gmask<K>());
+            load_frow(src + (int64_t)left * REC, r);
+            combine_row(r, slot[w], bad);
+            if constexpr (!PREFIX) relative_lg<K>(r);
+            store_frow(dst + (int64_t)t * REC, r);
         } else {
             const float4* p = reinterpret_cast<const float4*>(src + (int64_t)t * REC);
             float4* q = reinterpret_cast<float4*>(dst + (int64_t)t * REC);
@@ -471,8 +412,8 @@ __global__ void __launch_bounds__(NW * 32) spine_kernel(const float* __restrict_
     report_flags(status, bad, kFull, (threadIdx.x & 31) == 0);
 }
 
-// Forward apply: filt [T][K], loglik [T] (may be null), chain smoothing
-// aggregates; `pre` holds the inclusive tile prefixes from the spine.
+// Forward apply: filt [T][K], loglik [T] (may be null); `pre` holds the
+// inclusive tile prefixes from the spine.
 template <int K, int NW, int CH>
 __global__ void __launch_bounds__(NW * 32) filter_apply_kernel(const Const<K>* __restrict__ cg,
                                                                const float* __restrict__ lik, int64_t T,
@@ -481,7 +422,7 @@ __global__ void __launch_bounds__(NW * 32) filter_apply_kernel(const Const<K>* _
                                                                uint32_t* status) {
     __shared__ Smem<K, NW> sm;
     constexpr int NG = Smem<K, NW>::NG;
-    load_pi(cg, sm.Pi, sm.PiT, sm.q1);
+    load_pi(cg, sm.Pi, sm.q1);
     __syncthreads();
     const int w = threadIdx.x / K, lane = glane<K>();
     const int64_t nch = (T + CH - 1) / CH;
@@ -510,16 +451,19 @@ __global__ void __launch_bounds__(NW * 32) filter_apply_kernel(const Const<K>* _
             row0_state(r, p, L);
         }
         float comp = 0.f;
-        float a[K];   // this lane's row of the chain's smoothing aggregate
-        float* sacc = sm.slot[w];
-        __syncwarp(gmask<K>());
+        float col[K];   // this lane's column of Pi
+#pragma unroll
+        for (int y = 0; y < K; ++y) col[y] = sm.Pi[y * K + lane];
+        float* buf = sm.slot[w];
+        float ln = __ldg(lik + k0 * K + lane);
 #pragma unroll 1
         for (int64_t k = k0; k < k1; ++k) {
-            float l[K];
-            const float lm = lik_row(lik, k, l, bad);
-            float lx = 0.f;
-#pragma unroll
-            for (int x = 0; x < K; ++x) lx = (lane == x) ? l[x] : lx;
+            float lx = ln;
+            if (k + 1 < k1) ln = __ldg(lik + (k + 1) * K + lane);
+            const float m = group_max<K>(lx);
+            bad |= !(m > 0.f) || !(m <= 3.0e38f) || !(lx <= 3.0e38f);
+            lx *= 1.f / m;
+            const float lm = __logf(m);
             if (!has) {   // step 1
                 float v = sm.q1[lane] * lx;
                 const float s = group_sum<K>(v);
@@ -528,104 +472,68 @@ __global__ void __launch_bounds__(NW * 32) filter_apply_kernel(const Const<K>* _
                 L = lm + __logf(s);
                 has = true;
             } else {
-                advance_step<K>(p, L, comp, sm.Pi, lx, lm, bad);
+                advance_step<K>(p, L, comp, col, lx, lm, buf, bad);
             }
             filt[k * K + lane] = p;
             if (loglik && lane == 0) loglik[k] = L;
-            float e[K];
-            if (k == T - 1) selem_last_row(e, p);
-            else selem_row(e, p, sm.PiT, bad);
-            if (k == k0) {
-#pragma unroll
-                for (int x = 0; x < K; ++x) a[x] = e[x];
-            } else {       // a_k0 (x) ... (x) a_k = a_k ... a_k0: row z of e times the aggregate
-                put_srow(sacc, a);
-                __syncwarp(gmask<K>());
-                matmul_row(e, sacc);
-                __syncwarp(gmask<K>());
-#pragma unroll
-                for (int x = 0; x < K; ++x) a[x] = e[x];
-            }
         }
-        store_srow(b.schain + c * Dims<K>::SREC, a);
         bad |= !isfinite(p) || !isfinite(L);
     }
     report_flags(status, bad, kFull, (threadIdx.x & 31) == 0);
 }
 
-// Reverse reduce: scan position j = tile * NG + w covers chain nch - 1 - j.
-template <int K, int NW>
-__global__ void __launch_bounds__(NW * 32) smoother_reduce_kernel(int64_t nch, Bufs b, uint32_t* status) {
-    constexpr int NG = NW * 32 / K;
-    __shared__ __align__(16) float slot[NG][Dims<K>::SLOT];
-    const int w = threadIdx.x / K;
-    const int64_t j0 = (int64_t)blockIdx.x * NG;
-    const int nvalid = (nch - j0 < NG) ? (int)(nch - j0) : NG;
-    if (w < nvalid) {
-        float a[K];
-        load_srow(b.schain + (nch - 1 - (j0 + w)) * Dims<K>::SREC, a);
-        put_srow(slot[w], a);
-    }
-    __syncthreads();
-    if (w == 0) {
-        float acc[K];
-        smem_row<Dims<K>::Q>(slot[0], glane<K>(), acc);
-#pragma unroll 1
-        for (int t = 1; t < nvalid; ++t) {
-            store_srow(b.sexcl + (j0 + t) * Dims<K>::SREC, acc);
-            matmul_row(acc, slot[t]);   // scan order: (later in time) (x)_r (earlier) = acc . chain
-        }
-        store_srow(b.sspine0 + (int64_t)blockIdx.x * Dims<K>::SREC, acc);
-    }
-    (void)status;
-}
-
-// Reverse apply: smooth [T][K]; `pre` holds the inclusive tile suffixes.
+// Reverse apply: smooth [T][K] = filt . beta / sum; `suf` holds the inclusive
+// tile suffixes (rows of sum one, so that beta before a tile is its g).
 template <int K, int NW, int CH>
 __global__ void __launch_bounds__(NW * 32) smoother_apply_kernel(const Const<K>* __restrict__ cg,
+                                                                 const float* __restrict__ lik,
                                                                  const float* __restrict__ filt, int64_t T,
                                                                  float* __restrict__ smooth, Bufs b,
-                                                                 const float* __restrict__ pre, uint32_t* status) {
-    __shared__ Smem<K, NW> sm;
-    constexpr int NG = Smem<K, NW>::NG;
-    load_pi(cg, sm.Pi, sm.PiT, sm.q1);
-    __syncthreads();
+                                                                 const float* __restrict__ suf, int ntiles,
+                                                                 uint32_t* status) {
+    constexpr int NG = NW * 32 / K;
+    __shared__ __align__(16) float vec[NG][K];
     const int w = threadIdx.x / K, lane = glane<K>();
     const int64_t nch = (T + CH - 1) / CH;
-    const int64_t j = (int64_t)blockIdx.x * NG + w;   // scan position
+    const int64_t c = (int64_t)blockIdx.x * NG + w;
     Flags bad = 0u;
-    if (j < nch) {
-        const int64_t c = nch - 1 - j;
+    if (c < nch) {
         const int64_t k0 = c * CH, k1 = (k0 + CH < T) ? k0 + CH : T;
-        const bool has_tile = blockIdx.x > 0, has_in = w > 0;
-        float s = 0.f;
-        bool has = has_tile || has_in;
-        if (has) {
-            float a[K];
-            if (has_tile) {
-                load_srow(pre + ((int64_t)blockIdx.x - 1) * Dims<K>::SREC, a);
-                if (has_in) {
-                    float e[K];
-                    load_srow(b.sexcl + j * Dims<K>::SREC, e);
-                    put_srow(sm.slot[w], e);
-                    __syncwarp(gmask<K>());
-                    matmul_row(a, sm.slot[w]);
-                }
-            } else {
-                load_srow(b.sexcl + j * Dims<K>::SREC, a);
-            }
-            s = row0_vec(a);
+        float be = 1.f;   // lane z: beta(z) after the chain
+        float* buf = vec[w];
+        if ((int)blockIdx.x + 1 < ntiles) {
+            const float lg = __ldcg(suf + ((int64_t)blockIdx.x + 1) * Dims<K>::FREC + K * K + lane);
+            be = beta_of<K>(1.f, lg);
         }
+        const int64_t ctop = min(nch, ((int64_t)blockIdx.x + 1) * NG);
+#pragma unroll 1
+        for (int64_t j = ctop - 1; j > c; --j) {   // the tile's later chains
+            FRow<K> r;
+            load_frow(b.chain + j * Dims<K>::FREC, r);
+            be = beta_of<K>(row_dot<K>(r.f, be, buf), r.lg);
+        }
+        float row[K];   // this lane's row of Pi
+#pragma unroll
+        for (int x = 0; x < K; ++x) row[x] = __ldg(cg->Pi + lane * K + x);
+        constexpr float kUp = 1.152921504606847e18f;   // 2^60: see hmm::smoothed
+        float pn = __ldg(filt + (k1 - 1) * K + lane), ln = __ldg(lik + (k1 - 1) * K + lane);
+        float s = 0.f;
 #pragma unroll 1
         for (int64_t k = k1 - 1; k >= k0; --k) {
-            const float p = __ldg(filt + k * K + lane);
-            if (!has) {   // k = T - 1: the smoothed marginal is the filtered one
-                s = p;
-                has = true;
-            } else {
-                sadvance_step<K>(s, p, sm.PiT, bad);
+            const float p = pn, lx = ln;
+            if (k > k0) {
+                pn = __ldg(filt + (k - 1) * K + lane);
+                ln = __ldg(lik + (k - 1) * K + lane);
             }
+            s = (p * kUp) * (be * kUp);
+            const float t = group_sum<K>(s), m = group_max<K>(lx);
+            bad |= !(t > 0.f) || !(m > 0.f);
+            s = s / t;
             smooth[k * K + lane] = s;
+            // beta_{k-1} = Pi (l_k . beta_k), both factors rescaled by powers of two
+            int e;
+            const float v = row_dot<K>(row, lx * pow2_of(m, e) * be, buf);
+            be = v * pow2_of(group_max<K>(v), e);
         }
         bad |= !isfinite(s);
     }
