@@ -161,12 +161,11 @@ def _check(rc: int, what: str):
 
 
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    return torch.cuda.current_stream().cuda_stream if stream is None else stream.cuda_stream
 
 
 def _dev(x, dtype, device):
@@ -230,9 +229,10 @@ class Model:
                                  f"got {tuple(t.shape)}")
 
     def struct(self) -> _KsModel:
-        return _KsModel(self.nx, self.ny, int(self.time_varying), 0, self.F.data_ptr(),
-                        0 if self.u is None else self.u.data_ptr(), self.Q.data_ptr(),
-                        self.H.data_ptr(), 0 if self.d is None else self.d.data_ptr(),
+        F, u, H, d = self.F, self.u, self.H, self.d
+        return _KsModel(F.shape[-1], H.shape[-2], int(F.dim() == 3), 0, F.data_ptr(),
+                        0 if u is None else u.data_ptr(), self.Q.data_ptr(),
+                        H.data_ptr(), 0 if d is None else d.data_ptr(),
                         self.R.data_ptr(), self.m0.data_ptr(), self.P0.data_ptr())
 
 
@@ -258,9 +258,7 @@ def alloc_workspace(model: Model, T: int, purpose: int = KS_WS_SMOOTH, stream=No
 
 
 def _out(shape, like, out):
-    if out is not None:
-        return out
-    return torch.empty(shape, dtype=torch.float32, device=like.device)
+    return like.new_empty(shape, dtype=torch.float32) if out is None else out
 
 
 def smooth(model: Model, y: torch.Tensor, ws: torch.Tensor | None = None, *, fmean=None, fcov=None,
@@ -274,24 +272,25 @@ def smooth(model: Model, y: torch.Tensor, ws: torch.Tensor | None = None, *, fme
     returned for the smoothed moments.  ``events``: 4 recorded-or-fresh
     torch.cuda.Event objects to time the kernels (``ks_smooth_traced``).
     """
-    T = int(y.shape[0])
+    T = y.shape[0]
     model.check_steps(T)
     if filter_only and not keep_filtered:
         raise ValueError("filter_only needs keep_filtered")
-    purpose = KS_WS_SMOOTH if keep_filtered else KS_WS_ELEMENTS
-    ws = alloc_workspace(model, T, purpose, stream) if ws is None else ws
+    if ws is None:
+        ws = alloc_workspace(model, T, KS_WS_SMOOTH if keep_filtered else KS_WS_ELEMENTS, stream)
+    m = model.struct()
+    n = m.nx
     if keep_filtered:
-        fmean = _out((T, model.nx), y, fmean)
-        fcov = _out((T, model.nx, model.nx), y, fcov)
+        fmean = _out((T, n), y, fmean)
+        fcov = _out((T, n, n), y, fcov)
     else:
         fmean = fcov = None
     if filter_only:
         smean = scov = None
     else:
-        smean = _out((T, model.nx), y, smean)
-        scov = _out((T, model.nx, model.nx), y, scov)
-    m = model.struct()
-    args = (ctypes.byref(m), _p(y), T, _p(ws), ws.numel(), _p(fmean), _p(fcov), _p(smean), _p(scov),
+        smean = _out((T, n), y, smean)
+        scov = _out((T, n, n), y, scov)
+    args = (ctypes.byref(m), y.data_ptr(), T, ws.data_ptr(), ws.numel(), _p(fmean), _p(fcov), _p(smean), _p(scov),
             _stream(stream))
     if events is None:
         _check(lib().ks_smooth(*args), "ks_smooth")

@@ -114,12 +114,13 @@ int run(const ks_hmm* h, const float* lik, int64_t T, void* ws, size_t ws_bytes,
     return HImpl<K, 32>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev);
 }
 
-// K = 16, 32: one K-lane group per chain of CH steps, NG chains per tile
+// K = 8, 16, 32: one K-lane group per chain of CH steps, NG chains per tile
 // (ks_hmmw.cuh).
-template <int K>
+template <int K, int CH>
 struct WImpl {
-    static constexpr int NW = 4, CH = 64, NWS = 4;
-    static constexpr int NG = NW * 32 / K;
+    static constexpr int NW = 4, NWS = 4, R = K == 8 ? 1 : 2;   // R: chains a group folds together
+    static constexpr int NG = NW * 32 / K * R;                  // chains of a tile (one block of the reduce)
+    static constexpr int NA = NW * 32 / K;                      // chains of a block of the applies
     struct WLayout {
         int64_t nch = 0;
         int ntiles = 0;
@@ -156,7 +157,7 @@ struct WImpl {
         const WLayout L = layout(T);
         const int sgrid_tiles = NWS * 32 / K;   // tiles per spine block
         if (!ws || (reinterpret_cast<uintptr_t>(ws) & 255u) != 0 || ws_bytes < L.bytes) return KS_EINVAL;
-        if (!aligned16(lik)) return KS_EINVAL;   // likelihood rows are read as float4
+        if (K >= 16 && !aligned16(lik)) return KS_EINVAL;   // as documented for these sizes
         char* b = static_cast<char*>(ws);
         uint32_t* stat = static_cast<uint32_t*>(ws);
         hmmw::Const<K>* cg = reinterpret_cast<hmmw::Const<K>*>(b + L.off_const);
@@ -177,37 +178,50 @@ struct WImpl {
         hmmw::prep_kernel<K><<<1, 64, 0, st>>>(h->pi, h->Pi, cg, stat);
         if ((rc = launch_status())) return rc;
         if ((rc = rec(1))) return rc;
-        filter_reduce_kernel<K, NW, CH><<<L.ntiles, NW * 32, 0, st>>>(cg, lik, T, bf, stat);
-        if ((rc = launch_status())) return rc;
-        const float* src = bf.fspine0;
-        float* dst = bf.fspine1;
+        rc = launch_pdl(filter_reduce_kernel<K, NW, CH, R>, L.ntiles, NW * 32, 0, st, cg, lik, T, bf, stat);
+        if (rc) return rc;
+        const float *src = bf.fspine0, *ssrc = bf.sspine0;
+        float *dst = bf.fspine1, *sdst = bf.sspine1;
         for (int s = 1; s < L.ntiles; s <<= 1) {
-            spine_kernel<true, K, NWS><<<sgrid, NWS * 32, 0, st>>>(src, dst, L.ntiles, s, stat);
-            if ((rc = launch_status())) return rc;
-            float* t = const_cast<float*>(src);
+            if ((rc = launch_pdl2(spine_kernel<K, NWS>, dim3(sgrid, smooth ? 2 : 1), NWS * 32, 0, st, src, dst, ssrc,
+                                  sdst, L.ntiles, s, stat)))
+                return rc;
+            float *t = const_cast<float*>(src), *u = const_cast<float*>(ssrc);
             src = dst;
+            ssrc = sdst;
             dst = t;
+            sdst = u;
         }
-        filter_apply_kernel<K, NW, CH><<<L.ntiles, NW * 32, 0, st>>>(cg, lik, T, filt, loglik, bf, src, stat);
-        if ((rc = launch_status())) return rc;
+        const int nap = (int)((L.nch + NA - 1) / NA);
+        rc = launch_pdl(filter_apply_kernel<K, NW, CH, NG>, nap, NW * 32, 0, st, cg, lik, T, filt, loglik, bf, src,
+                        stat);
+        if (rc) return rc;
         if ((rc = rec(2))) return rc;
         if (smooth) {
-            const float* ssrc = bf.sspine0;
-            float* sdst = bf.sspine1;
-            for (int s = 1; s < L.ntiles; s <<= 1) {
-                spine_kernel<false, K, NWS><<<sgrid, NWS * 32, 0, st>>>(ssrc, sdst, L.ntiles, s, stat);
-                if ((rc = launch_status())) return rc;
-                float* t = const_cast<float*>(ssrc);
-                ssrc = sdst;
-                sdst = t;
-            }
-            smoother_apply_kernel<K, NW, CH><<<L.ntiles, NW * 32, 0, st>>>(cg, lik, filt, T, smooth, bf, ssrc, L.ntiles,
-                                                                           stat);
-            if ((rc = launch_status())) return rc;
+            rc = launch_pdl(smoother_apply_kernel<K, NW, CH, NG>, nap, NW * 32, 0, st, cg, lik, filt, T, smooth, bf,
+                            ssrc, L.ntiles, stat);
+            if (rc) return rc;
         }
         return rec(3);
     }
 };
+
+// Chains of 32 steps for shorter sequences (more of them than lane groups the
+// chip can hold only from there on), else of `LONG` steps: fewer tiles for the
+// spine's levels.
+template <int K, int LONG>
+struct WSize {
+    static constexpr int64_t kLong = 128 * 1024;
+    static size_t bytes(int64_t T) { return std::max(WImpl<K, 32>::layout(T).bytes, WImpl<K, LONG>::layout(T).bytes); }
+    static int smooth(const ks_hmm* h, const float* lik, int64_t T, void* ws, size_t ws_bytes, float* filt,
+                      float* smooth, float* loglik, cudaStream_t st, void* const* ev) {
+        return T < kLong ? WImpl<K, 32>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev)
+                         : WImpl<K, LONG>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev);
+    }
+};
+using W8 = WSize<8, 128>;
+using W16 = WSize<16, 64>;
+using W32 = WSize<32, 64>;
 
 }  // namespace
 }  // namespace hmm
@@ -224,9 +238,9 @@ size_t ks_hmm_workspace_bytes(int K, int64_t T) {
     switch (K) {
         case 2: return hmm::bytes<2>(T);
         case 4: return hmm::bytes<4>(T);
-        case 8: return hmm::bytes<8>(T);
-        case 16: return hmm::WImpl<16>::layout(T).bytes;
-        case 32: return hmm::WImpl<32>::layout(T).bytes;
+        case 8: return hmm::W8::bytes(T);
+        case 16: return hmm::W16::bytes(T);
+        case 32: return hmm::W32::bytes(T);
         default: return 0;
     }
 }
@@ -240,9 +254,9 @@ int ks_hmm_smooth_traced(const ks_hmm* h, const float* lik, int64_t T, void* ws,
     switch (h->K) {
         case 2: return hmm::run<2>(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, events);
         case 4: return hmm::run<4>(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, events);
-        case 8: return hmm::run<8>(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, events);
-        case 16: return hmm::WImpl<16>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, events);
-        default: return hmm::WImpl<32>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, events);
+        case 8: return hmm::W8::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, events);
+        case 16: return hmm::W16::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, events);
+        default: return hmm::W32::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, events);
     }
 }
 

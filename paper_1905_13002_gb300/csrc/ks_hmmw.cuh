@@ -1,4 +1,4 @@
-// ks_hmmw.cuh -- the discrete-state (HMM) filter and smoother for K = 16 and
+// ks_hmmw.cuh -- the discrete-state (HMM) filter and smoother for K = 8, 16 and
 // 32 states: one K-lane group of a warp per chain of steps, lane z holding
 // row z of each K x K element (Section III's Definitions 1 and 2 with sums,
 // as in ks_hmm.cuh).
@@ -39,13 +39,9 @@ struct Dims {
     static constexpr int FREC = K * K + K;       // global filtering record: rows, then log g
 };
 
-// A chain is K lanes of one warp (lane z = row z); 32 / K chains per warp.
-template <int K>
-KS_DEV unsigned gmask() {
-    if constexpr (K == 32) return 0xffffffffu;
-    else return ((1u << K) - 1u) << (threadIdx.x & (32 - K));
-}
-
+// A chain is K lanes of one warp (lane z = row z); 32 / K chains per warp.  The
+// chains of a warp step together (a shorter or absent one repeats its last step
+// with the results dropped), so that every exchange is among all lanes.
 template <int K>
 KS_DEV int glane() { return threadIdx.x & (K - 1); }
 
@@ -65,21 +61,21 @@ struct FRow {
 template <int K>
 KS_DEV float group_sum(float v) {
 #pragma unroll
-    for (int o = K / 2; o > 0; o >>= 1) v += __shfl_xor_sync(gmask<K>(), v, o, K);
+    for (int o = K / 2; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o, K);
     return v;
 }
 
 template <int K>
 KS_DEV float group_max(float v) {
 #pragma unroll
-    for (int o = K / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(gmask<K>(), v, o, K));
+    for (int o = K / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(kFull, v, o, K));
     return v;
 }
 
 template <int K>
 KS_DEV int group_max_i(int v) {
 #pragma unroll
-    for (int o = K / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(gmask<K>(), v, o, K));
+    for (int o = K / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(kFull, v, o, K));
     return v;
 }
 
@@ -153,57 +149,80 @@ KS_DEV float pow2_of(float r, int& e) {
     return __uint_as_float((uint32_t)(127 - e) << 23);
 }
 
-// Likelihood row of step k (the same for every lane) scaled by a power of two
-// to a maximum in [1, 2); returns the exponent taken out.
-template <int K>
-KS_DEV int lik_row2(const float* __restrict__ lik, int64_t k, float (&l)[K], Flags& bad) {
-    const float4* p = reinterpret_cast<const float4*>(lik + k * K);
-    float m = 0.f;
-#pragma unroll
-    for (int i = 0; i < K / 4; ++i) {
-        const float4 q = __ldg(p + i);
-        l[4 * i] = q.x;
-        l[4 * i + 1] = q.y;
-        l[4 * i + 2] = q.z;
-        l[4 * i + 3] = q.w;
-    }
-#pragma unroll
-    for (int x = 0; x < K; ++x) m = fmaxf(m, l[x]);
-    const bool ok = m > 0.f && m <= 3.0e38f;
-    bad |= !ok;
-    int e;
-    const float s = pow2_of(ok ? m : 1.f, e);
-#pragma unroll
-    for (int x = 0; x < K; ++x) l[x] *= s;
-    return e;
+// Two FP32 multiply-adds in one instruction (each rounded as fmaf).
+KS_DEV void ffma2(uint64_t& d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
+KS_DEV uint64_t dup2(float v) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+    return r;
+}
+KS_DEV void unpack2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
 
-// Fold of a step element into row z: (f Pi)[z] . l, kept at a sum in [1, 2) by
-// a power of two (exponents added up in ex: no division, no logarithm).
-template <int K>
-KS_DEV void fold_row(FRow<K>& r, int& ex, const float* __restrict__ Pi, const float (&l)[K], int le, Flags& bad) {
-    float o[K];
+// o[r][x] = sum_y f[r][y] M[y][x] for a shared-memory M whose rows (pitch PITCH
+// floats) all lanes of the chain read together: pairs of columns in packed
+// multiply-adds (half the instructions of the scalar form), each loaded row
+// used for R rows (the loads bound the K = 32 fold with R = 1).
+template <int PITCH, int K, int R>
+KS_DEV void rows_times(const float* const (&f)[R], const float* __restrict__ M, uint64_t (&acc)[R][K / 2]) {
 #pragma unroll
-    for (int x = 0; x < K; ++x) o[x] = 0.f;
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i) acc[r][i] = 0ull;
 #pragma unroll
     for (int y = 0; y < K; ++y) {
-        float pr[K];
-        smem_row<K>(Pi, y, pr);
+        const ulonglong2* p = reinterpret_cast<const ulonglong2*>(M + y * PITCH);
+        uint64_t fy[R];
 #pragma unroll
-        for (int x = 0; x < K; ++x) o[x] = fmaf(r.f[y], pr[x], o[x]);
+        for (int r = 0; r < R; ++r) fy[r] = dup2(f[r][y]);
+#pragma unroll
+        for (int i = 0; i < K / 4; ++i) {
+            const ulonglong2 q = p[i];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                ffma2(acc[r][2 * i], fy[r], q.x);
+                ffma2(acc[r][2 * i + 1], fy[r], q.y);
+            }
+        }
     }
-    float s = 0.f;
+}
+
+// Fold of a step element into row z of R chains: (f Pi)[z] . l, kept at a sum in
+// [1, 2) by a power of two (exponents added up in ex: no division, no
+// logarithm).  l[r]: the chain's scaled likelihood row in shared memory, le its
+// exponent; on[r] false: nothing happens to chain r.
+template <int K, int R>
+KS_DEV void fold_rows(FRow<K> (&fr)[R], int (&ex)[R], const float* __restrict__ Pi, const float* const (&l)[R],
+                      const int (&le)[R], const bool (&on)[R], Flags& bad) {
+    uint64_t acc[R][K / 2];
+    const float* f[R];
 #pragma unroll
-    for (int x = 0; x < K; ++x) {
-        o[x] *= l[x];
-        s += o[x];
+    for (int r = 0; r < R; ++r) f[r] = fr[r].f;
+    rows_times<K, K, R>(f, Pi, acc);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        float o[K], s = 0.f;
+#pragma unroll
+        for (int i = 0; i < K / 2; ++i) unpack2(acc[r][i], o[2 * i], o[2 * i + 1]);
+#pragma unroll
+        for (int x = 0; x < K; x += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(l[r] + x);
+            o[x] *= q.x;
+            o[x + 1] *= q.y;
+            o[x + 2] *= q.z;
+            o[x + 3] *= q.w;
+            s += (o[x] + o[x + 1]) + (o[x + 2] + o[x + 3]);
+        }
+        int e;
+        const float rs = pow2_of(s, e);
+        if (on[r]) {
+            bad |= !(s > 0.f);
+#pragma unroll
+            for (int x = 0; x < K; ++x) fr[r].f[x] = o[x] * rs;
+            ex[r] += e + le[r];
+        }
     }
-    bad |= !(s > 0.f);
-    int e;
-    const float rs = pow2_of(s, e);
-#pragma unroll
-    for (int x = 0; x < K; ++x) r.f[x] = o[x] * rs;
-    ex += e + le;
 }
 
 // End of a fold: row of sum one, log g from the exponents and the last sum.
@@ -225,17 +244,18 @@ KS_DEV void combine_row(FRow<K>& r, const float* __restrict__ ej, Flags& bad) {
     float mx = ej[K * Dims<K>::Q];
 #pragma unroll
     for (int y = 1; y < K; ++y) mx = fmaxf(mx, ej[K * Dims<K>::Q + y]);
-    float o[K], d = 0.f;
-#pragma unroll
-    for (int x = 0; x < K; ++x) o[x] = 0.f;
+    float o[K], fw[K], d = 0.f;
 #pragma unroll
     for (int y = 0; y < K; ++y) {
-        const float fw = r.f[y] * __expf(ej[K * Dims<K>::Q + y] - mx);
-        d += fw;
-        float er[K];
-        smem_row<Dims<K>::Q>(ej, y, er);
+        fw[y] = r.f[y] * __expf(ej[K * Dims<K>::Q + y] - mx);
+        d += fw[y];
+    }
+    {
+        uint64_t acc[1][K / 2];
+        const float* const f[1] = {fw};
+        rows_times<Dims<K>::Q, K, 1>(f, ej, acc);
 #pragma unroll
-        for (int x = 0; x < K; ++x) o[x] = fmaf(fw, er[x], o[x]);
+        for (int i = 0; i < K / 2; ++i) unpack2(acc[0][i], o[2 * i], o[2 * i + 1]);
     }
     bad |= !(d > 0.f);
     const float rd = 1.f / d;
@@ -251,10 +271,10 @@ KS_DEV void row0_state(const FRow<K>& r, float& p, float& L) {
     p = 0.f;
 #pragma unroll
     for (int x = 0; x < K; ++x) {
-        const float v = __shfl_sync(gmask<K>(), r.f[x], 0, K);
+        const float v = __shfl_sync(kFull, r.f[x], 0, K);
         if (lane == x) p = v;
     }
-    L = __shfl_sync(gmask<K>(), r.lg, 0, K);
+    L = __shfl_sync(kFull, r.lg, 0, K);
 }
 
 // sum_x m[x] v(x) for a vector with v(x) on lane x, through the group's buffer
@@ -262,9 +282,9 @@ KS_DEV void row0_state(const FRow<K>& r, float& p, float& L) {
 // shuffles.
 template <int K>
 KS_DEV float row_dot(const float (&m)[K], float v, float* __restrict__ buf) {
-    __syncwarp(gmask<K>());
+    __syncwarp(kFull);
     buf[glane<K>()] = v;
-    __syncwarp(gmask<K>());
+    __syncwarp(kFull);
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
     for (int x = 0; x < K; x += 4) {
@@ -275,21 +295,6 @@ KS_DEV float row_dot(const float (&m)[K], float v, float* __restrict__ buf) {
         a3 = fmaf(m[x + 3], t.w, a3);
     }
     return (a0 + a1) + (a2 + a3);
-}
-
-// Filtering state (lane x: p(x)) (x) step: p'(x) = (p Pi)(x) l(x) / c, with the
-// lane's column of Pi in registers.
-template <int K>
-KS_DEV void advance_step(float& p, float& L, float& comp, const float (&col)[K], float lx, float lm, float* buf,
-                         Flags& bad) {
-    const float v = row_dot<K>(col, p, buf) * lx;
-    const float c = group_sum<K>(v);
-    bad |= !(c > 0.f);
-    p = v / c;
-    const float t = (lm + __logf(c)) - comp;   // Kahan-compensated running log-likelihood
-    const float Ln = L + t;
-    comp = (Ln - L) - t;
-    L = Ln;
 }
 
 // beta(z) of an element with log weights lg followed by v(z) = (f beta')(z):
@@ -311,180 +316,281 @@ struct Bufs {
     float* sspine1;
 };
 
-// NG = NW * 32 / K chains per block (one K-lane group each).
-template <int K, int NW>
+constexpr int kAhead = 4;   // steps a chain loads ahead: a step is much shorter than a load from memory
+
+// NG = NW * 32 / K * R chains per block: one K-lane group each R chains in the
+// reduce, one chain in the applies.
+template <int K, int NG>
 struct alignas(16) Smem {
-    static constexpr int NG = NW * 32 / K;
     float Pi[K * K];
     float q1[K];
     int top[(NG + 3) / 4 * 4];
     float slot[NG][Dims<K>::SLOT];   // one element per chain (pitch Q rows + lg)
 };
 
-template <int K, int NW, int CH>
+// One chain's column of a [T][K] array (this lane's state), kAhead steps at a
+// time and a group ahead: step i sits at base + i stride.
+template <int K>
+struct Ahead {
+    const float* base;
+    int n, stride;
+    float next[kAhead];
+    KS_DEV void fetch(int i0) {
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) next[j] = __ldg(base + min(i0 + j, n - 1) * stride);
+    }
+    KS_DEV void init(const float* b, int steps, int st) {
+        base = b;
+        n = steps;
+        stride = st;
+        fetch(0);
+    }
+    KS_DEV void take(int i0, float (&v)[kAhead]) {
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) v[j] = next[j];
+        fetch(i0 + kAhead);
+    }
+};
+
+// Likelihood entries scaled by a power of two to a row maximum in [1, 2); le:
+// the exponents taken out.
+template <int K>
+KS_DEV void scale_rows(float (&lx)[kAhead], int (&le)[kAhead], Flags& bad) {
+#pragma unroll
+    for (int j = 0; j < kAhead; ++j) {
+        const float m = group_max<K>(lx[j]);
+        const bool ok = m > 0.f && m <= 3.0e38f && lx[j] <= 3.0e38f;
+        bad |= !ok;
+        lx[j] *= pow2_of(ok ? m : 1.f, le[j]);
+    }
+}
+
+template <int K, int NW, int CH, int R>
 __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* __restrict__ cg,
                                                                 const float* __restrict__ lik, int64_t T, Bufs b,
                                                                 uint32_t* status) {
-    __shared__ Smem<K, NW> sm;
-    constexpr int NG = Smem<K, NW>::NG;
+    constexpr int NG = NW * 32 / K * R;
+    __shared__ Smem<K, NG> sm;
+    pdl_trigger();
+    pdl_wait();
     load_pi(cg, sm.Pi, sm.q1);
     __syncthreads();
-    const int w = threadIdx.x / K;
+    const int w = threadIdx.x / K, lane = glane<K>();
     const int64_t nch = (T + CH - 1) / CH;
-    const int64_t c = (int64_t)blockIdx.x * NG + w;
-    const int64_t left = nch - (int64_t)blockIdx.x * NG;
-    const int nvalid = left < NG ? (int)left : NG;
+    const int64_t c0 = (int64_t)blockIdx.x * NG;
+    const int nvalid = nch - c0 < NG ? (int)(nch - c0) : NG;
     Flags bad = 0u;
-    if (w < nvalid) {
-        const int64_t k0 = c * CH, k1 = (k0 + CH < T) ? k0 + CH : T;
-        FRow<K> r;
-        float l[K];
-        int ex = lik_row2(lik, k0, l, bad);
-        const float* first = k0 == 0 ? sm.q1 : sm.Pi + glane<K>() * K;   // k = 1: every row p(x_1, y_1)
+    {
+        FRow<K> fr[R];
+        int ex[R], n[R], nmax = 0;
+        Ahead<K> lk[R];
+        float* buf[R];
+        const float* cbuf[R];
 #pragma unroll
-        for (int x = 0; x < K; ++x) r.f[x] = first[x] * l[x];
-#pragma unroll 1
-        for (int64_t k = k0 + 1; k < k1; ++k) {
-            const int le = lik_row2(lik, k, l, bad);
-            fold_row(r, ex, sm.Pi, l, le, bad);
+        for (int r = 0; r < R; ++r) {
+            const int64_t k0 = min(c0 + w * R + r, nch - 1) * CH;
+            n[r] = (int)((k0 + CH < T ? k0 + CH : T) - k0);
+            nmax = max(nmax, n[r]);
+            lk[r].init(lik + k0 * K + lane, n[r], K);
+            cbuf[r] = buf[r] = sm.slot[w * R + r];   // the chain's scaled likelihood row
+            ex[r] = 0;
         }
-        // log g relative to the chain's largest exponent, which is kept beside it
-        const int top = group_max_i<K>(ex);
-        fold_end(r, ex - top, bad);
-        put_frow(sm.slot[w], r);
-        if (glane<K>() == 0) sm.top[w] = top;
-        if (b.chain != nullptr) store_frow(b.chain + c * Dims<K>::FREC, r);
+        nmax = (int)__reduce_max_sync(kFull, (unsigned)nmax);
+#pragma unroll 1
+        for (int i0 = 0; i0 < nmax; i0 += kAhead) {
+            float lx[R][kAhead];
+            int le[R][kAhead];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                lk[r].take(i0, lx[r]);
+                scale_rows<K>(lx[r], le[r], bad);
+            }
+#pragma unroll
+            for (int j = 0; j < kAhead; ++j) {
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < R; ++r) buf[r][lane] = lx[r][j];
+                __syncwarp();
+                if (i0 + j == 0) {   // the chain's first element; k = 1: every row p(x_1, y_1)
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        const float* first = c0 + w * R + r == 0 ? sm.q1 : sm.Pi + lane * K;
+#pragma unroll
+                        for (int x = 0; x < K; ++x) fr[r].f[x] = first[x] * buf[r][x];
+                        ex[r] = le[r][j];
+                    }
+                } else {
+                    int lej[R];
+                    bool on[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        lej[r] = le[r][j];
+                        on[r] = i0 + j < n[r];
+                    }
+                    fold_rows<K, R>(fr, ex, sm.Pi, cbuf, lej, on, bad);
+                }
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int t = w * R + r;
+            // log g relative to the chain's largest exponent, which is kept beside it
+            const int top = group_max_i<K>(ex[r]);
+            fold_end(fr[r], ex[r] - top, bad);
+            put_frow(sm.slot[t], fr[r]);
+            if (lane == 0) sm.top[t] = top;
+            if (b.chain != nullptr && t < nvalid) store_frow(b.chain + (c0 + t) * Dims<K>::FREC, fr[r]);
+        }
     }
     __syncthreads();
-    if (w == 0) {   // in-tile combine, chain order
+    if (threadIdx.x < 32) {   // in-tile combine, chain order (every chain group of the warp does the same)
         FRow<K> acc;
-        smem_row<Dims<K>::Q>(sm.slot[0], glane<K>(), acc.f);
-        acc.lg = sm.slot[0][K * Dims<K>::Q + glane<K>()];
+        smem_row<Dims<K>::Q>(sm.slot[0], lane, acc.f);
+        acc.lg = sm.slot[0][K * Dims<K>::Q + lane];
         int top = sm.top[0];
+        const bool mine = w == 0;
         auto absolute = [&](float* dst) {   // log g itself, for the prefixes
             FRow<K> q = acc;
             q.lg = fmaf((float)top, 0.693147180559945f, q.lg);
-            store_frow(dst, q);
+            if (mine) store_frow(dst, q);
         };
 #pragma unroll 1
         for (int t = 1; t < nvalid; ++t) {
-            absolute(b.fexcl + ((int64_t)blockIdx.x * NG + t) * Dims<K>::FREC);
+            absolute(b.fexcl + (c0 + t) * Dims<K>::FREC);
             combine_row(acc, sm.slot[t], bad);
             top += sm.top[t];
         }
         absolute(b.fspine0 + (int64_t)blockIdx.x * Dims<K>::FREC);
         if (b.chain != nullptr) {
             relative_lg<K>(acc);
-            store_frow(b.sspine0 + (int64_t)blockIdx.x * Dims<K>::FREC, acc);
+            if (mine) store_frow(b.sspine0 + (int64_t)blockIdx.x * Dims<K>::FREC, acc);
         }
     }
     report_flags(status, bad, kFull, (threadIdx.x & 31) == 0);
 }
 
 // Kogge-Stone level s over tile aggregates: dst[t] = src[t - s] (x) src[t]
-// (prefixes), or src[t] (x) src[t + s] (suffixes).
-template <bool PREFIX, int K, int NW>
-__global__ void __launch_bounds__(NW * 32) spine_kernel(const float* __restrict__ src, float* __restrict__ dst,
+// (prefixes, blockIdx.y = 0), and in the same launch src[t] (x) src[t + s]
+// (suffixes, blockIdx.y = 1).
+template <int K, int NW>
+__global__ void __launch_bounds__(NW * 32) spine_kernel(const float* __restrict__ psrc, float* __restrict__ pdst,
+                                                        const float* __restrict__ ssrc, float* __restrict__ sdst,
                                                         int ntiles, int s, uint32_t* status) {
     constexpr int NG = NW * 32 / K;
     __shared__ __align__(16) float slot[NG][Dims<K>::SLOT];
     constexpr int REC = Dims<K>::FREC;
+    pdl_trigger();
+    pdl_wait();
+    const bool prefix = blockIdx.y == 0;
+    const float* src = prefix ? psrc : ssrc;
+    float* dst = prefix ? pdst : sdst;
     const int w = threadIdx.x / K;
     const int t = blockIdx.x * NG + w;
-    Flags bad = 0u;
-    if (t < ntiles) {
-        const int left = PREFIX ? t - s : t, right = PREFIX ? t : t + s;
-        if (left >= 0 && right < ntiles) {
-            FRow<K> r;
-            load_frow(src + (int64_t)right * REC, r);
-            put_frow(slot[w], r);
-            __syncwarp(gmask<K>());
-            load_frow(src + (int64_t)left * REC, r);
-            combine_row(r, slot[w], bad);
-            if constexpr (!PREFIX) relative_lg<K>(r);
-            store_frow(dst + (int64_t)t * REC, r);
-        } else {
-            const float4* p = reinterpret_cast<const float4*>(src + (int64_t)t * REC);
-            float4* q = reinterpret_cast<float4*>(dst + (int64_t)t * REC);
-            for (int i = glane<K>(); i < REC / 4; i += K) q[i] = __ldcg(p + i);
-        }
+    Flags bad = 0u, none = 0u;
+    const int left = prefix ? t - s : t, right = prefix ? t : t + s;
+    const bool in = t < ntiles, comb = in && left >= 0 && right < ntiles;
+    FRow<K> r;   // every group combines; one without a partner copies instead
+    load_frow(src + (int64_t)(comb ? right : 0) * REC, r);
+    put_frow(slot[w], r);
+    __syncwarp();
+    load_frow(src + (int64_t)(comb ? left : 0) * REC, r);
+    combine_row(r, slot[w], comb ? bad : none);
+    if (!prefix) relative_lg<K>(r);
+    if (comb) {
+        store_frow(dst + (int64_t)t * REC, r);
+    } else if (in) {
+        const float4* p = reinterpret_cast<const float4*>(src + (int64_t)t * REC);
+        float4* q = reinterpret_cast<float4*>(dst + (int64_t)t * REC);
+        for (int i = glane<K>(); i < REC / 4; i += K) q[i] = __ldcg(p + i);
     }
     report_flags(status, bad, kFull, (threadIdx.x & 31) == 0);
 }
 
 // Forward apply: filt [T][K], loglik [T] (may be null); `pre` holds the
 // inclusive tile prefixes from the spine.
-template <int K, int NW, int CH>
+// TC: chains per tile (of the reduce).
+template <int K, int NW, int CH, int TC>
 __global__ void __launch_bounds__(NW * 32) filter_apply_kernel(const Const<K>* __restrict__ cg,
                                                                const float* __restrict__ lik, int64_t T,
                                                                float* __restrict__ filt, float* __restrict__ loglik,
                                                                Bufs b, const float* __restrict__ pre,
                                                                uint32_t* status) {
-    __shared__ Smem<K, NW> sm;
-    constexpr int NG = Smem<K, NW>::NG;
-    load_pi(cg, sm.Pi, sm.q1);
-    __syncthreads();
+    constexpr int NG = NW * 32 / K;
+    __shared__ __align__(16) float slot[NG][Dims<K>::SLOT];
+    pdl_trigger();
+    pdl_wait();
     const int w = threadIdx.x / K, lane = glane<K>();
     const int64_t nch = (T + CH - 1) / CH;
-    const int64_t c = (int64_t)blockIdx.x * NG + w;
-    Flags bad = 0u;
-    if (c < nch) {
-        const int64_t k0 = c * CH, k1 = (k0 + CH < T) ? k0 + CH : T;
-        // incoming prefix: tile prefix (x) the chain's exclusive in-tile prefix
-        const bool has_tile = blockIdx.x > 0, has_in = w > 0;
-        float p = 0.f, L = 0.f;
-        bool has = has_tile || has_in;
-        if (has) {
-            FRow<K> r;
-            if (has_tile) {
-                load_frow(pre + ((int64_t)blockIdx.x - 1) * Dims<K>::FREC, r);
-                if (has_in) {
-                    FRow<K> e;
-                    load_frow(b.fexcl + c * Dims<K>::FREC, e);
-                    put_frow(sm.slot[w], e);
-                    __syncwarp(gmask<K>());
-                    combine_row(r, sm.slot[w], bad);
-                }
-            } else {
-                load_frow(b.fexcl + c * Dims<K>::FREC, r);
-            }
-            row0_state(r, p, L);
-        }
-        float comp = 0.f;
-        float col[K];   // this lane's column of Pi
-#pragma unroll
-        for (int y = 0; y < K; ++y) col[y] = sm.Pi[y * K + lane];
-        float* buf = sm.slot[w];
-        float ln = __ldg(lik + k0 * K + lane);
-#pragma unroll 1
-        for (int64_t k = k0; k < k1; ++k) {
-            float lx = ln;
-            if (k + 1 < k1) ln = __ldg(lik + (k + 1) * K + lane);
-            const float m = group_max<K>(lx);
-            bad |= !(m > 0.f) || !(m <= 3.0e38f) || !(lx <= 3.0e38f);
-            lx *= 1.f / m;
-            const float lm = __logf(m);
-            if (!has) {   // step 1
-                float v = sm.q1[lane] * lx;
-                const float s = group_sum<K>(v);
-                bad |= !(s > 0.f);
-                p = v / s;
-                L = lm + __logf(s);
-                has = true;
-            } else {
-                advance_step<K>(p, L, comp, col, lx, lm, buf, bad);
-            }
-            filt[k * K + lane] = p;
-            if (loglik && lane == 0) loglik[k] = L;
-        }
-        bad |= !isfinite(p) || !isfinite(L);
+    const int64_t cr = (int64_t)blockIdx.x * NG + w, c = min(cr, nch - 1);
+    const bool own = cr < nch;
+    const int64_t k0 = c * CH;
+    const int n = (int)((k0 + CH < T ? k0 + CH : T) - k0);
+    Flags bad = 0u, none = 0u;
+    // incoming prefix: tile prefix (x) the chain's exclusive in-tile prefix (absent: not used)
+    const int64_t tile = c / TC;
+    const bool has_tile = tile > 0, has_in = c % TC > 0;
+    float p, L;
+    {
+        FRow<K> r, e;
+        load_frow(has_tile ? pre + (tile - 1) * Dims<K>::FREC : b.fspine0, r);
+        load_frow(has_in ? b.fexcl + c * Dims<K>::FREC : b.fspine0, e);
+        put_frow(slot[w], e);
+        __syncwarp();
+        FRow<K> both = r;
+        combine_row(both, slot[w], has_tile && has_in ? bad : none);
+        float p1, L1, p2, L2;
+        row0_state(has_tile ? r : e, p1, L1);
+        row0_state(both, p2, L2);
+        p = has_tile && has_in ? p2 : p1;
+        L = has_tile && has_in ? L2 : L1;
     }
-    report_flags(status, bad, kFull, (threadIdx.x & 31) == 0);
+    const bool start = !has_tile && !has_in;   // the chain of step 1
+    float col[K], comp = 0.f;                  // this lane's column of Pi
+#pragma unroll
+    for (int y = 0; y < K; ++y) col[y] = __ldg(cg->Pi + y * K + lane);
+    const float q1 = __ldg(cg->q1 + lane);
+    if (start) L = 0.f;
+    float* buf = slot[w];
+    float* fo = filt + k0 * K + lane;
+    float* lo = loglik ? loglik + k0 : nullptr;
+    Ahead<K> lk;
+    lk.init(lik + k0 * K + lane, n, K);
+    const int nmax = (int)__reduce_max_sync(kFull, (unsigned)n);
+#pragma unroll 1
+    for (int i0 = 0; i0 < nmax; i0 += kAhead) {
+        float lx[kAhead];
+        int le[kAhead];
+        lk.take(i0, lx);
+        scale_rows<K>(lx, le, bad);
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            // p'(x) = (p Pi)(x) l(x) / c, L' = L + log c (Kahan-compensated)
+            float v = row_dot<K>(col, p, buf);
+            if (start && i0 + j == 0) v = q1;
+            v *= lx[j];
+            const float s = group_sum<K>(v);
+            if (i0 + j < n) {
+                bad |= !(s > 0.f);
+                p = v * (1.f / s);
+                const float t = fmaf((float)le[j], 0.693147180559945f, __logf(s)) - comp;
+                const float Ln = L + t;
+                comp = (Ln - L) - t;
+                L = Ln;
+                if (own) {
+                    fo[(i0 + j) * K] = p;
+                    if (lo != nullptr && lane == 0) lo[i0 + j] = L;
+                }
+            }
+        }
+    }
+    bad |= !isfinite(p) || !isfinite(L);
+    report_flags(status, own ? bad : 0u, kFull, (threadIdx.x & 31) == 0);
 }
 
 // Reverse apply: smooth [T][K] = filt . beta / sum; `suf` holds the inclusive
 // tile suffixes (rows of sum one, so that beta before a tile is its g).
-template <int K, int NW, int CH>
+template <int K, int NW, int CH, int TC>
 __global__ void __launch_bounds__(NW * 32) smoother_apply_kernel(const Const<K>* __restrict__ cg,
                                                                  const float* __restrict__ lik,
                                                                  const float* __restrict__ filt, int64_t T,
@@ -493,51 +599,69 @@ __global__ void __launch_bounds__(NW * 32) smoother_apply_kernel(const Const<K>*
                                                                  uint32_t* status) {
     constexpr int NG = NW * 32 / K;
     __shared__ __align__(16) float vec[NG][K];
+    pdl_trigger();
+    pdl_wait();
     const int w = threadIdx.x / K, lane = glane<K>();
     const int64_t nch = (T + CH - 1) / CH;
-    const int64_t c = (int64_t)blockIdx.x * NG + w;
+    const int64_t cr = (int64_t)blockIdx.x * NG + w, c = min(cr, nch - 1);
+    const bool own = cr < nch;
+    const int64_t k0 = c * CH;
+    const int n = (int)((k0 + CH < T ? k0 + CH : T) - k0);
     Flags bad = 0u;
-    if (c < nch) {
-        const int64_t k0 = c * CH, k1 = (k0 + CH < T) ? k0 + CH : T;
-        float be = 1.f;   // lane z: beta(z) after the chain
-        float* buf = vec[w];
-        if ((int)blockIdx.x + 1 < ntiles) {
-            const float lg = __ldcg(suf + ((int64_t)blockIdx.x + 1) * Dims<K>::FREC + K * K + lane);
-            be = beta_of<K>(1.f, lg);
-        }
-        const int64_t ctop = min(nch, ((int64_t)blockIdx.x + 1) * NG);
+    const int64_t tile = c / TC;
+    float* buf = vec[w];
+    float be = 1.f;   // lane z: beta(z) after the chain
+    {
+        const bool more = (int)tile + 1 < ntiles;
+        const float b1 = beta_of<K>(1.f, __ldcg(suf + (more ? tile + 1 : tile) * Dims<K>::FREC + K * K + lane));
+        be = more ? b1 : 1.f;
+        const int64_t ctop = min(nch, (tile + 1) * TC);
+        const int later = (int)(ctop - 1 - c);   // the tile's later chains, a record ahead
+        const int lmax = (int)__reduce_max_sync(kFull, (unsigned)later);
+        FRow<K> nx;
+        load_frow(b.chain + (ctop - 1) * Dims<K>::FREC, nx);
 #pragma unroll 1
-        for (int64_t j = ctop - 1; j > c; --j) {   // the tile's later chains
-            FRow<K> r;
-            load_frow(b.chain + j * Dims<K>::FREC, r);
-            be = beta_of<K>(row_dot<K>(r.f, be, buf), r.lg);
+        for (int j = 0; j < lmax; ++j) {
+            const FRow<K> r = nx;
+            load_frow(b.chain + max(ctop - 2 - j, c) * Dims<K>::FREC, nx);
+            const float v = beta_of<K>(row_dot<K>(r.f, be, buf), r.lg);
+            if (j < later) be = v;
         }
-        float row[K];   // this lane's row of Pi
-#pragma unroll
-        for (int x = 0; x < K; ++x) row[x] = __ldg(cg->Pi + lane * K + x);
-        constexpr float kUp = 1.152921504606847e18f;   // 2^60: see hmm::smoothed
-        float pn = __ldg(filt + (k1 - 1) * K + lane), ln = __ldg(lik + (k1 - 1) * K + lane);
-        float s = 0.f;
-#pragma unroll 1
-        for (int64_t k = k1 - 1; k >= k0; --k) {
-            const float p = pn, lx = ln;
-            if (k > k0) {
-                pn = __ldg(filt + (k - 1) * K + lane);
-                ln = __ldg(lik + (k - 1) * K + lane);
-            }
-            s = (p * kUp) * (be * kUp);
-            const float t = group_sum<K>(s), m = group_max<K>(lx);
-            bad |= !(t > 0.f) || !(m > 0.f);
-            s = s / t;
-            smooth[k * K + lane] = s;
-            // beta_{k-1} = Pi (l_k . beta_k), both factors rescaled by powers of two
-            int e;
-            const float v = row_dot<K>(row, lx * pow2_of(m, e) * be, buf);
-            be = v * pow2_of(group_max<K>(v), e);
-        }
-        bad |= !isfinite(s);
     }
-    report_flags(status, bad, kFull, (threadIdx.x & 31) == 0);
+    float row[K];   // this lane's row of Pi
+#pragma unroll
+    for (int x = 0; x < K; ++x) row[x] = __ldg(cg->Pi + lane * K + x);
+    constexpr float kUp = 1.152921504606847e18f;   // 2^60: see hmm::smoothed
+    Ahead<K> pf, lk;
+    pf.init(filt + (k0 + n - 1) * K + lane, n, -K);
+    lk.init(lik + (k0 + n - 1) * K + lane, n, -K);
+    float* so = smooth + (k0 + n - 1) * K + lane;
+    float s = 0.f;
+    const int nmax = (int)__reduce_max_sync(kFull, (unsigned)n);
+#pragma unroll 1
+    for (int i0 = 0; i0 < nmax; i0 += kAhead) {
+        float p[kAhead], lx[kAhead];
+        int le[kAhead];
+        pf.take(i0, p);
+        lk.take(i0, lx);
+        scale_rows<K>(lx, le, bad);
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) {
+            // beta_{k-1} = Pi (l_k . beta_k), rescaled by a power of two, beside the row's own sum
+            const float v = row_dot<K>(row, lx[j] * be, buf);
+            s = (p[j] * kUp) * (be * kUp);
+            const float t = group_sum<K>(s), m = group_max<K>(v);
+            if (i0 + j < n) {
+                bad |= !(t > 0.f);
+                s *= 1.f / t;
+                if (own) so[-(i0 + j) * K] = s;
+                int e;
+                be = v * pow2_of(m, e);
+            }
+        }
+    }
+    bad |= !isfinite(be);
+    report_flags(status, own ? bad : 0u, kFull, (threadIdx.x & 31) == 0);
 }
 
 template <int K>

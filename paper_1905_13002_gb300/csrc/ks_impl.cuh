@@ -75,9 +75,9 @@ inline int launch_status() {
 // reading that kernel's results), which hides the launch gap between the
 // preparation and the scans.
 template <class... KArgs, class... Args>
-inline int launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args... args) {
+inline int launch_pdl2(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -87,6 +87,10 @@ inline int launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? KS_OK : KS_ECUDA;
+}
+template <class... KArgs, class... Args>
+inline int launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, Args... args) {
+    return launch_pdl2(kernel, dim3((unsigned)grid), block, smem, st, args...);
 }
 
 // Chained launch of a scan kernel that takes a gate (may be null) as its last
@@ -170,8 +174,8 @@ struct Impl {
         return s;
     }
     // The forward scan's retry with refinement: its own counter and flags.
-    static ScanState fstate_retry(void* ws, const Layout& L, bool gated = false) {
-        ScanState s = fstate(ws, L, gated);
+    static ScanState fstate_retry(void* ws, const Layout& L) {
+        ScanState s = fstate(ws, L);
         char* b = static_cast<char*>(ws);
         s.counter = reinterpret_cast<uint32_t*>(b + L.off_flags + 8);
         s.flags = reinterpret_cast<uint32_t*>(b + L.off_flags + 16 + 4 * (size_t)(L.ntf + L.nts));
@@ -236,23 +240,21 @@ struct Impl {
         return reinterpret_cast<float*>(static_cast<char*>(ws) + L.off_sblk);
     }
 
+    // Gated behind the settled path (launch_steady).  What comes here is mostly
+    // ill-conditioned or slow to settle, so the scan refines at once: a first
+    // scan that only detects, with a second one behind it, is one launch more on
+    // every call (TV calls, which always scan, keep the two).
     template <bool SEG>
     static int launch_filter_fused(void* ws, const Layout& L, const float* y, float* fm, float* fc,
                                    Segs<N, M> segs, cudaStream_t st) {
         constexpr int smem = filter_dyn_smem<N, FNT>();
-        auto k = filter_scan_kernel<N, M, FNT, FCH, true, true, SEG, false, REF_DETECT, false>;
-        auto kr = filter_scan_kernel<N, M, FNT, FCH, true, true, SEG, false, REF_FP64, true>;
-        static const bool ok = allow_smem(k, smem) && allow_smem(kr, smem);
+        auto k = filter_scan_kernel<N, M, FNT, FCH, true, true, SEG, false, REF_FP64, false>;
+        static const bool ok = allow_smem(k, smem);
         if (!ok) return KS_ECUDA;
         const ModelConst<N, M>* mc = mconst(ws, L);
-        // both gated: the settled path ran first (launch_steady)
         const float* none = nullptr;
-        float* sb = sblk(ws, L);
-        int rc = launch_pdl(k, L.ntf, FNT, smem, st, mc, y, none, L.ld, L.T, fm, fc, fstate(ws, L, true), sb, segs,
-                            TVArgs{});
-        if (rc) return rc;
-        return launch_pdl(kr, L.ntf, FNT, smem, st, mc, y, none, L.ld, L.T, fm, fc, fstate_retry(ws, L, true), sb, segs,
-                          TVArgs{});
+        return launch_pdl(k, L.ntf, FNT, smem, st, mc, y, none, L.ld, L.T, fm, fc, fstate(ws, L, true), sblk(ws, L),
+                          segs, TVArgs{});
     }
 
     // Time-varying model: elements from the TVElem records `el`, smoothing

@@ -35,7 +35,6 @@ struct MixedGroup {
     const float* y = nullptr;
     float *fmean = nullptr, *fcov = nullptr, *smean = nullptr, *scov = nullptr;
     ScanState fs{}, ss{};   // look-back flags and records of the two scans (counters unused)
-    ScanState fs2{};        // the forward scan's retry with refinement
     float* sagg = nullptr;  // fused smoothing aggregates, one per forward block
     uint32_t* zero = nullptr;   // the group's flags region
     int nzero = 0;
@@ -51,7 +50,6 @@ using MG2 = MixedGroup<2, 1>;
 struct MixedQueue {
     uint32_t* fcounter;
     uint32_t* scounter;
-    uint32_t* fcounter2;   // the forward scan's retry
     uint32_t* status;
 };
 
@@ -63,21 +61,17 @@ constexpr int kMixedThreads = 128;
 int launch_mixed_plan(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, bool fold, cudaStream_t st);
 int launch_mixed_steady(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, cudaStream_t st);
 
-template <int CH, int REF, bool RETRY>
+template <int CH>
 KS_DEV void mixed_filter_tile(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q);
 
-// REF / RETRY as for filter_scan_kernel: the first launch detects
-// ill-conditioned inverses, the retry repeats the scan with refinement only
-// when the first met one.
-template <int CH, int REF, bool RETRY>
+// Behind the settled path: runs when some sequence wants the scans, and then
+// refines ill-conditioned inverses at once.
+template <int CH>
 __global__ void __launch_bounds__(kMixedThreads) mixed_filter_kernel(MG6 g6, MG4 g4, MG2 g2, MixedQueue q) {
     pdl_trigger();
     pdl_wait();
     if (!general_wanted(q.status)) return;   // the settled path took every sequence
-    if constexpr (RETRY) {
-        if (*(volatile uint32_t*)(q.status + HDR_NEED) == 0u) return;
-    }
-    mixed_filter_tile<CH, REF, RETRY>(g6, g4, g2, q);
+    mixed_filter_tile<CH>(g6, g4, g2, q);
 }
 
 // Dynamic shared memory of one size's body: its block-scan state first, its
@@ -101,27 +95,27 @@ constexpr int mixed_smoother_smem() {
                      mixed_smoother_smem_of<2, 1>());
 }
 
-template <int N, int M, int CH, int REF, bool RETRY>
+template <int N, int M, int CH>
 KS_DEV void mixed_filter_one(char* dsm, int t, const MixedGroup<N, M>& g) {
     auto& sm = *reinterpret_cast<FilterSmem<N, M, kMixedThreads>*>(dsm);
     char* stage = dsm + align16(sizeof(FilterSmem<N, M, kMixedThreads>));
-    filter_scan_body<N, M, kMixedThreads, CH, true, true, true, false, REF>(
-        sm, stage, t, g.y, nullptr, 0, g.T, g.fmean, g.fcov, RETRY ? g.fs2 : g.fs, g.sagg, g.segs, TVArgs{});
+    filter_scan_body<N, M, kMixedThreads, CH, true, true, true, false, REF_FP64>(
+        sm, stage, t, g.y, nullptr, 0, g.T, g.fmean, g.fcov, g.fs, g.sagg, g.segs, TVArgs{});
 }
 
-template <int CH, int REF, bool RETRY>
+template <int CH>
 KS_DEV void mixed_filter_tile(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q) {
     __shared__ int s_tile;
     extern __shared__ __align__(16) char dsm[];
-    if (threadIdx.x == 0) s_tile = (int)atomicAdd(RETRY ? q.fcounter2 : q.fcounter, 1u);
+    if (threadIdx.x == 0) s_tile = (int)atomicAdd(q.fcounter, 1u);
     __syncthreads();
     int t = s_tile;
     if (t < g6.ntiles) {
-        mixed_filter_one<6, 3, CH, REF, RETRY>(dsm, t, g6);
+        mixed_filter_one<6, 3, CH>(dsm, t, g6);
     } else if ((t -= g6.ntiles) < g4.ntiles) {
-        mixed_filter_one<4, 2, CH, REF, RETRY>(dsm, t, g4);
+        mixed_filter_one<4, 2, CH>(dsm, t, g4);
     } else if ((t -= g4.ntiles) < g2.ntiles) {
-        mixed_filter_one<2, 1, CH, REF, RETRY>(dsm, t, g2);
+        mixed_filter_one<2, 1, CH>(dsm, t, g2);
     }
 }
 
@@ -212,8 +206,6 @@ struct Mixed {
         o.fs.pre = reinterpret_cast<float*>(b + L.off_fpre);
         o.fs.status = status;
         o.fs.spin_limit = kSpinLimit;
-        o.fs2 = o.fs;
-        o.fs2.flags = reinterpret_cast<uint32_t*>(b + L.off_flags + 16 + 4 * (size_t)(L.ntf + L.nts));
         o.ss.counter = nullptr;
         o.ss.flags = reinterpret_cast<uint32_t*>(b + L.off_flags + 16 + 4 * (size_t)L.ntf);
         o.ss.agg = reinterpret_cast<float*>(b + L.off_sagg);
@@ -241,22 +233,16 @@ struct Mixed {
         const MG4 g4 = group<4, 2>(gs, slot[1], w, base[1], fold);
         const MG2 g2 = group<2, 1>(gs, slot[2], w, base[2], fold);
         const MixedQueue q{reinterpret_cast<uint32_t*>(w + kMixedQueueOff),
-                           reinterpret_cast<uint32_t*>(w + kMixedQueueOff + 4),
-                           reinterpret_cast<uint32_t*>(w + kMixedQueueOff + 8), reinterpret_cast<uint32_t*>(w)};
+                           reinterpret_cast<uint32_t*>(w + kMixedQueueOff + 4), reinterpret_cast<uint32_t*>(w)};
         const int ntiles = g6.ntiles + g4.ntiles + g2.ntiles;
-        static const bool ok = allow_smem(mixed_filter_kernel<CH, REF_DETECT, false>, mixed_filter_smem()) &&
-                               allow_smem(mixed_filter_kernel<CH, REF_FP64, true>, mixed_filter_smem()) &&
+        static const bool ok = allow_smem(mixed_filter_kernel<CH>, mixed_filter_smem()) &&
                                allow_smem(mixed_smoother_kernel<CH>, mixed_smoother_smem());
         if (!ok) return KS_ECUDA;
         int rc = launch_mixed_plan(g6, g4, g2, q, fold, st);
         if (rc) return rc;
         if ((rc = launch_mixed_steady(g6, g4, g2, q, st))) return rc;
-        if ((rc = launch_pdl(mixed_filter_kernel<CH, REF_DETECT, false>, ntiles, kMixedThreads, mixed_filter_smem(),
-                             st, g6, g4, g2, q)))
-            return rc;
-        if ((rc = launch_pdl(mixed_filter_kernel<CH, REF_FP64, true>, ntiles, kMixedThreads, mixed_filter_smem(), st,
-                             g6, g4, g2, q)))
-            return rc;
+        rc = launch_pdl(mixed_filter_kernel<CH>, ntiles, kMixedThreads, mixed_filter_smem(), st, g6, g4, g2, q);
+        if (rc) return rc;
         return launch_pdl(mixed_smoother_kernel<CH>, ntiles, kMixedThreads, mixed_smoother_smem(), st, g6, g4, g2, q);
     }
 };

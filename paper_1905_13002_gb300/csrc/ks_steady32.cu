@@ -150,55 +150,86 @@ __global__ void __launch_bounds__(kPlanNT) plan32_kernel(Args32 g) {
     if (blockIdx.x == 0 && t == 0) g.status[HDR_GENERAL] = 0u;
     prep_inputs<N, M>(p, 0, 1, g.F, g.u, g.Q, g.H, g.d, g.R, g.m0, g.P0, g.y, g.status, g.zero,
                       blockIdx.x == 0 ? g.nzero : 0, nullptr, g.T, nullptr);
-    if (blockIdx.x == 1) {   // the k = 1 element in FP64
+    if (blockIdx.x == 1) {   // the k = 1 element in FP64, and beside it the scans' own constants
         if (t < kFirstThreads) first_element_fp64<N, M>(p, mc, t);
+        else if (w == 4) prep_consts<N, M>(p, mc, lane);
         __syncthreads();
-        for (int e = t; e < sym_size(N); e += kPlanNT) g.mconst->C1[e] = mc.C1[e];
-        for (int e = t; e < N; e += kPlanNT) { g.mconst->b1[e] = mc.b1[e]; out.b1[e] = mc.b1[e]; }
+        prep_store<N, M>(p, mc, g.mconst, g.status);
+        for (int e = t; e < N; e += kPlanNT) out.b1[e] = mc.b1[e];
         for (int e = t; e < N * N; e += kPlanNT) out.C1[e] = mc.C1[sidx(e / N, e % N)];
-        if (t == 0) {
-            out.ok1 = p.ok1;
-            if (!p.ok1) atomicOr(g.status, ST_NUMERIC);
-        }
+        if (t == 0) out.ok1 = p.ok0 && p.ok1;
         return;
     }
     PlanSmem32& s = *reinterpret_cast<PlanSmem32*>(dsm32 + plan32_off());
     const tc::VS<N> vs{s.vs};
     if (t == 0) s.ok = 1;
-    if (w == 0) prep_consts<N, M>(p, mc, lane);
-    __syncthreads();
-    {   // the constants for the scans (b1, C1 come from block 1)
-        const float* src = reinterpret_cast<const float*>(&mc);
-        float* dst = reinterpret_cast<float*>(g.mconst);
-        using MC = ModelConst<N, M>;
-        const int skip = (int)offsetof(MC, b1) / 4;
-        for (int i = t; i < skip; i += kPlanNT) dst[i] = src[i];
-        if (t < 4) g.mconst->pad[t] = 0.f;
-        if (t == 0 && !p.ok0) atomicOr(g.status, ST_NUMERIC);
+    // Lemma 3's constants with S^-1 in place of its factor: HQ, HF; S; K = (H Q)^T S^-1, V = S^-1 H F;
+    // A = F - K H F, C = Q - K H Q, J = (H F)^T V
+    float *HQ = s.X, *V8 = s.W;
+    {
+        const int q = (t & 255) / N, a = t % N;
+        float v = 0.f;
+        if (t < 256) {
+#pragma unroll 8
+            for (int c = 0; c < N; ++c) v = fmaf(p.H[q][c], 0.5f * (p.Q[c][a] + p.Q[a][c]), v);
+            HQ[q * P + a] = v;
+        } else {
+#pragma unroll 8
+            for (int c = 0; c < N; ++c) v = fmaf(p.H[q][c], p.F[c][a], v);
+            s.HF[q * P + a] = v;
+            out.HF[q * N + a] = v;
+            s.H[q * P + a] = p.H[q][a];
+            out.H[q * N + a] = p.H[q][a];
+        }
     }
+    __syncthreads();
+    if (t < 64) {
+        const int a = t / M, b = t % M;
+        const float r = 0.5f * (p.R[a][b] + p.R[b][a]);
+        s.R[t] = r;
+        out.R[t] = r;
+        float v = r;
+#pragma unroll 8
+        for (int c = 0; c < N; ++c) v = fmaf(HQ[a * P + c], p.H[b][c], v);
+        s.S[t] = v;
+    }
+    __syncthreads();
+    if (w == 0) {
+        float cond;
+        const bool ok = warp_inverse<M>(s.S, s.Si, lane, cond) && cond <= kRefineCond;
+        if (!__all_sync(kAll, ok) && lane == 0) s.ok = 0;
+    }
+    __syncthreads();
+    {
+        const int q = (t & 255) / N, a = t % N;
+        float v = 0.f;
+#pragma unroll
+        for (int r = 0; r < M; ++r) v = fmaf(s.Si[q * M + r], t < 256 ? HQ[r * P + a] : s.HF[r * P + a], v);
+        if (t < 256) s.KB[a * M + q] = v;
+        else V8[q * P + a] = v;
+    }
+    __syncthreads();
     for (int e = t; e < N * N; e += kPlanNT) {
         const int a = e / N, b = e % N;
-        s.A[0][a * P + b] = mc.A[e];
-        s.C[0][a * P + b] = mc.C[sidx(a, b)];
-        float j = 0.f;
-        for (int q = 0; q < M; ++q) j = fmaf(mc.U[q * N + a], mc.U[q * N + b], j);
-        s.J[0][a * P + b] = j;
-        out.F[e] = mc.F[e];
-        out.Q[e] = mc.Q[sidx(a, b)];
+        const float qs = 0.5f * (p.Q[a][b] + p.Q[b][a]);
+        float va = p.F[a][b], vc = qs, vj = 0.f;
+#pragma unroll
+        for (int q = 0; q < M; ++q) {
+            va = fmaf(-s.KB[a * M + q], s.HF[q * P + b], va);
+            vc = fmaf(-s.KB[a * M + q], HQ[q * P + b], vc);
+            vj = fmaf(s.HF[q * P + a], V8[q * P + b], vj);
+        }
+        s.A[0][a * P + b] = va;
+        s.C[0][a * P + b] = vc;
+        s.J[0][a * P + b] = vj;
+        out.F[e] = p.F[a][b];
+        out.Q[e] = qs;
     }
-    for (int e = t; e < M * N; e += kPlanNT) {
-        const int q = e / N, a = e % N;
-        s.H[q * P + a] = p.H[q][a];
-        s.HF[q * P + a] = p.HF[q][a];
-        out.H[e] = p.H[q][a];
-        out.HF[e] = p.HF[q][a];
-    }
-    for (int e = t; e < M * M; e += kPlanNT) {
-        s.R[e] = 0.5f * (p.R[e / M][e % M] + p.R[e % M][e / M]);
-        out.R[e] = s.R[e];
-    }
-    if (t < N) out.u[t] = mc.u[t];
+    if (t < N) out.u[t] = p.u[t];
     if (t < M) out.d[t] = p.d[t];
+    __syncthreads();
+    symmetrise(s.C[0], t, kPlanNT);
+    symmetrise(s.J[0], t, kPlanNT);
     __syncthreads();
     // ---- doubling: 16 warps, four to a product
     int cur = 0;
@@ -235,7 +266,7 @@ __global__ void __launch_bounds__(kPlanNT) plan32_kernel(Args32 g) {
     // ---- settled covariances, gains, Phi
     const float *A = s.A[cur], *Pf = s.C[cur], *J = s.J[cur];
     float* Fs = s.V;
-    for (int e = t; e < N * N; e += kPlanNT) Fs[(e / N) * P + e % N] = mc.F[e];
+    for (int e = t; e < N * N; e += kPlanNT) Fs[(e / N) * P + e % N] = p.F[e / N][e % N];
     __syncthreads();
     if (grp == 0) mprod<8, false, false>(Fs, Pf, s.X, gw, lane);          // F P
     else if (grp == 1) mprod<8, false, false>(Pf, J, s.Mx, gw, lane);     // P J
@@ -252,7 +283,7 @@ __global__ void __launch_bounds__(kPlanNT) plan32_kernel(Args32 g) {
     for (int e = t; e < N * N; e += kPlanNT) {
         const int a = e / N, b = e % N;
         if (b <= a) {
-            const float v = 0.5f * (s.Y[a * P + b] + s.Y[b * P + a]) + mc.Q[sidx(a, b)];
+            const float v = 0.5f * (s.Y[a * P + b] + s.Y[b * P + a]) + 0.5f * (p.Q[a][b] + p.Q[b][a]);
             s.Z[a * P + b] = v;                                           // P-
             s.Z[b * P + a] = v;
         }
@@ -335,7 +366,7 @@ __global__ void __launch_bounds__(kPlanNT) plan32_kernel(Args32 g) {
             out.nphi = nf;
             out.ndual = nd;
             // wait settings of the look-back are a test's: it wants the scans
-            out.ok = (s.ok != 0 && p.ok0 != 0 && nf <= kStPowTol && nd <= kStPowTol && g.status[HDR_WAIT] == 0u &&
+            out.ok = (s.ok != 0 && nf <= kStPowTol && nd <= kStPowTol && g.status[HDR_WAIT] == 0u &&
                       g.status[HDR_FIRST_TILE] == 0u) ? 1 : 0;
         }
     }
@@ -430,8 +461,20 @@ struct RowSmem32 {
     float Ph[2][MATF], O[2][MATF], X[MATF], Y[MATF], Mx[MATF], Mi[MATF], D[MATF], Pk[MATF], Pf[MATF];
     float H[M * P], HF[M * P], HP[M * P], R[64], S[64], Si[64], vs[tc::VS<N>::FLOATS];
     WarpBuf wb[8];
+    float yb[8][(kS32Chunk + 1) * M];
     alignas(128) float pat[1024];
 };
+
+// n floats of a warp's measurements into its buffer (all in flight at once; a
+// step is shorter than a load).
+KS_DEV void stage(float* __restrict__ dst, const float* __restrict__ src, int n, int lane) {
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+        if (lane + 32 * i < n) cp_async4(dst + lane + 32 * i, src + lane + 32 * i);
+    cp_async_wait_all();
+    __syncwarp();
+}
 
 // Bulk copies of one covariance row `pat` to rows [r0, r1) of dst, spread over the block's threads.
 KS_DEV void fill_rows(float* __restrict__ dst, const float* pat, int64_t r0, int64_t r1, int t, int nt) {
@@ -468,14 +511,11 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
             st.load(p, lane);
             float K[M];
             load_row8(p.K, lane, K);
-            const float* y = g.y + r0 * M;
-            float x = lift32(p, y, lane), yq = y[lane >> 2];
+            float* y = s.yb[w];
+            stage(y, g.y + r0 * M, (kS32Chunk + 1) * M, lane);
+            float x = lift32(p, y, lane);
 #pragma unroll 1
-            for (int i = 0; i < kS32Chunk; ++i) {
-                const float yn = y[(i + 1) * M + (lane >> 2)];
-                st.step(x, K, yq, s.wb[w], lane);
-                yq = yn;
-            }
+            for (int i = 0; i < kS32Chunk; ++i) st.step(x, K, y[i * M + (lane >> 2)], s.wb[w], lane);
             g.s.miss[c * 32 + lane] = x - lift32(p, y + kS32Chunk * M, lane);
         }
         if (g.keep) {
@@ -657,24 +697,22 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
     if (head) {
         // head chunk w: rows 16 w + 1 .. 16 w + 16 (the last: .. 127), its own gains
         const int a = 16 * w, cnt = w < 7 ? 16 : 15;
-        const float* y = g.y + (int64_t)(a + 1) * M;
+        float* y = s.eps[w];
+        stage(y, g.y + (int64_t)(a + 1) * M, cnt * M, lane);
         const float guess = w == 0 ? p.b1[lane] : lift32(p, g.y + (int64_t)a * M, lane);
         s.guess[w][lane] = guess;
         auto pass = [&](float x, bool write) {
-            float K[M], yq = y[lane >> 2];
+            float K[M];
             load_row8(g.s.Kr + (int64_t)(a + 1) * 256, lane, K);
 #pragma unroll 1
             for (int i = 0; i < cnt; ++i) {
-                float Kn[M], yn = 0.f;
-                const bool more = i + 1 < cnt;
-                load_row8(g.s.Kr + (int64_t)(a + 1 + (more ? i + 1 : i)) * 256, lane, Kn);
-                if (more) yn = y[(i + 1) * M + (lane >> 2)];
-                const float e = st.step(x, K, yq, s.wb[w], lane);
+                float Kn[M];
+                load_row8(g.s.Kr + (int64_t)(a + 1 + (i + 1 < cnt ? i + 1 : i)) * 256, lane, Kn);
+                const float e = st.step(x, K, y[i * M + (lane >> 2)], s.wb[w], lane);
                 if (write) {
                     g.fm[(int64_t)(a + 1 + i) * N + lane] = x;
                     if ((lane & 3) == 0) g.s.eps[(int64_t)(a + 1 + i) * M + (lane >> 2)] = e;
                 }
-                yq = yn;
 #pragma unroll
                 for (int q = 0; q < M; ++q) K[q] = Kn[q];
             }
@@ -712,22 +750,23 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
         __syncthreads();
         d = s.d[w][lane];
     } else if (c < nch) {
-#pragma unroll 1
-        for (int i = kS32Back; i >= 1; --i) d = mv(P32, d, s.wb[w].x, lane) + g.s.miss[(c - i) * 32 + lane];
+        float m[kS32Back];
+#pragma unroll
+        for (int i = 0; i < kS32Back; ++i) m[i] = g.s.miss[(c - 1 - i) * 32 + lane];
+#pragma unroll
+        for (int i = kS32Back - 1; i >= 0; --i) d = mv(P32, d, s.wb[w].x, lane) + m[i];
         if (!(p.nphi * fabsf(d) * p.rsd[lane] <= kStMeanTol)) bad = true;
     }
     if (c < nch) {
         const int cnt = (int)min((int64_t)kS32Chunk, T - r0);
-        const float* y = g.y + r0 * M;
+        float* ep = s.eps[w];                         // measurements, then innovations
+        stage(ep, g.y + r0 * M, cnt * M, lane);
         float K[M];
         load_row8(p.K, lane, K);
-        float x = lift32(p, y, lane) + d, yq = y[lane >> 2];
-        float* ep = s.eps[w];
+        float x = lift32(p, ep, lane) + d;
 #pragma unroll 1
         for (int i = 0; i < cnt; ++i) {
-            const float yn = i + 1 < cnt ? y[(i + 1) * M + (lane >> 2)] : 0.f;
-            const float e = st.step(x, K, yq, s.wb[w], lane);
-            yq = yn;
+            const float e = st.step(x, K, ep[i * M + (lane >> 2)], s.wb[w], lane);
             g.fm[(r0 + i) * N + lane] = x;
             if ((lane & 3) == 0) ep[i * M + (lane >> 2)] = e;
         }
@@ -760,9 +799,10 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
 struct RevSmem32 {
     WarpBuf wb[8];
     float nu[8][N], l[9][N];
+    float eps[8][kS32Chunk * M];
 };
 
-__global__ void __launch_bounds__(256) reverse32_kernel(Args32 g) {
+__global__ void __launch_bounds__(256, 2) reverse32_kernel(Args32 g) {
     __shared__ RevSmem32 s;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const Plan32& p = *g.s.plan;
@@ -774,12 +814,11 @@ __global__ void __launch_bounds__(256) reverse32_kernel(Args32 g) {
     load_row(p.P32T, lane, P32T);
     // the adjoint that enters chunk c from the eight chunks after it
     auto enter = [&](int64_t c) {
-        float l = 0.f;
-#pragma unroll 1
-        for (int i = kS32Back; i >= 1; --i) {
-            l = mv(P32T, l, s.wb[w].x, lane);
-            if (c + i < nch) l += g.s.mu[(c + i) * 32 + lane];
-        }
+        float l = 0.f, m[kS32Back];
+#pragma unroll
+        for (int i = 0; i < kS32Back; ++i) m[i] = c + 1 + i < nch ? g.s.mu[(c + 1 + i) * 32 + lane] : 0.f;
+#pragma unroll
+        for (int i = kS32Back - 1; i >= 0; --i) l = mv(P32T, l, s.wb[w].x, lane) + m[i];
         return l;
     };
     bool bad = false;
@@ -856,27 +895,39 @@ __global__ void __launch_bounds__(256) reverse32_kernel(Args32 g) {
             load_row(p.PhT, lane, PhT);
             load_row(p.Pf, lane, Pr);
             load_row8(p.B, lane, B);
+            stage(s.eps[w], g.s.eps + r0 * M, cnt * M, lane);
             float l = enter(c);
             if (c + kS32Back < nch && !(p.ndual * fabsf(l) * p.sd[lane] <= kStMeanTol)) bad = true;
-            float m = g.fm[(r0 + cnt - 1) * N + lane], e = g.s.eps[(r0 + cnt - 1) * M + (lane >> 2)];
-#pragma unroll 1
-            for (int i = cnt - 1; i >= 0; --i) {
-                const int64_t r = r0 + i, n = i > 0 ? r - 1 : r;
-                const float mn = g.fm[n * N + lane], en = g.s.eps[n * M + (lane >> 2)];
-                g.sm[r * N + lane] = m + mv(Pr, l, s.wb[w].x, lane);
-                // the same buffer holds l: Phi^T l needs no second broadcast
-                float a0 = 0.f, a1 = 0.f;
+            constexpr int AH = 4;                       // filtered means loaded ahead
+            float mn[AH];
 #pragma unroll
-                for (int q = 0; q < N; q += 4) {
-                    const float4 v = *reinterpret_cast<const float4*>(s.wb[w].x + q);
-                    a0 = fmaf(PhT[q], v.x, a0);
-                    a1 = fmaf(PhT[q + 1], v.y, a1);
-                    a0 = fmaf(PhT[q + 2], v.z, a0);
-                    a1 = fmaf(PhT[q + 3], v.w, a1);
+            for (int j = 0; j < AH; ++j) mn[j] = g.fm[(r0 + max(cnt - 1 - j, 0)) * N + lane];
+            const float* ep = s.eps[w];
+#pragma unroll 1
+            for (int i0 = cnt - 1; i0 >= 0; i0 -= AH) {
+                float m[AH];
+#pragma unroll
+                for (int j = 0; j < AH; ++j) {
+                    m[j] = mn[j];
+                    mn[j] = g.fm[(r0 + max(i0 - AH - j, 0)) * N + lane];
                 }
-                l = (a0 + a1) + mv8(B, e);
-                m = mn;
-                e = en;
+#pragma unroll
+                for (int j = 0; j < AH; ++j) {
+                    const int i = i0 - j;
+                    if (i < 0) break;
+                    g.sm[(r0 + i) * N + lane] = m[j] + mv(Pr, l, s.wb[w].x, lane);
+                    // the same buffer holds l: Phi^T l needs no second broadcast
+                    float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+                    for (int q = 0; q < N; q += 4) {
+                        const float4 v = *reinterpret_cast<const float4*>(s.wb[w].x + q);
+                        a0 = fmaf(PhT[q], v.x, a0);
+                        a1 = fmaf(PhT[q + 1], v.y, a1);
+                        a0 = fmaf(PhT[q + 2], v.z, a0);
+                        a1 = fmaf(PhT[q + 3], v.w, a1);
+                    }
+                    l = (a0 + a1) + mv8(B, ep[i * M + (lane >> 2)]);
+                }
             }
             if (!(fabsf(l) < 1e30f)) bad = true;
         }

@@ -37,7 +37,6 @@ __global__ void __launch_bounds__(kPlanThreads) mixed_plan_kernel(MG6 g6, MG4 g4
     if (b == 0 && threadIdx.x == 0) {
         *q.fcounter = 0u;
         *q.scounter = 0u;
-        *q.fcounter2 = 0u;
     }
     if (b < g6.B) { plan_block<6, 3, FOLD>(prep_dsm, b, plan_args(g6)); return; }
     b -= g6.B;
