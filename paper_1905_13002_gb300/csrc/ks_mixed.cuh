@@ -1,4 +1,4 @@
-// ks_mixed.cuh -- one preparation, one settled-path launch (ks_steady.cuh) and,
+// ks_mixed.cuh -- one preparation, the settled path (ks_steady.cuh) and,
 // when a sequence needs them, one forward and one reverse scan launch over a
 // batch whose sequences have different state sizes (nx in {2, 4, 6}).
 //
@@ -57,7 +57,7 @@ constexpr int kMixedThreads = 128;
 
 // The preparation with the settled path's plans, one block per sequence of all
 // groups (nx = 6 sequences first; it also zeroes the queue counters), and the
-// settled path, one launch over the windows of all groups (ks_steady_mixed.cu).
+// settled path, one launch per state size (ks_steady_mixed.cu).
 int launch_mixed_plan(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, bool fold, cudaStream_t st);
 int launch_mixed_steady(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, cudaStream_t st);
 

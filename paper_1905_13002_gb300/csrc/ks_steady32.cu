@@ -476,10 +476,11 @@ KS_DEV void stage(float* __restrict__ dst, const float* __restrict__ src, int n,
     __syncwarp();
 }
 
-// Bulk copies of one covariance row `pat` to rows [r0, r1) of dst, spread over the block's threads.
-KS_DEV void fill_rows(float* __restrict__ dst, const float* pat, int64_t r0, int64_t r1, int t, int nt) {
-    for (int64_t r = r0 + t; r < r1; r += nt) bulk_store(dst + r * 1024, pat, 4096u);
-    bulk_commit();
+// A chunk's constant covariance rows go out as bulk copies of a shared-memory
+// row, one beside each step of the chunk's recursion: the memory takes them no
+// faster than it writes, and a step is longer than its share of that.
+KS_DEV void fill_row(float* __restrict__ dst, const float* pat, int64_t r, int64_t end, int lane) {
+    if (lane == 0 && r < end) bulk_store(dst + r * 1024, pat, 4096u);
 }
 
 __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
@@ -504,9 +505,12 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
     const int64_t T = g.T;
     if (blockIdx.x >= kS32Head) {
         // ---- eight chunks: one pass from the guess, what it misses the next chunk's guess by
-        const int64_t cb = blockIdx.x - kS32Head;
-        const int64_t c = cb * 8 + w, r0 = kS32Head + c * kS32Chunk;
-        if (r0 + kS32Chunk < T) {                     // the last chunk's miss is not needed
+        const int64_t c = (blockIdx.x - kS32Head) * 8 + w, r0 = kS32Head + c * kS32Chunk;
+        const int64_t fend = g.keep ? T : 0;          // constant filtered rows: all of them
+        for (int e = t; e < 1024; e += kRowNT) s.pat[e] = p.Pf[e];
+        fence_proxy_async();
+        __syncthreads();
+        if (r0 + kS32Chunk < T) {
             Step32 st;
             st.load(p, lane);
             float K[M];
@@ -515,16 +519,15 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
             stage(y, g.y + r0 * M, (kS32Chunk + 1) * M, lane);
             float x = lift32(p, y, lane);
 #pragma unroll 1
-            for (int i = 0; i < kS32Chunk; ++i) st.step(x, K, y[i * M + (lane >> 2)], s.wb[w], lane);
+            for (int i = 0; i < kS32Chunk; ++i) {
+                st.step(x, K, y[i * M + (lane >> 2)], s.wb[w], lane);
+                fill_row(g.fc, s.pat, r0 + i, fend, lane);
+            }
             g.s.miss[c * 32 + lane] = x - lift32(p, y + kS32Chunk * M, lane);
+        } else {                                      // the last chunk's miss is not needed
+            for (int i = 0; i < kS32Chunk; ++i) fill_row(g.fc, s.pat, r0 + i, fend, lane);
         }
-        if (g.keep) {
-            for (int e = t; e < 1024; e += kRowNT) s.pat[e] = p.Pf[e];
-            fence_proxy_async();
-            __syncthreads();
-            const int64_t f0 = kS32Head + cb * 256;
-            fill_rows(g.fc, s.pat, f0, min(f0 + 256, T), t, kRowNT);
-        }
+        bulk_commit();
         bulk_wait_read_all();
         return;
     }
@@ -661,6 +664,7 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
 
 // ---------------------------------------------------------------- forward
 constexpr int kFwdNT = 256;
+constexpr int kS32Fwd = 18;         // rows of a chunk whose smoothed covariance the forward kernel fills
 struct FwdSmem32 {
     WarpBuf wb[8];
     float guess[9][N], miss[8][N], d[8][N], xlast[N];
@@ -689,6 +693,12 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
     const int64_t c = (int64_t)blockIdx.x * 8 + w, r0 = kS32Head + c * kS32Chunk;
     const bool head = blockIdx.x == 0;
     bool bad = false;
+    // constant smoothed rows, all but the last 128 (the first kS32Fwd of each
+    // chunk here, the others in the reverse kernel)
+    const int64_t fend = g.sc != nullptr ? T - kS32Head : 0;
+    for (int e = t; e < 1024; e += kFwdNT) s.pat[e] = p.Ps[e];
+    fence_proxy_async();
+    __syncthreads();
     Step32 st;
     st.load(p, lane);
     float P32[N];
@@ -744,7 +754,7 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
 #pragma unroll 1
             for (int h = 0; h < 8; ++h) {
                 s.d[h][lane] = dd;
-                dd = mv(P32, dd, s.wb[0].x, lane) + g.s.miss[h * 32 + lane];
+                dd = mv(P32, dd, s.wb[0].x, lane) + (h + 1 < nch ? g.s.miss[h * 32 + lane] : 0.f);
             }
         }
         __syncthreads();
@@ -769,6 +779,7 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
             const float e = st.step(x, K, ep[i * M + (lane >> 2)], s.wb[w], lane);
             g.fm[(r0 + i) * N + lane] = x;
             if ((lane & 3) == 0) ep[i * M + (lane >> 2)] = e;
+            if (i < kS32Fwd) fill_row(g.sc, s.pat, r0 + i, fend, lane);
         }
         if (!(fabsf(x) < 1e30f)) bad = true;
         __syncwarp();
@@ -784,13 +795,7 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
             g.s.mu[c * 32 + lane] = l;
         }
     }
-    if (g.sc != nullptr) {                            // constant smoothed rows of these chunks
-        for (int e = t; e < 1024; e += kFwdNT) s.pat[e] = p.Ps[e];
-        fence_proxy_async();
-        __syncthreads();
-        const int64_t f0 = kS32Head + (int64_t)blockIdx.x * 256;
-        fill_rows(g.sc, s.pat, f0, min(f0 + 256, T - kS32Head), t, kFwdNT);
-    }
+    bulk_commit();
     if (__any_sync(kAll, bad) && lane == 0) atomicOr(g.status + HDR_GENERAL, 1u);
     bulk_wait_read_all();
 }
@@ -800,6 +805,7 @@ struct RevSmem32 {
     WarpBuf wb[8];
     float nu[8][N], l[9][N];
     float eps[8][kS32Chunk * M];
+    alignas(128) float pat[1024];
 };
 
 __global__ void __launch_bounds__(256, 2) reverse32_kernel(Args32 g) {
@@ -889,6 +895,9 @@ __global__ void __launch_bounds__(256, 2) reverse32_kernel(Args32 g) {
         if (w == 0) smooth_row(0, l);
     } else {
         const int64_t c = (int64_t)(blockIdx.x - 1) * 8 + w, r0 = kS32Head + c * kS32Chunk;
+        for (int e = t; e < 1024; e += 256) s.pat[e] = p.Ps[e];
+        fence_proxy_async();
+        __syncthreads();
         if (c < nch) {
             const int cnt = (int)min((int64_t)kS32Chunk, T - r0);
             float PhT[N], Pr[N], B[M];
@@ -896,6 +905,7 @@ __global__ void __launch_bounds__(256, 2) reverse32_kernel(Args32 g) {
             load_row(p.Pf, lane, Pr);
             load_row8(p.B, lane, B);
             stage(s.eps[w], g.s.eps + r0 * M, cnt * M, lane);
+            const int64_t fend = T - kS32Head;
             float l = enter(c);
             if (c + kS32Back < nch && !(p.ndual * fabsf(l) * p.sd[lane] <= kStMeanTol)) bad = true;
             constexpr int AH = 4;                       // filtered means loaded ahead
@@ -915,6 +925,7 @@ __global__ void __launch_bounds__(256, 2) reverse32_kernel(Args32 g) {
                 for (int j = 0; j < AH; ++j) {
                     const int i = i0 - j;
                     if (i < 0) break;
+                    if (i >= kS32Fwd) fill_row(g.sc, s.pat, r0 + i, fend, lane);
                     g.sm[(r0 + i) * N + lane] = m[j] + mv(Pr, l, s.wb[w].x, lane);
                     // the same buffer holds l: Phi^T l needs no second broadcast
                     float a0 = 0.f, a1 = 0.f;
@@ -933,6 +944,8 @@ __global__ void __launch_bounds__(256, 2) reverse32_kernel(Args32 g) {
         }
     }
     if (__any_sync(kAll, bad) && lane == 0) atomicOr(g.status + HDR_GENERAL, 1u);
+    bulk_commit();
+    bulk_wait_read_all();
 }
 
 template <class K>

@@ -28,7 +28,7 @@ namespace ks {
 constexpr int kS32Head = 128;       // rows with gains of their own
 constexpr int kS32Chunk = 32;       // rows of a chunk
 constexpr int kS32Back = 8;         // chunks that reach 256 rows
-constexpr int kS32MinT = 768;       // shorter sequences go through the scans
+constexpr int kS32MinT = 256;       // head and end rows apart; shorter sequences go through the scans
 
 struct Plan32 {
     float F[1024], Ph[1024], PhT[1024], P32[1024], P32T[1024], Pf[1024], Ps[1024];

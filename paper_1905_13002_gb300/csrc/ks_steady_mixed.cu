@@ -1,9 +1,15 @@
 // The settled path (ks_steady.cuh) of a mixed-size batch (ks_mixed.cuh): one
-// preparation and one window launch over the sequences of all sizes.
+// preparation over the sequences of all sizes, and the windows one size after
+// another.  (One launch for all three gave every block nx = 6's 250 registers
+// and 104 KB, two blocks per SM where nx = 4 and 2 fit three and four.)
 #include "ks_mixed.cuh"
 #include "ks_steady_kernels.cuh"
 
 namespace ks {
+
+extern template int launch_steady_kernel<6, 3>(const SteadyArgs<6, 3>&, cudaStream_t);   // ks_steady6.cu, ...
+extern template int launch_steady_kernel<4, 2>(const SteadyArgs<4, 2>&, cudaStream_t);
+extern template int launch_steady_kernel<2, 1>(const SteadyArgs<2, 1>&, cudaStream_t);
 
 namespace {
 
@@ -23,7 +29,7 @@ KS_DEV PlanArgs<N, M> plan_args(const MixedGroup<N, M>& g) {
 }
 
 template <int N, int M>
-KS_DEV SteadyArgs<N, M> steady_args(const MixedGroup<N, M>& g) {
+SteadyArgs<N, M> steady_args(const MixedGroup<N, M>& g) {
     return SteadyArgs<N, M>{g.plan, g.segs.off, g.B, g.T, g.y, g.fmean, g.fcov, g.smean, g.scov, 1, g.fs.status};
 }
 
@@ -45,18 +51,6 @@ __global__ void __launch_bounds__(kPlanThreads) mixed_plan_kernel(MG6 g6, MG4 g4
     if (b < g2.B) plan_block<2, 1, FOLD>(prep_dsm, b, plan_args(g2));
 }
 
-// The windows of all groups, nx = 6 first (n6, n4: its and nx = 4's slots).
-__global__ void __launch_bounds__(kStNT, kSteadyMinBlocks<6>) mixed_steady_kernel(MG6 g6, MG4 g4, MG2 g2, int64_t n6,
-                                                                                  int64_t n4) {
-    extern __shared__ __align__(16) char dsm[];
-    pdl_trigger();
-    int64_t s = (int64_t)blockIdx.x;
-    if (s < n6) { steady_block<6, 3>(dsm, steady_args(g6), s); return; }
-    s -= n6;
-    if (s < n4) { steady_block<4, 2>(dsm, steady_args(g4), s); return; }
-    steady_block<2, 1>(dsm, steady_args(g2), s - n4);
-}
-
 }  // namespace
 
 int launch_mixed_plan(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, bool fold, cudaStream_t st) {
@@ -71,14 +65,11 @@ int launch_mixed_plan(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQu
 }
 
 int launch_mixed_steady(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue&, cudaStream_t st) {
-    constexpr int smem =
-        (int)cmax(cmax(sizeof(SteadySmem<6, 3>), sizeof(SteadySmem<4, 2>)), sizeof(SteadySmem<2, 1>));
-    static const bool ok = cudaFuncSetAttribute(mixed_steady_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                smem) == cudaSuccess;
-    if (!ok) return KS_ECUDA;
-    const int64_t n6 = g6.B ? steady_blocks(g6.T, g6.B) : 0, n4 = g4.B ? steady_blocks(g4.T, g4.B) : 0,
-                  n2 = g2.B ? steady_blocks(g2.T, g2.B) : 0;
-    return launch_pdl(mixed_steady_kernel, (int)(n6 + n4 + n2), kStNT, smem, st, g6, g4, g2, n6, n4);
+    int rc = KS_OK;
+    if (g6.B && (rc = launch_steady_kernel(steady_args(g6), st))) return rc;
+    if (g4.B && (rc = launch_steady_kernel(steady_args(g4), st))) return rc;
+    if (g2.B) rc = launch_steady_kernel(steady_args(g2), st);
+    return rc;
 }
 
 }  // namespace ks

@@ -127,9 +127,9 @@ def test_non_finite_measurement_takes_the_scans(ks, nx, value, at):
         assert general == 1
 
 
-# nx = 32 takes the settled path from 768 rows on: edges of its chunks of 32,
+# nx = 32 takes the settled path from 256 rows on: edges of its chunks of 32,
 # of the eight chunks behind a chunk, and of a block's eight chunks
-@pytest.mark.parametrize("T", [767, 768, 769, 799, 800, 801, 1151, 1152, 1153, 2000, 5000])
+@pytest.mark.parametrize("T", [256, 257, 383, 384, 385, 416, 767, 768, 769, 799, 800, 801, 1153, 2000, 5000])
 def test_edges_nx32(ks, T):
     rng = np.random.default_rng(9000 + T)
     m = model_of(32, rng)
