@@ -37,20 +37,32 @@ struct GBuf {
 };
 
 // Copy an element slot (n floats) between two locations, by the lanes of the
-// calling chain's group.
-template <int N>
-KS_DEV void copy_floats(float* dst, const float* src, int n) {
+// calling chain's group: kCopy loads of each lane in flight before the first is
+// stored (one load at a time, a 234-float element took ~30 trips to L2, longer
+// than its combine).  CG: data written by other blocks or launches (L2 loads).
+constexpr int kCopy = 16;
+template <int N, bool CG>
+KS_DEV void copy_slot(float* dst, const float* src, int n) {
     constexpr int GS = Grp<N>::GS;
-    for (int i = threadIdx.x & (GS - 1); i < n; i += GS) dst[i] = src[i];
+    for (int i0 = threadIdx.x & (GS - 1); i0 < n; i0 += GS * kCopy) {
+        float v[kCopy];
+#pragma unroll
+        for (int u = 0; u < kCopy; ++u) {
+            const int i = i0 + u * GS;
+            v[u] = i < n ? (CG ? __ldcg(src + i) : src[i]) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < kCopy; ++u) {
+            const int i = i0 + u * GS;
+            if (i < n) dst[i] = v[u];
+        }
+    }
     gsync<N>();
 }
-// The same from data written by other blocks or launches (L2 loads).
 template <int N>
-KS_DEV void copy_floats_cg(float* dst, const float* src, int n) {
-    constexpr int GS = Grp<N>::GS;
-    for (int i = threadIdx.x & (GS - 1); i < n; i += GS) dst[i] = __ldcg(src + i);
-    gsync<N>();
-}
+KS_DEV void copy_floats(float* dst, const float* src, int n) { copy_slot<N, false>(dst, src, n); }
+template <int N>
+KS_DEV void copy_floats_cg(float* dst, const float* src, int n) { copy_slot<N, true>(dst, src, n); }
 
 template <int N, int M>
 KS_DEV void load_const_all(const ModelConst<N, M>* __restrict__ g, ModelConst<N, M>& s) {
