@@ -42,6 +42,13 @@ KS_DEV void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "me
 KS_DEV void cp_async4(void* sdst, const void* gsrc) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" :: "r"(smem_addr(sdst)), "l"(gsrc) : "memory");
 }
+// 16-byte asynchronous copies (both addresses 16-byte aligned), not kept in L1.
+KS_DEV void cp_async16(void* sdst, const void* gsrc) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_addr(sdst)), "l"(gsrc) : "memory");
+}
+KS_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>
+KS_DEV void cp_async_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(LEFT) : "memory"); }
 KS_DEV void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 KS_DEV void mbar_init(uint64_t* m, uint32_t count) {

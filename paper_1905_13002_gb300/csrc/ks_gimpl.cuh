@@ -102,7 +102,8 @@ struct GImpl {
                      const uint32_t* gate = nullptr) {
         grp::GBuf fb, sb;
         buffers(ws, L, fb, sb);
-        constexpr int smem = SM::BYTES;
+        constexpr int smem = grp::GSmem<N, M, NW, TV && grp::Stage<N, M>::on>::BYTES;   // reduce, filter's apply
+        constexpr int asmem = SM::BYTES;                                               // smoother's apply
         constexpr int SW = grp::gspine_warps<N>();
         constexpr int ssmem = grp::GSpineSmem<N, SW>::BYTES;
         constexpr int SG = grp::GSpineSmem<N, SW>::NG;          // tiles per spine block
@@ -136,7 +137,7 @@ struct GImpl {
             auto kr = grp::gsmoother_reduce_kernel<N, M, NW, CH, SEG, TV>;
             auto ks = grp::gspine_smoother_kernel<N, SW>;
             auto ka = grp::gsmoother_apply_kernel<N, M, NW, CH>;
-            static const bool ok = allow_smem(kr, smem) && allow_smem(ks, ssmem) && allow_smem(ka, smem);
+            static const bool ok = allow_smem(kr, smem) && allow_smem(ks, ssmem) && allow_smem(ka, asmem);
             if (!ok) return KS_ECUDA;
             rc = launch_gated(kr, L.nts, NW * 32, smem, st, gate,
                               mconst(ws, L), fm, fc, L.T, sb, stat, segs);
@@ -151,7 +152,7 @@ struct GImpl {
                 src = dst;
                 dst = t;
             }
-            if ((rc = launch_gated(ka, L.nts, NW * 32, smem, st, gate, L.T, sm, sc, sb, src, stat))) return rc;
+            if ((rc = launch_gated(ka, L.nts, NW * 32, asmem, st, gate, L.T, sm, sc, sb, src, stat))) return rc;
         }
         return KS_OK;
     }
@@ -225,7 +226,7 @@ struct GImpl {
     }
 
     // Time-varying model: per-step constants (prep_kernel for step 0 with its
-    // FP64 k = 1 element, tv_const_kernel for the rest) after the elements
+    // FP64 k = 1 element, grp::tv_const_kernel for the rest) after the elements
     // region, read by the scans through a per-step Cursor.
     static size_t tv_offset(int64_t T) { return align_up(layout(T).bytes_elements, 256); }
     static size_t tv_bytes(int64_t T) { return tv_offset(T) + sizeof(ModelConst<N, M>) * (size_t)T; }
@@ -262,9 +263,9 @@ struct GImpl {
             if ((rc = launch_status())) return rc;
         }
         if (T > 1) {
-            const int blocks = (int)std::min<int64_t>((T + 127) / 128, 152 * 8);
-            tv_const_kernel<N, M><<<blocks, 128, 0, st>>>(tv, T, tvc, status(ws));
-            if ((rc = launch_status())) return rc;
+            constexpr int nt = grp::kTvThreads<N>, per = nt / grp::Grp<N>::GS;
+            const int blocks = (int)std::min<int64_t>((T - 1 + per - 1) / per, 152 * 16);
+            if ((rc = launch_pdl(grp::tv_const_kernel<N, M>, blocks, nt, 0, st, tv, T, tvc, status(ws)))) return rc;
         }
         if (ev && ev[1] && record_event(ev[1], st) != cudaSuccess) return KS_ECUDA;
         if ((rc = scans<false, true>(ws, L, y, fm, fc, sm, sc, Segs<N, M>{tvc, nullptr, 1}, st, ev, true,
