@@ -134,28 +134,6 @@ def tv_bytes_per_step(nx: int, ny: int) -> dict:
             "smoother": post + trans + post}
 
 
-def tensor_flops_per_step(N: int, M: int) -> dict:
-    """Algorithmic (FP32-equivalent, FMA = 2) flops per step of the dense
-    products the nx >= 32 kernels run on the tensor cores.  Forward scan: the
-    block fold of a measurement element (3 N^3 and 6 N^2 M products) and its
-    application to the running posterior (2 N^3, 4 N^2 M).  Reverse scan:
-    the Lemma 5 element (4 N^3), its block fold (3 N^3) and its application
-    (2 N^3).  The pivoted inverses (CUDA cores) and the tile-level combines are
-    not counted."""
-    return {"filter": 2 * (5 * N ** 3 + 10 * N * N * M), "smoother": 2 * 9 * N ** 3}
-
-
-def tf32_peak():
-    """Dense TF32 tensor peak of this GPU: the measured bf16 GEMM peak times
-    the nominal TF32 / bf16 ratio (1.1 / 2.25 PFLOP/s)."""
-    p = os.path.join(ROOT, "MEASURED_PEAKS.json")
-    if os.path.exists(p):
-        with open(p) as f:
-            d = json.load(f)
-        return float(d["bf16_tflops"]) * 1.1 / 2.25, "measured bf16 GEMM x nominal TF32/bf16 (1.1/2.25)"
-    return 1900.0 * 1.1 / 2.25, "fallback bf16 1.9 PFLOP/s x nominal TF32/bf16 (1.1/2.25)"
-
-
 # ---------------------------------------------------------------- clocks
 class ClockSampler:
     FIELDS = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
@@ -208,6 +186,8 @@ class ClockSampler:
 
 
 # ---------------------------------------------------------------- CPU oracle
+
+
 def output_errors(got, ref) -> dict:
     """Errors of the GPU outputs (fmean, fcov, smean, scov as float arrays)
     against the oracle's FP64 ones, max over steps: normwise relative
@@ -362,15 +342,24 @@ def block_length(ks, nx: int, T: int) -> dict:
 
 
 def launches_per_call(nx: int, T: int) -> int:
-    """Kernels one ks_smooth call launches: nx <= 6: preparation, forward scan,
-    its refinement retry (returns at once unless needed), reverse scan;
-    nx = 32: preparation, then per scan a reduce, one spine launch per
-    Kogge-Stone level over the tiles of 3 chains x 72 steps, and an apply."""
+    """Kernels one ks_smooth call launches: nx <= 6: preparation with the
+    settled plan, settled path, forward and reverse scan (both return at once
+    unless the model is unsettled; time-varying: preparation, forward scan, its
+    refinement retry, reverse scan); nx = 32: preparation, then per scan a
+    reduce, one spine launch per Kogge-Stone level over the tiles of 3 chains x
+    72 steps, and an apply (settled_launches: what the settled path adds)."""
     if nx <= 6:
         return 4
     tiles = -(-T // (3 * 72))
     levels = (tiles - 1).bit_length() if tiles > 1 else 0
     return 1 + 2 * (2 + levels)
+
+
+def settled_launches(nx: int, T: int) -> int:
+    """Further kernels of a time-invariant ks_smooth call at nx = 32: from 256
+    steps on the settled path's rows, forward and reverse kernels stand before
+    the scans."""
+    return 3 if nx == 32 and T >= 256 else 0
 
 
 def run_single(args, rank, world, local, mode):
@@ -539,13 +528,12 @@ def run_single(args, rank, world, local, mode):
     if tv:
         roof = tv_roofline(nx, ny, T, hbm, which, {"elements": statistics.mean(kel), "filter": statistics.mean(kf),
                                                    "smoother": statistics.mean(ksm)})
-    bps = bytes_per_step(nx, ny)
-    fps = flops_per_step(nx, ny, fused_smoothing=nx <= 6,
-                         block_fold=nx <= 6 and not tv and ks.chunk_fold(nx, T) == 1)
-    kernels = {"filter": statistics.mean(kf), "smoother": statistics.mean(ksm)}
     if not tv:
-        roof = scan_roofline(nx, ny, T, hbm, which, kernels, bps, fps)
-        roof["prep_ms"] = round(statistics.mean(kel), 4)   # model constants (and block-fold coefficients)
+        # the settled path writes all four outputs between the first two
+        # events; after it come the scans' launches, closed unless needed
+        roof = settled_roofline(nx, ny, T, hbm, which, {"settled": statistics.mean(kf),
+                                                        "closed_smoother_scan": statistics.mean(ksm)})
+        roof["prep_ms"] = round(statistics.mean(kel), 4)   # model constants and the settled plan
 
     # the batched workload beside it (the metric's "batched FP32 scan vs plain
     # scan"): one mixed-size launch per scan, and the plain per-sequence scan
@@ -571,7 +559,7 @@ def run_single(args, rank, world, local, mode):
                       "block_length": block_length(ks, nx, T),
                       "l2": "flushed between timed steps (256 MiB memset outside the events)"},
            "clocks": {k: clk[k] for k in ("sm_mhz", "sm_max_mhz", "reasons")},
-           "gpu_launches": 2 * launches_per_call(nx, T) * args.steps, "latency": lat, "e2e": e2e, "roofline": roof}
+           "gpu_launches": 2 * (launches_per_call(nx, T) + (0 if tv else settled_launches(nx, T))) * args.steps, "latency": lat, "e2e": e2e, "roofline": roof}
     if world == 1 and not args.no_cpu_baseline:
         out["cpu_baseline"] = cpu_oracle_rate(seq, args.cpu_seconds, host_out)
         out["max_err"] = out["cpu_baseline"].pop("_max_err")
@@ -597,58 +585,31 @@ def tv_roofline(nx, ny, T, hbm, which, kernels):
             "gbs_by_kernel": {k: round(bps[k] * T / (v / 1e3) / 1e9, 1) for k, v in kernels.items()}}
 
 
-def scan_roofline(nx, ny, T, hbm, which, kernels, bps, fps):
-    """Time-invariant scans: the dominant kernel against the ALU, HBM or
-    tensor roof, whichever its work model reaches first."""
-    dom = max(kernels, key=kernels.get)
-    dur_s = kernels[dom] / 1e3
-    gbs = bps[dom] * T / dur_s / 1e9
-    alu_peak = NUM_SMS * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
-    tfl = fps[dom] * T / dur_s / 1e12
-    kname = ({"filter": "filter_scan_kernel", "smoother": "smoother_scan_kernel"} if nx <= 6 else
-             {"filter": "tfilter_reduce+spine+apply", "smoother": "tsmoother_reduce+spine+apply"} if nx >= 32 else
-             {"filter": "gfilter_reduce+spine+apply", "smoother": "gsmoother_reduce+spine+apply"})[dom]
-    traffic = recorded_traffic(kname, T)
-    if nx >= 32:
-        tpeak, tsrc = tf32_peak()
-        tfs = tensor_flops_per_step(nx, ny)[dom]
-        ttf = tfs * T / dur_s / 1e12
-        roof = {"bound": "tensor", "achieved": ttf, "peak": tpeak, "unit": "TFLOP/s", "frac": ttf / tpeak,
-                "traffic": traffic, "kernel": kname, "peak_source": tsrc, "ms_per_launch": kernels[dom],
-                "split": "3xTF32: 3 TF32 mma per FP32 product, so the tensor pipe issues 3x achieved",
-                "tensor_flops_per_step": tfs, "hbm_frac": gbs / hbm, "bytes_per_step": bps[dom],
-                "kernels_ms": {k: round(v, 4) for k, v in kernels.items()}}
-    elif tfl / alu_peak >= gbs / hbm:
-        roof = {"bound": "alu", "achieved": tfl, "peak": alu_peak, "unit": "TFLOP/s",
-                "frac": tfl / alu_peak, "traffic": traffic}
-    else:
-        roof = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s",
-                "frac": gbs / hbm, "traffic": traffic}
-    if nx < 32:
-        roof.update({"kernel": kname, "peak_source": which if roof["bound"] == "hbm" else
-                     "152 SMs x 128 FP32 lanes x 2 x 2070 MHz",
-                     "ms_per_launch": kernels[dom], "hbm_frac": gbs / hbm, "alu_frac": tfl / alu_peak,
-                     "bytes_per_step": bps[dom], "flops_per_step": fps[dom],
-                     "kernels_ms": {k: round(v, 4) for k, v in kernels.items()}})
-
-    return roof
+def settled_roofline(nx, ny, T, hbm, which, kernels):
+    """A time-invariant call: each measurement read once, each posterior (mean
+    and covariance, filtered and smoothed) written once, against HBM."""
+    bps = 4 * ny + 2 * 4 * (nx + nx * nx)
+    ms = sum(kernels.values())
+    gbs = bps * T / (ms / 1e3) / 1e9
+    kname = "steady_kernel" if nx <= 8 else "rows32+forward32+reverse32"
+    return {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm,
+            "traffic": recorded_traffic(kname, T), "kernel": kname, "peak_source": which, "ms_per_launch": ms,
+            "hbm_frac": gbs / hbm, "bytes_per_step": bps,
+            "kernels_ms": {k: round(v, 4) for k, v in kernels.items()}}
 
 
 # ---------------------------------------------------------------- discrete-state workload
 def hmm_work_per_step(K: int) -> tuple[dict, dict]:
     """(flops, algorithmic DRAM bytes) per step of the two HMM scans (FP32,
     FMA = 2).  Forward: the fold of the step element ((f Pi) then the
-    likelihood scaling and row normalisation), its application to the running
-    marginal, the step's Definition 2 element from that marginal and its fold
-    into the thread's smoothing aggregate; reads lik, writes filt and loglik.
-    Reverse: the Definition 2 element and its application; reads filt, writes
-    smooth.  Tile-level combines are not counted."""
+    likelihood scaling and row normalisation) and its application to the
+    running marginal; reads lik, writes filt and loglik.  Reverse: beta one
+    step back (Pi (l . beta)) and filt . beta normalised; reads lik and filt,
+    writes smooth.  Tile-level combines are not counted."""
     fold = 2 * K ** 3 + 3 * K * K + 2 * K
     adv = 2 * K * K + 3 * K
-    sel = 2 * K * K + K
-    smul = 2 * K ** 3
-    flops = {"filter": fold + adv + sel + smul, "smoother": sel + 2 * K * K}
-    nbytes = {"filter": 4 * K + 4 * K + 4, "smoother": 4 * K + 4 * K}
+    flops = {"filter": fold + adv, "smoother": 2 * K * K + 6 * K}
+    nbytes = {"filter": 4 * K + 4 * K + 4, "smoother": 12 * K}
     return flops, nbytes
 
 
@@ -742,11 +703,12 @@ def run_hmm(args, rank, world, local):
            "d2h_bytes_per_step": int((filt_h.numel() + smooth_h.numel() + ll_h.numel()) * 4)}
 
     flops, nbytes = hmm_work_per_step(K)
-    if K <= 8:
+    if K <= 4:
         launches_per_step = 3
-    else:   # prep, then per scan a reduce, ceil(log2(tiles)) spine levels and an apply
-        tiles = -(-T // (64 * 128 // K))    # 64 steps per chain, 128 / K chains per tile
-        launches_per_step = 1 + 2 * (2 + max(0, math.ceil(math.log2(tiles))))
+    else:   # prep, reduce, ceil(log2(tiles)) spine levels of both directions, two applies
+        ch = 32 if T < 128 * 1024 else 128 if K == 8 else 64
+        tiles = -(-T // (ch * (128 // K * (1 if K == 8 else 2))))
+        launches_per_step = 4 + max(0, math.ceil(math.log2(tiles)))
     kernels = {"filter": kf, "smoother": ksm}
     dom = max(kernels, key=kernels.get)
     dur_s = kernels[dom] / 1e3
@@ -758,7 +720,7 @@ def run_hmm(args, rank, world, local):
             if tfl / alu_peak >= gbs / hbm else
             {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm})
     roof.update({"traffic": recorded_traffic("hmm:" + dom, T) if K == 8 else None,
-                 "kernel": f"hmm_{dom}_kernel<{K}>" if K <= 8 else f"hmmw {dom} reduce+spine+apply (K={K})",
+                 "kernel": f"hmm_{dom}_kernel<{K}>" if K <= 4 else f"hmmw {dom} reduce+spine+apply (K={K})",
                  "peak_source": "152 SMs x 128 FP32 lanes x 2 x 2070 MHz" if roof["bound"] == "alu" else which,
                  "ms_per_launch": kernels[dom], "alu_frac": tfl / alu_peak, "hbm_frac": gbs / hbm,
                  "flops_per_step": flops[dom], "bytes_per_step": nbytes[dom],
@@ -897,12 +859,12 @@ def measure_batched(args, rank, world, dev, full: bool) -> dict:
     res = {"value": total * world / (ms / 1e3), "unit": UNIT, "ms_per_step": ms,
            "latency": {"p50_ms": float(np.percentile(times, 50)), "p99_ms": float(np.percentile(times, 99))},
            "clocks": {k: clk[k] for k in ("sm_mhz", "sm_max_mhz", "reasons")},
-           "gpu_launches": 4 * args.steps,
+           "gpu_launches": (3 + len(groups)) * args.steps,
            "config": {"workload": "batched: log-uniform T in [256,16384], nx in {2,4,6} Wiener-velocity, "
                                   "q~U[0.5,2], R=rI r~U[0.1,1]", "sequences": len(seqs), "total_steps": total,
                       "groups": [{"nx": g["nx"], "B": g["B"], "T": g["T"]} for g in groups],
-                      "launch": "ks_smooth_batched: prep + forward + refinement retry + reverse launches over "
-                                "all sizes (CUDA graph)",
+                      "launch": "ks_smooth_batched: plans over all sizes, the settled path one size after "
+                                "another, closed forward and reverse scans (CUDA graph)",
                       "block_length": block_length(ks, 0, total),
                       "l2": "flushed between timed steps (256 MiB memset outside the events)"}}
 
@@ -928,25 +890,13 @@ def measure_batched(args, rank, world, dev, full: bool) -> dict:
                          "how": "ks_smooth once per sequence, sequentially on one stream"}
     del plain
 
-    # roofline over the whole step: algorithmic bytes and flops of all groups
+    # roofline over the whole step: algorithmic bytes of all groups
     hbm, which = peaks()
-    nbytes = nflops = 0
-    for g in groups:
-        bps = bytes_per_step(g["nx"], g["nx"] // 2)
-        fps = flops_per_step(g["nx"], g["nx"] // 2, block_fold=ks.chunk_fold(0, total) == 1)
-        nbytes += (bps["filter"] + bps["smoother"]) * g["T"]
-        nflops += (fps["filter"] + fps["smoother"]) * g["T"]
-    dur = ms / 1e3
-    gbs = nbytes / dur / 1e9
-    tfl = nflops / dur / 1e12
-    alu_peak = NUM_SMS * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
-    if tfl / alu_peak >= gbs / hbm:
-        roof = {"bound": "alu", "achieved": tfl, "peak": alu_peak, "unit": "TFLOP/s", "frac": tfl / alu_peak}
-    else:
-        roof = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm}
-    roof.update({"traffic": None, "kernel": "whole step (mixed prep + forward + reverse launches)",
-                 "hbm_frac": gbs / hbm, "alu_frac": tfl / alu_peak,
-                 "peak_source": "152 SMs x 128 FP32 lanes x 2 x 2070 MHz" if roof["bound"] == "alu" else which})
+    nbytes = sum((4 * (g["nx"] // 2) + 2 * 4 * (g["nx"] + g["nx"] ** 2)) * g["T"] for g in groups)
+    gbs = nbytes / (ms / 1e3) / 1e9
+    roof = {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm, "hbm_frac": gbs / hbm,
+            "traffic": None, "kernel": "whole step (mixed plans, settled path per size, closed scans)",
+            "peak_source": which}
     res["roofline"] = roof
     if not full:
         return res

@@ -17,6 +17,11 @@
  * The scans use block-level elements (Section III-C): each thread folds a
  * contiguous block of steps, blocks are scanned within a thread block, and
  * thread blocks are chained by a decoupled look-back.
+ * The fused calls (ks_smooth, ks_smooth_batch, ks_smooth_batched) of a
+ * time-invariant model whose covariances settle within 128 steps take them in
+ * closed form and scan the means alone, in windows that need no look-back;
+ * the scans are launched behind it and return at once unless a model did not
+ * settle or a value was not finite.  Results agree to FP32 rounding.
  *
  * Conventions (all entry points)
  * ------------------------------
@@ -254,8 +259,8 @@ int ks_chunk_fold(int nx, int64_t T);
 
 /*
  * Batched end to end over sequences of different state sizes, in one
- * preparation, one forward-scan and one reverse-scan launch.  The sequences
- * come in G groups (1 <= G <= 3), one per state size, with distinct
+ * preparation, one settled-path launch per state size, and one forward- and
+ * one reverse-scan launch behind them.  The sequences come in G groups (1 <= G <= 3), one per state size, with distinct
  * (nx, ny) among (2, 1), (4, 2) and (6, 3) (others: KS_EUNSUPPORTED).  A
  * group is a segmented batch exactly as for ks_smooth_batch: its models
  * (ks_model_batch: nx, ny, B >= 1 sequences, per-sequence parameters and the
@@ -284,7 +289,9 @@ int ks_smooth_batched(int G, const ks_batch_group *groups, void *ws, size_t ws_b
  * ks_smooth with per-kernel timing: `events` points to 4 cudaEvent_t handles
  * (passed as void*; any may be NULL) that are recorded on `stream` before the
  * model preparation, before the forward scan kernel, between the two scans
- * and after the reverse scan kernel.  Otherwise identical to ks_smooth.
+ * and after the reverse scan kernel.  The settled path of a time-invariant
+ * model, filter and smoother, lies between the second and the third.
+ * Otherwise identical to ks_smooth.
  */
 int ks_smooth_traced(const ks_model *m, const float *y, int64_t T, void *ws, size_t ws_bytes,
                      float *fmean, float *fcov, float *smean, float *scov, void *stream,
@@ -304,7 +311,8 @@ int ks_status(void *ws, void *stream);
  * changed or until ks_workspace_init:
  *   wait_polls  polls a look-back wait makes before it gives up, records
  *               KS_ETIMEOUT for ks_status and goes on with an empty prefix
- *               (0: the default, about one second);
+ *               (0: the default, about one second); any other value also
+ *               keeps a fused call from the settled path (the scans run);
  *   first_tile  1 makes the forward scan of ks_smooth / ks_smooth_batch at
  *               nx <= 6 number its tiles from 1, so that tile 0 is never
  *               published and tile 1's wait must run out; 0 restores the

@@ -327,7 +327,10 @@ struct GImpl {
 // Steps per chain of the nx = 8 scans by length: a chain is one 8-lane group
 // and folds its steps one after another, so that at 32 steps a 20000-step call
 // is 157 warps on 152 SMs.  Shorter chains give more of them; long calls keep
-// 32 (fewer tiles for the spine's levels).
+// 32 (fewer tiles for the spine's levels).  Time-varying, 20011 steps: 880 us at
+// 32, 574 at 8 when the lines were drawn.  Either side of them since: 40001 steps
+// 417 us at 8, 410 at 16; 60001 steps 486 at 8, 452 at 16; 140001 steps 997 at 16,
+// 1035 at 32; 200001 steps 1295 at 16, 1309 at 32.
 struct GVariant {
     Layout (*layout)(int64_t T, int B);
     int (*smooth_scan)(const ks_model*, int64_t, const float*, const float*, void*, size_t, float*, float*,

@@ -6,26 +6,24 @@
 // enter only through their likelihoods lik[k][j] = p(y_k | x_k = j) (0-based
 // k here; step k + 1 of the paper).
 //
-// Elements, each thread holding whole elements in registers (K <= 8):
+// Elements, each thread holding whole elements in registers (K = 2, 4; the
+// lane-group form of ks_hmmw.cuh takes over from K = 8):
 //  * filtering element (f, g) of Definition 1: f row-stochastic,
 //    f[z*K + x] = f(x | z), and g kept as lg[z] = log g(z), so that the
 //    marginal likelihoods p(y_1:k) (Theorem 1) survive long prefixes;
-//  * smoothing element a of Definition 2: a[z*K + x] = a(x | z),
-//    row-stochastic.
+//  * the reverse scan's beta(z) = p(y_k+1:n | x_k = z), up to a factor: the
+//    smoothed marginal is filt . beta over its sum (Theorem 2's suffix, without
+//    Definition 2's K x K elements).
 // The prefix of the filtering scan from step 1 has identical rows
 // p(x_k | y_1:k) and a constant g = p(y_1:k) (Theorem 1), so it is carried
-// as the state (p, L = log p(y_1:k)); the suffix of the smoothing scan to
-// step n has identical rows p(x_k | y_1:n) (Theorem 2), carried as s.
+// as the state (p, L = log p(y_1:k)).
 //
-// The per-step elements are never stored: with the likelihood row scaled to
-// a maximum of 1 (its log maximum added to lg), the step-k element is
+// The per-step elements are never stored: with the likelihood row scaled by a
+// power of two to a maximum in [1, 2), the step-k element is
 //   f_k(x | z) = Pi[z][x] l(x) / c(z),  c(z) = sum_x Pi[z][x] l(x),  g_k = c,
-// and folding it into a running aggregate (f, lg) is
-//   f'(x | z) = (f Pi)[z][x] l(x) / r(z),  r(z) = sum_x (f Pi)[z][x] l(x),
-//   lg'(z) = lg(z) + log r(z) + log max lik[k]
-// (Definition 1 with g_k f_k = Pi diag(l)).  Smoothing elements
-//   a_k(x | z) = p_k(x) Pi[x][z] / sum_x' p_k(x') Pi[x'][z]
-// are built from each filtered marginal p_k as the forward scan produces it.
+// and folding it into a running aggregate keeps (f Pi) . l at row sums in
+// [1, 2) by powers of two, whose exponents are added up; log g is formed once
+// at the fold's end (Definition 1 with g_k f_k = Pi diag(l)).
 #pragma once
 
 #include "ks_scan.cuh"
@@ -54,12 +52,11 @@ struct SS {
     float pad[K % 2 == 0 ? 1 : 0];
 };
 
-// Model constants: the transition matrix, its transpose and the prior
-// predicted to step 1 (16-byte aligned: rows are read as float4).
+// Model constants: the transition matrix and the prior predicted to step 1
+// (16-byte aligned: rows are read as float4).
 template <int K>
 struct alignas(16) Const {
     float Pi[K * K];
-    float PiT[K * K];
     float q1[K];   // p(x_1) = (pi Pi)
     float pad[(4 - K % 4) % 4];
 };
@@ -430,7 +427,6 @@ __global__ void __launch_bounds__(64) hmm_prep_kernel(const float* __restrict__ 
         const float v = Pi[e];
         bad |= !(v >= 0.f) || !(v <= 3.0e38f);
         out->Pi[e] = v;
-        out->PiT[(e % K) * K + e / K] = v;
     }
     for (int e = t; e < (4 - K % 4) % 4; e += blockDim.x) out->pad[e] = 0.f;
     for (int x = t; x < K; x += blockDim.x) {

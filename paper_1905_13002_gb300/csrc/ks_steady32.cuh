@@ -28,7 +28,10 @@ namespace ks {
 constexpr int kS32Head = 128;       // rows with gains of their own
 constexpr int kS32Chunk = 32;       // rows of a chunk
 constexpr int kS32Back = 8;         // chunks that reach 256 rows
-constexpr int kS32MinT = 256;       // head and end rows apart; shorter sequences go through the scans
+// Head and end rows apart need 256 rows; shorter sequences go through the
+// scans.  At the line, 256 steps: 2262 us in the scans, 213 here; 65536
+// steps 3406 -> 350 us.
+constexpr int kS32MinT = 256;
 
 struct Plan32 {
     float F[1024], Ph[1024], PhT[1024], P32[1024], P32T[1024], Pf[1024], Ps[1024];
