@@ -258,7 +258,7 @@ def alloc_workspace(model: Model, T: int, purpose: int = KS_WS_SMOOTH, stream=No
 
 
 def _out(shape, like, out):
-    return like.new_empty(shape, dtype=torch.float32) if out is None else out
+    return torch.empty(shape, dtype=torch.float32, device=like.device) if out is None else out
 
 
 def smooth(model: Model, y: torch.Tensor, ws: torch.Tensor | None = None, *, fmean=None, fcov=None,
