@@ -359,10 +359,10 @@ KS_DEV void plan_block(char* dsm, int sg, const PlanArgs<N, M>& g) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(0xffffffffu, f, o));
         const float n = s.Hh[0];
+        // at every length: the head's closed forms hold for a fixed point P only
         const bool settled = s.settled != 0 && fmaxf(f, 1.f) * n * n <= kStCovTol;
-        const int64_t len = g.off ? g.off[sg + 1] - g.off[sg] : g.T;
         // wait settings of the look-back are a test's: it wants the scans
-        ok = s.ok != 0 && p.ok0 != 0 && p.ok1 != 0 && (len <= kStHead || settled) && g.status[HDR_WAIT] == 0u &&
+        ok = s.ok != 0 && p.ok0 != 0 && p.ok1 != 0 && settled && g.status[HDR_WAIT] == 0u &&
              g.status[HDR_FIRST_TILE] == 0u;
         if (lane == 0) out->ok = ok ? 1 : 0;
         if constexpr (FOLD) {
