@@ -44,16 +44,10 @@
 #pragma once
 
 #include "ks_scan.cuh"
+#include "ks_window.h"
 
 namespace ks {
 
-constexpr int kStNT = 128;                        // threads of a block = rows of the head
-constexpr int kStHead = 128;
-constexpr int kStCH = 16;                         // steps per thread of a window
-constexpr int kStWin = kStNT * kStCH;             // 2048 rows
-constexpr int kStHalo = 256;                      // rows before and after a window's own rows
-constexpr int kStOut = kStWin - 2 * kStHalo;      // rows of an inner window: 1536
-constexpr int kStFirst = kStWin - kStHalo;        // rows of a first window (it starts exactly): 1792
 constexpr int kStLev = 7;                         // doublings to 128 steps
 constexpr int kStPow = 5;                         // Phi^16 .. Phi^256
 static_assert(kStHead == 1 << kStLev && (kStCH << (kStPow - 1)) == kStHalo, "levels");

@@ -992,24 +992,20 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
     }
     const int64_t j = slot - first;
     const int len = (int)(a1 - a0);
-    const int nt = len <= kStHead + kStWin ? 1 : 1 + (len - kStHead - kStWin + kStOut - 1) / kStOut;
-    if (j >= nt) {
+    if (j >= steady_windows(len)) {
         pdl_wait();
         return;
     }
-    const bool head = j == 0, last = j == nt - 1;
-    // own rows [o0, o1) of the window [w0, w1), as rows of the sequence
-    const int o0 = head ? kStHead : kStHead + kStFirst + (int)(j - 1) * kStOut;
-    const int w0 = head ? kStHead : o0 - kStHalo;
-    const int o1 = last ? len : (head ? kStHead + kStFirst : o0 + kStOut);
-    const int w1 = min(len, w0 + kStWin);
+    const StWindow win = steady_window(len, (int)j);
+    const bool head = win.head, last = win.last;
+    const int o0 = win.o0, o1 = win.o1, w0 = win.w0, rows = win.rows;
     const float* y = g.y + a0 * M;
     float *fm = g.fm + a0 * N, *fc = g.fc + a0 * NN;
     float* so = g.sm ? g.sm + a0 * N : nullptr;
     float* sc = g.sc ? g.sc + a0 * NN : nullptr;
     {   // the measurements on their way, one thread's 16 steps side by side, before the plan is there
         const float* src = y + (int64_t)w0 * M;
-        const int n = (w1 - w0) * M;
+        const int n = rows * M;
         for (int i = tid; i < n; i += kStNT) {
             const int w = i / M;
             cp_async4(sm.ys + (w / kStCH) * YP + (w % kStCH) * M + i % M, src + i);
@@ -1058,10 +1054,10 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
     if (head || (last && sc != nullptr)) head_covs<N, M>(sm, head, last, len, o0, fc, sc, bad);
     if (head) head_forward<N, M>(sm, y, len, fm, bad);
     else if (last) __syncthreads();   // the tables are read, the window may take their place
-    if (w1 > w0) {
+    if (rows > 0) {
         cp_async_wait_all();
         __syncthreads();
-        const int c0 = w0 + tid * kStCH, cnt = min(max(w1 - c0, 0), kStCH);
+        const int c0 = tid * kStCH, cnt = steady_chunk(rows, c0);   // the thread's chunk
         float* yc = sm.ys + tid * YP;
         float* mc = sm.ms + tid * MP;
         float xg[N], x[N], v[N];
@@ -1095,7 +1091,7 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
                 load_y(yc + i * M, yv);
                 mean_step<N, M>(F, u, H, d, K, yv, x, e);
             }
-            if (c0 + kStCH < w1) {
+            if (c0 + kStCH < rows) {
                 float xn[N];
                 load_y(yc + YP, yv);
                 lift<N, M>(pl.Lf, pl.d, yv, xn);
@@ -1189,7 +1185,7 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
                     l[a] = s;
                 }
             };
-            const int top = c0 + cnt == w1 ? cnt - 2 : cnt - 1;    // the window's last row keeps l = 0
+            const int top = c0 + cnt == rows ? cnt - 2 : cnt - 1;    // the window's last row keeps l = 0
 #pragma unroll
             for (int a = 0; a < N; ++a) x[a] = 0.f;
 #pragma unroll(N <= 4 ? 2 : 1)
@@ -1235,7 +1231,7 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
                 for (int a = 0; a < N; ++a) v[a] += z[a];
             }
             if (cnt > 0 && !last && !(pl.ndual * in_sd<N>(v, pl.sd) <= kStMeanTol)) bad |= FL_NEED;
-            if (c0 + cnt == w1) {                                  // the row after the window does not count
+            if (c0 + cnt == rows) {                                // the row after the window does not count
 #pragma unroll
                 for (int a = 0; a < N; ++a) v[a] = 0.f;
             }
