@@ -759,6 +759,8 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
         }
         __syncthreads();
         d = s.d[w][lane];
+        // chunk c + 8 leaves out what lies before chunk c, which only this block sees
+        if (c + kS32Back < nch && !(p.nphi * fabsf(d) * p.rsd[lane] <= kStMeanTol)) bad = true;
     } else if (c < nch) {
         float m[kS32Back];
 #pragma unroll
@@ -907,7 +909,8 @@ __global__ void __launch_bounds__(256, 2) reverse32_kernel(Args32 g) {
             stage(s.eps[w], g.s.eps + r0 * M, cnt * M, lane);
             const int64_t fend = T - kS32Head;
             float l = enter(c);
-            if (c + kS32Back < nch && !(p.ndual * fabsf(l) * p.sd[lane] <= kStMeanTol)) bad = true;
+            // chunk c - 8 (the head before chunk 7) leaves out what enters here
+            if (nch > kS32Back && !(p.ndual * fabsf(l) * p.sd[lane] <= kStMeanTol)) bad = true;
             constexpr int AH = 4;                       // filtered means loaded ahead
             float mn[AH];
 #pragma unroll

@@ -1144,7 +1144,10 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
 #pragma unroll
             for (int a = 0; a < N; ++a) v[a] += z[a];
         }
-        if (cnt > 0 && !head && !(pl.nphi * in_sd<N>(v, pl.rsd) <= kStMeanTol)) bad |= FL_NEED;
+        // a neighbour leaves out what lies beyond its halo, which only this window sees (the
+        // first and the last one too, although their own outer ends are exact)
+        const bool alone = head && last;
+        if (cnt > 0 && !alone && !(pl.nphi * in_sd<N>(v, pl.rsd) <= kStMeanTol)) bad |= FL_NEED;
         // ---- pass 2: the means, and the innovations in the measurements' place
 #pragma unroll
         for (int a = 0; a < N; ++a) x[a] = xg[a] + v[a];
@@ -1230,7 +1233,7 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
 #pragma unroll
                 for (int a = 0; a < N; ++a) v[a] += z[a];
             }
-            if (cnt > 0 && !last && !(pl.ndual * in_sd<N>(v, pl.sd) <= kStMeanTol)) bad |= FL_NEED;
+            if (cnt > 0 && !alone && !(pl.ndual * in_sd<N>(v, pl.sd) <= kStMeanTol)) bad |= FL_NEED;
             if (c0 + cnt == rows) {                                // the row after the window does not count
 #pragma unroll
                 for (int a = 0; a < N; ++a) v[a] = 0.f;
