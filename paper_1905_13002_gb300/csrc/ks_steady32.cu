@@ -566,7 +566,8 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
         __syncthreads();
     }
     const float *Phk = s.Ph[cur], *Ok = s.O[cur];
-    // (I + L R)^-1 of two symmetric matrices into Mi
+    // (I + L R)^-1 of two symmetric matrices into Mi, its Skeel condition tested
+    // (see inverse_ixj)
     auto inverse_of = [&](const float* L, const float* R) {
         mprod<4, false, false>(L, R, s.Mx, w, lane);
         __syncthreads();
@@ -574,8 +575,12 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
         __syncthreads();
         if (w == 0) {
             bool ok = true;
-            const float cond = tc::gj_inverse<N>(s.Mx, s.Mi, vs, ok);
-            if (!(__all_sync(kAll, ok) && cond <= kRefineCond)) bad = true;
+            tc::gj_inverse<N>(s.Mx, s.Mi, vs, ok);
+            float e = 0.f, c = 0.f;
+            for (int q = 0; q < N; ++q) e += fabsf(s.Mx[lane * P + q]);
+            __syncwarp();
+            for (int q = 0; q < N; ++q) c = fmaf(fabsf(s.Mi[lane * P + q]), __shfl_sync(kAll, e, q), c);
+            if (!__all_sync(kAll, ok && c <= kHeadCond)) bad = true;
         }
         __syncthreads();
     };
@@ -635,15 +640,15 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
         __syncthreads();
     }
     if (g.sc != nullptr) {
-        // smoothed head row: P_k - P_k (I + O_128 D_k)^-1 O_128 P_k
+        // smoothed head row: (I - P O_128) (I + D_k O_128)^-1 P_k
         load32(s.X, p.OW[7], t, kRowNT);
         __syncthreads();
-        inverse_of(s.X, s.D);
-        mprod<4, false, false>(s.Mi, s.X, s.Y, w, lane);
+        inverse_of(s.D, s.X);
+        mprod<4, false, false>(s.Mi, s.Pk, s.Y, w, lane);
         __syncthreads();
-        mprod<4, false, false>(s.Pk, s.Y, s.Mx, w, lane);
+        mprod<4, false, false>(s.X, s.Y, s.Mx, w, lane);
         __syncthreads();
-        mprod<4, false, false>(s.Mx, s.Pk, s.Mi, w, lane, s.Pk, -1.f);
+        mprod<4, false, false>(s.Pf, s.Mx, s.Mi, w, lane, s.Y, -1.f);
         __syncthreads();
         symmetrise(s.Mi, t, kRowNT);
         __syncthreads();

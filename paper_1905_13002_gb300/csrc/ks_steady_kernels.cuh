@@ -398,22 +398,42 @@ struct SteadySmem {
     static_assert(kStHead * (N * N + SY) <= kStNT * MP && SY <= N * M + N, "the tables fit");
 };
 
-// X <- A (I + X J)^-1 X A^T (X, J symmetric).
+// Mi = (I + X J)^-1 (X, J symmetric).  What it may cost is told by its Skeel
+// condition max |Mi| |I + X J| 1, which the scale of a row does not enter: a prior
+// that is wide along a coordinate (an unknown velocity, say) makes rows large
+// and loses nothing (30 for a Wiener velocity model with P_0 = 1e5 I, whose 1-norm
+// condition is 1e5), one that is wide across coordinates loses about that many
+// ulps.  Beyond kHeadCond the scans are as good.
+constexpr float kHeadCond = 256.f;
 template <int N>
-KS_DEV void congruence(float (&X)[sym_size(N)], const float* __restrict__ A, const float* __restrict__ J, Flags& bad) {
-    float Mx[N][N], Mi[N][N];
+KS_DEV void inverse_ixj(const float (&X)[sym_size(N)], const float (&J)[sym_size(N)], float (&Mi)[N][N], Flags& bad) {
+    float Mx[N][N], e[N];
 #pragma unroll
-    for (int a = 0; a < N; ++a)
+    for (int a = 0; a < N; ++a) {
+        e[a] = 0.f;
 #pragma unroll
         for (int b = 0; b < N; ++b) {
             float s = (a == b) ? 1.f : 0.f;
 #pragma unroll
-            for (int c = 0; c < N; ++c) s = fmaf(X[sidx(a, c)], J[sidx(c, b)], s);
+            for (int l = 0; l < N; ++l) s = fmaf(X[sidx(a, l)], J[sidx(l, b)], s);
             Mx[a][b] = s;
+            e[a] += fabsf(s);
         }
-    const float nm = norm1<N>(Mx);
-    if (!inverse_pp<N>(Mx, Mi)) bad |= FL_BAD;
-    if (!(nm * norm1<N>(Mi) <= kRefineCond)) bad |= FL_NEED;
+    }
+    bool ok = inverse_pp<N>(Mx, Mi);
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+        float s = 0.f;
+#pragma unroll
+        for (int b = 0; b < N; ++b) s = fmaf(fabsf(Mi[a][b]), e[b], s);
+        ok = ok && s <= kHeadCond;
+    }
+    if (!ok) bad |= FL_NEED;
+}
+
+// X <- A Mi X A^T with Mi = (I + X J)^-1 (Mi X is symmetric).
+template <int N>
+KS_DEV void congruence(float (&X)[sym_size(N)], const float* __restrict__ A, const float (&Mi)[N][N]) {
     float W[sym_size(N)];
 #pragma unroll
     for (int a = 0; a < N; ++a)
@@ -440,6 +460,38 @@ KS_DEV void congruence(float (&X)[sym_size(N)], const float* __restrict__ A, con
 #pragma unroll
             for (int c = 0; c < N; ++c) s = fmaf(y[c], A[b * N + c], s);
             X[sidx(a, b)] = s;
+        }
+    }
+}
+
+// The smoothed covariance (I - P O) Mi P_k of a row, Mi = (I + D_k O)^-1, to dst.
+template <int N>
+KS_DEV void smoothed_cov(const float (&Pk)[sym_size(N)], const float (&Mi)[N][N], const float (&O)[sym_size(N)],
+                         const float* __restrict__ P, float* __restrict__ dst) {
+#pragma unroll
+    for (int b = 0; b < N; ++b) {
+        float w[N], o[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            float s = 0.f;
+#pragma unroll
+            for (int c = 0; c < N; ++c) s = fmaf(Mi[a][c], Pk[sidx(c, b)], s);
+            w[a] = s;
+        }
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            float s = 0.f;
+#pragma unroll
+            for (int c = 0; c < N; ++c) s = fmaf(O[sidx(a, c)], w[c], s);
+            o[a] = s;
+        }
+#pragma unroll
+        for (int a = b; a < N; ++a) {
+            float s = w[a];
+#pragma unroll
+            for (int c = 0; c < N; ++c) s = fmaf(-P[a * N + c], o[c], s);
+            dst[a * N + b] = s;
+            if (a != b) dst[b * N + a] = s;
         }
     }
 }
@@ -622,9 +674,9 @@ KS_DEV void copy_rows(const float* __restrict__ ms, int w0, int r0, int r1, floa
 // last 128 rows after the head): the tables Phi^n, O_n for n = 1..128, thread
 // n - 1 its n, rows h+1..2h from the rows before by
 //     Phi^{h+m} = Phi^m Phi^h,  O_{h+m} = O_h + (Phi^h)^T O_m Phi^h,
-// then D_k and the smoothed rows by one copy of the congruence (a block runs
-// this code once a launch, and fetching it is a large part of its time).  The
-// rows' P_k are left in sm.hd for head_forward.
+// then D_k and the smoothed rows by one copy of the inverse (a block runs this
+// code once a launch, and fetching it is a large part of its time).  The rows'
+// P_k are left in sm.hd for head_forward.
 template <int N, int M>
 KS_DEV void head_covs(SteadySmem<N, M>& sm, bool head, bool tail, int len, int o0, float* __restrict__ fc,
                       float* __restrict__ sc, Flags& bad) {
@@ -693,7 +745,7 @@ KS_DEV void head_covs(SteadySmem<N, M>& sm, bool head, bool tail, int len, int o
         }
 #pragma unroll 1
     for (int it = 0; it < 3; ++it) {
-        float X[SY], A[NN], J[SY];
+        float X[SY], J[SY];
         bool run;
         int n = 0;                                         // later measurements of the row
         if (it == 0) {
@@ -706,14 +758,12 @@ KS_DEV void head_covs(SteadySmem<N, M>& sm, bool head, bool tail, int len, int o
             n = k;
         }
         if (run) {
+            const float* e = tab + max(k - 1, 0) * TS;
             if (it == 0) {
-                const float* e = tab + max(k - 1, 0) * TS;
 #pragma unroll
                 for (int i = 0; i < SY; ++i) X[i] = pl.C1[i] - P[i];
 #pragma unroll
-                for (int i = 0; i < NN; ++i) A[i] = k > 0 ? e[i] : (i / N == i % N ? 1.f : 0.f);
-#pragma unroll
-                for (int i = 0; i < SY; ++i) J[i] = k > 0 ? e[NN + i] : 0.f;
+                for (int i = 0; i < SY; ++i) J[i] = e[NN + i];
             } else {
                 const float* o = n >= kStHead ? pl.On : tab + max(n - 1, 0) * TS + NN;
                 if (it == 2) {
@@ -723,28 +773,21 @@ KS_DEV void head_covs(SteadySmem<N, M>& sm, bool head, bool tail, int len, int o
                         for (int c = 0; c <= a; ++c) { P[sidx(a, c)] = pl.Pf[a * N + c]; D[sidx(a, c)] = 0.f; }
                 }
 #pragma unroll
-                for (int i = 0; i < SY; ++i) X[i] = n > 0 ? o[i] : 0.f;
-#pragma unroll
-                for (int a = 0; a < N; ++a)
-#pragma unroll
-                    for (int c = 0; c < N; ++c) A[a * N + c] = P[sidx(a, c)];
-#pragma unroll
-                for (int i = 0; i < SY; ++i) J[i] = D[i];
+                for (int i = 0; i < SY; ++i) { X[i] = D[i]; J[i] = n > 0 ? o[i] : 0.f; }
             }
-            congruence<N>(X, A, J, bad);
+            float Mi[N][N];
+            inverse_ixj<N>(X, J, Mi, bad);
             if (it == 0) {
+                if (k > 0) {
+                    congruence<N>(X, e, Mi);
 #pragma unroll
-                for (int i = 0; i < SY; ++i) { D[i] = X[i]; P[i] += X[i]; }
-                if (k == 0) {
+                    for (int i = 0; i < SY; ++i) { D[i] = X[i]; P[i] += X[i]; }
+                } else {
 #pragma unroll
-                    for (int i = 0; i < SY; ++i) P[i] = pl.C1[i];
+                    for (int i = 0; i < SY; ++i) { D[i] = X[i]; P[i] = pl.C1[i]; }
                 }
             } else {
-                float* dst = sc + (int64_t)(it == 1 ? k : len - 1 - k) * NN;
-#pragma unroll
-                for (int a = 0; a < N; ++a)
-#pragma unroll
-                    for (int c = 0; c < N; ++c) dst[a * N + c] = P[sidx(a, c)] - X[sidx(a, c)];
+                smoothed_cov<N>(P, Mi, J, pl.Pf, sc + (int64_t)(it == 1 ? k : len - 1 - k) * NN);
             }
         }
         if (it == 0 && head) {
