@@ -13,7 +13,7 @@
 //     (I - P O_n) (I + D_k O_n)^{-1} P_k: a product, since the difference from
 //     P_k loses the digits by which a wide prior's P_k exceeds it (Wiener
 //     velocity, q = r = 1, P_0 = 1000 I: 1.4e-4 off by that difference, 1.4e-5
-//     in the scans, below 1e-5 here).  The tables Phi^n, O_n of the first
+//     in the scans, 9e-7 here).  The tables Phi^n, O_n of the first
 //     128 n (the head of a sequence, and its end) take log2 levels of plain
 //     products and each row one inverse, with no scan over the rows;
 //   * after the head every covariance is P, every gain constant, and only the
@@ -65,8 +65,16 @@ constexpr float kStCovTol = 1.2e-7f;              // 2^-23
 constexpr float kStMeanTol = 2.4e-7f;             // 2^-22
 constexpr float kStPowTol = 9.5e-7f;              // 2^-20
 
+// From a start known far better than P (a known initial state), P + D_k would
+// leave P_k the rounding of P: below an eighth of it in some variance the head
+// takes P_1 through the element powers of the bits of k instead, sums of
+// non-negative parts, up to seven inverses for
+// one: 5 us more at nx = 4 (1000 steps, P_0 = 1e-6 I: 63 -> 68 us, the scans 90), and
+// the filtered variances 4.4e-6 -> 2.4e-7 off (q = r = 1, dt = 0.1, P_0 = 1e-4 I).
+constexpr float kStNarrow = 0.125f;
+
 template <int N, int M>
-struct alignas(16) SteadyPlan {
+struct alignas(16) SteadyCore {
     // what every window needs
     float F[N * N], Ph[N * N], H[M * N], K[N * M], B[N * M], Lf[N * M], u[N], d[M];
     float Pf[N * N], Ps[N * N];                   // settled filtered and smoothed covariance
@@ -76,6 +84,13 @@ struct alignas(16) SteadyPlan {
     // what the head and the end of a sequence need besides
     alignas(16) float W[sym_size(N)], On[sym_size(N)];   // F^T H^T S^-1 H F; O_128
     float Q[sym_size(N)], R[sym_size(M)], C1[sym_size(N)], b1[N];
+    int narrow;                                   // P_1 lies far below P somewhere: see kStNarrow
+};
+
+// A plan in memory: what the blocks copy, and the element powers a^(2^i).
+template <int N, int M>
+struct alignas(16) SteadyPlan : SteadyCore<N, M> {
+    float EA[kStLev][N * N], EC[kStLev][sym_size(N)], EJ[kStLev][sym_size(N)];
 };
 
 // Arguments of the preparation with the plan: one block per sequence.

@@ -246,6 +246,10 @@ __global__ void __launch_bounds__(kPlanNT) plan32_kernel(Args32 g) {
             bool ok = true;
             const float cond = tc::gj_inverse<N>(s.Mx, s.Mi, vs, ok);
             if (!(__all_sync(kAll, ok) && cond <= kRefineCond) && lane == 0) s.ok = 0;
+        } else {   // the powers, beside it
+            store32(out.EA[lev], A, t - 32, kPlanNT - 32);
+            store32(out.EC[lev], C, t - 32, kPlanNT - 32);
+            store32(out.EJ[lev], J, t - 32, kPlanNT - 32);
         }
         __syncthreads();
         if (grp == 0) mprod<8, false, false>(A, s.Mi, s.X, gw, lane);
@@ -490,9 +494,10 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
     const Plan32& p = *g.s.plan;
     pdl_trigger();
     pdl_wait();
-    bool okp;
+    bool okp, narrow;
     {   // the chain's checks, and the transient of P_1 (relative to P) after 128 steps
         float f = p.C1[lane * 33] * p.rsd[lane] * p.rsd[lane];
+        narrow = __any_sync(kAll, !(f >= kStNarrow));
         if (!(f < 1e18f)) f = 1e18f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(kAll, f, o));
@@ -584,24 +589,50 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
         }
         __syncthreads();
     };
-    for (int e = t; e < N * N; e += kRowNT) s.D[(e / N) * P + e % N] = p.C1[e] - s.Pf[(e / N) * P + e % N];
-    __syncthreads();
-    if (k > 0) {
-        inverse_of(s.D, Ok);
-        mprod<4, false, false>(s.Mi, s.D, s.X, w, lane);
-        __syncthreads();
-        mprod<4, false, false>(Phk, s.X, s.Y, w, lane);
-        __syncthreads();
-        mprod<4, false, true>(s.Y, Phk, s.D, w, lane);
-        __syncthreads();
-        symmetrise(s.D, t, kRowNT);
+    if (narrow) {   // P_1 through the element powers of the bits of k
+        load32(s.Pk, p.C1, t, kRowNT);
+#pragma unroll 1
+        for (int i = 0; i < 7; ++i) {
+            if (!(k >> i & 1)) continue;
+            load32(s.X, p.EJ[i], t, kRowNT);
+            load32(s.Y, p.EA[i], t, kRowNT);
+            load32(s.D, p.EC[i], t, kRowNT);
+            __syncthreads();
+            inverse_of(s.Pk, s.X);
+            mprod<4, false, false>(s.Mi, s.Pk, s.X, w, lane);
+            __syncthreads();
+            mprod<4, false, false>(s.Y, s.X, s.Mx, w, lane);
+            __syncthreads();
+            mprod<4, false, true>(s.Mx, s.Y, s.Pk, w, lane, s.D);
+            __syncthreads();
+            symmetrise(s.Pk, t, kRowNT);
+            __syncthreads();
+        }
         __syncthreads();
     }
     for (int e = t; e < N * N; e += kRowNT) {
-        const int a = e / N, b = e % N;
-        s.Pk[a * P + b] = k == 0 ? p.C1[e] : s.Pf[a * P + b] + s.D[a * P + b];
+        const int i = (e / N) * P + e % N;
+        s.D[i] = (narrow ? s.Pk[i] : p.C1[e]) - s.Pf[i];
     }
     __syncthreads();
+    if (!narrow) {
+        if (k > 0) {
+            inverse_of(s.D, Ok);
+            mprod<4, false, false>(s.Mi, s.D, s.X, w, lane);
+            __syncthreads();
+            mprod<4, false, false>(Phk, s.X, s.Y, w, lane);
+            __syncthreads();
+            mprod<4, false, true>(s.Y, Phk, s.D, w, lane);
+            __syncthreads();
+            symmetrise(s.D, t, kRowNT);
+            __syncthreads();
+        }
+        for (int e = t; e < N * N; e += kRowNT) {
+            const int i = (e / N) * P + e % N;
+            s.Pk[i] = k == 0 ? p.C1[e] : s.Pf[i] + s.D[i];
+        }
+        __syncthreads();
+    }
     store32(g.fc + (int64_t)k * 1024, s.Pk, t, kRowNT);
     // the next row's gain
     if (k + 1 < kS32Head) {

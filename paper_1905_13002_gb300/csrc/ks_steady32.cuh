@@ -36,6 +36,7 @@ constexpr int kS32MinT = 256;
 struct Plan32 {
     float F[1024], Ph[1024], PhT[1024], P32[1024], P32T[1024], Pf[1024], Ps[1024];
     float PW[7][1024], OW[8][1024];                 // Phi^(2^i), O_(2^i)
+    float EA[7][1024], EC[7][1024], EJ[7][1024];    // the element powers a^(2^i), for a narrow start (kStNarrow)
     float Q[1024], C1[1024];
     float H[256], K[256], B[256], Lf[256], HF[256], R[64], u[32], d[8], b1[32], sd[32], rsd[32];
     float nphi, ndual, nA;

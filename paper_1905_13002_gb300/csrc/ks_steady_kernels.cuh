@@ -164,6 +164,15 @@ KS_DEV void plan_body(PlanSmem<N, M>& s, const PS& p, const ModelConst<N, M>& mc
             float cond;
             const bool ok = warp_inverse<N>(s.Mx, s.Mi, lane, cond);
             if (lane == 0 && !(ok && cond <= kRefineCond)) s.ok = 0;
+        } else {   // the powers, beside it
+            for (int e = t - 32; e < NN; e += NT - 32) {
+                const int a = e / N, b = e % N;
+                out->EA[lev][e] = A[e];
+                if (b <= a) {
+                    out->EC[lev][sidx(a, b)] = C[e];
+                    out->EJ[lev][sidx(a, b)] = J[e];
+                }
+            }
         }
         chain_sync();
         for (int e = t; e < 3 * NN; e += NT) {
@@ -355,9 +364,11 @@ KS_DEV void plan_block(char* dsm, int sg, const PlanArgs<N, M>& g) {
     bool ok = false;
     if (warp == 0) {
         float f = lane < N ? mc.C1[sidx(lane, lane)] / (s.sd[lane] * s.sd[lane]) : 0.f;
+        const bool narrow = __any_sync(0xffffffffu, lane < N && !(f >= kStNarrow));
         if (!(f < 1e18f)) f = 1e18f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(0xffffffffu, f, o));
+        if (lane == 0) out->narrow = narrow ? 1 : 0;
         const float n = s.Hh[0];
         // at every length: the head's closed forms hold for a fixed point P only
         const bool settled = s.settled != 0 && fmaxf(f, 1.f) * n * n <= kStCovTol;
@@ -387,7 +398,7 @@ struct SteadySmem {
     static constexpr int PR = N * N * 4 >= 256 ? 16 : 4096 / (N * N * 4);   // rows of a covariance pattern
     float ms[kStNT * MP];                      // window means; before that the tables Phi^n, O_n
     float ys[kStNT * YP];                      // measurements, then innovations
-    SteadyPlan<N, M> pl;
+    SteadyCore<N, M> pl;
     alignas(128) float pat[2][PR * N * N];
     float hd[kStHead * (N * M + N)];           // head rows: P_k, then their gains and adjoint inputs
     float lam[kStHead * N];                    // means, then adjoint, of the head rows
@@ -601,7 +612,7 @@ KS_DEV void mean_step(const float* __restrict__ F, const float* __restrict__ u, 
 
 // Phi = F - K H F.
 template <int N, int M>
-KS_DEV void phi_of(const SteadyPlan<N, M>& pl, const float (&K)[N * M], float (&A)[N * N]) {
+KS_DEV void phi_of(const SteadyCore<N, M>& pl, const float (&K)[N * M], float (&A)[N * N]) {
     float HF[M][N];
 #pragma unroll
     for (int q = 0; q < M; ++q)
@@ -678,10 +689,10 @@ KS_DEV void copy_rows(const float* __restrict__ ms, int w0, int r0, int r1, floa
 // code once a launch, and fetching it is a large part of its time).  The rows'
 // P_k are left in sm.hd for head_forward.
 template <int N, int M>
-KS_DEV void head_covs(SteadySmem<N, M>& sm, bool head, bool tail, int len, int o0, float* __restrict__ fc,
-                      float* __restrict__ sc, Flags& bad) {
+KS_DEV void head_covs(SteadySmem<N, M>& sm, const SteadyPlan<N, M>* __restrict__ gp, bool head, bool tail, int len,
+                      int o0, float* __restrict__ fc, float* __restrict__ sc, Flags& bad) {
     constexpr int SY = sym_size(N), NN = N * N, TS = NN + SY;
-    const SteadyPlan<N, M>& pl = sm.pl;
+    const SteadyCore<N, M>& pl = sm.pl;
     const int k = threadIdx.x;
     const bool smooth = sc != nullptr;
     float* tab = sm.ms;                                    // entry n - 1: Phi^n, O_n
@@ -734,22 +745,32 @@ KS_DEV void head_covs(SteadySmem<N, M>& sm, bool head, bool tail, int len, int o
             __syncthreads();
         }
     }
-    // rounds: D_k of the head, its smoothed rows, the smoothed rows of the end
+    // rounds: D_k of the head, its smoothed rows, the smoothed rows of the end;
+    // from a narrow start, before these, P_1 through the powers of the bits of k
+    const bool narrow = head && pl.narrow != 0;
     float P[SY], D[SY];
 #pragma unroll
     for (int a = 0; a < N; ++a)
 #pragma unroll
         for (int c = 0; c <= a; ++c) {
-            P[sidx(a, c)] = pl.Pf[a * N + c];
+            P[sidx(a, c)] = narrow ? pl.C1[sidx(a, c)] : pl.Pf[a * N + c];
             D[sidx(a, c)] = 0.f;
         }
 #pragma unroll 1
-    for (int it = 0; it < 3; ++it) {
+    for (int it = narrow ? -kStLev : 0; it < 3; ++it) {
         float X[SY], J[SY];
         bool run;
         int n = 0;                                         // later measurements of the row
-        if (it == 0) {
-            run = head;
+        if (it < 0) {
+            run = (k >> (it + kStLev)) & 1;
+        } else if (it == 0) {
+            run = head && !narrow;
+            if (narrow) {
+#pragma unroll
+                for (int a = 0; a < N; ++a)
+#pragma unroll
+                    for (int c = 0; c <= a; ++c) D[sidx(a, c)] = P[sidx(a, c)] - pl.Pf[a * N + c];
+            }
         } else if (it == 1) {
             run = head && smooth && k < len;
             n = len - 1 - k;
@@ -758,12 +779,12 @@ KS_DEV void head_covs(SteadySmem<N, M>& sm, bool head, bool tail, int len, int o
             n = k;
         }
         if (run) {
-            const float* e = tab + max(k - 1, 0) * TS;
-            if (it == 0) {
+            const float* e = tab + max(k - 1, 0) * TS;     // Phi^k, O_k
+            const float* A = it < 0 ? gp->EA[it + kStLev] : e;
+            if (it <= 0) {
+                const float* j = it < 0 ? gp->EJ[it + kStLev] : e + NN;
 #pragma unroll
-                for (int i = 0; i < SY; ++i) X[i] = pl.C1[i] - P[i];
-#pragma unroll
-                for (int i = 0; i < SY; ++i) J[i] = e[NN + i];
+                for (int i = 0; i < SY; ++i) { X[i] = it < 0 ? P[i] : pl.C1[i] - P[i]; J[i] = j[i]; }
             } else {
                 const float* o = n >= kStHead ? pl.On : tab + max(n - 1, 0) * TS + NN;
                 if (it == 2) {
@@ -777,17 +798,18 @@ KS_DEV void head_covs(SteadySmem<N, M>& sm, bool head, bool tail, int len, int o
             }
             float Mi[N][N];
             inverse_ixj<N>(X, J, Mi, bad);
-            if (it == 0) {
-                if (k > 0) {
-                    congruence<N>(X, e, Mi);
-#pragma unroll
-                    for (int i = 0; i < SY; ++i) { D[i] = X[i]; P[i] += X[i]; }
-                } else {
-#pragma unroll
-                    for (int i = 0; i < SY; ++i) { D[i] = X[i]; P[i] = pl.C1[i]; }
-                }
-            } else {
+            if (it > 0) {
                 smoothed_cov<N>(P, Mi, J, pl.Pf, sc + (int64_t)(it == 1 ? k : len - 1 - k) * NN);
+            } else if (it == 0 && k == 0) {
+#pragma unroll
+                for (int i = 0; i < SY; ++i) { D[i] = X[i]; P[i] = pl.C1[i]; }
+            } else {
+                congruence<N>(X, A, Mi);
+#pragma unroll
+                for (int i = 0; i < SY; ++i) {
+                    D[i] = X[i];
+                    P[i] = X[i] + (it < 0 ? gp->EC[it + kStLev][i] : P[i]);
+                }
             }
         }
         if (it == 0 && head) {
@@ -812,7 +834,7 @@ template <int N, int M>
 KS_DEV void head_forward(SteadySmem<N, M>& sm, const float* __restrict__ y, int len, float* __restrict__ fm,
                          Flags& bad) {
     constexpr int SY = sym_size(N);
-    const SteadyPlan<N, M>& pl = sm.pl;
+    const SteadyCore<N, M>& pl = sm.pl;
     const int k = threadIdx.x, warp = k >> 5, lane = k & 31;
     const float* ptab = sm.hd;
     const bool on = k < len;
@@ -959,7 +981,7 @@ KS_DEV void head_forward(SteadySmem<N, M>& sm, const float* __restrict__ y, int 
 template <int N, int M>
 KS_DEV void head_reverse(SteadySmem<N, M>& sm, int len, const float* fm, const float* fc, float* __restrict__ smo,
                          Flags& bad) {
-    const SteadyPlan<N, M>& pl = sm.pl;
+    const SteadyCore<N, M>& pl = sm.pl;
     const int k = threadIdx.x, warp = k >> 5, lane = k & 31;
     float A[N * N], b[N], in[N], l[N];
 #pragma unroll
@@ -1061,14 +1083,14 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
         return;
     }
     {   // the plan (the head's part too for a head)
-        using Plan = SteadyPlan<N, M>;
-        const int n = (int)((head || last ? sizeof(Plan) : offsetof(Plan, W)) / 16);
+        using Core = SteadyCore<N, M>;
+        const int n = (int)((head || last ? sizeof(Core) : offsetof(Core, W)) / 16);
         const float4* src = reinterpret_cast<const float4*>(g.plan + b);
         float4* dst = reinterpret_cast<float4*>(&sm.pl);
         for (int i = tid; i < n; i += kStNT) dst[i] = src[i];
     }
     __syncthreads();
-    const SteadyPlan<N, M>& pl = sm.pl;
+    const SteadyCore<N, M>& pl = sm.pl;
     Flags bad = 0u;
     // ---- constant covariance rows: bulk copies of a pattern, in flight while the means are computed
     const int s1 = last ? max(o0, len - kStHead) : o1;         // smoothed rows that are settled: [o0, s1)
@@ -1094,7 +1116,7 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
         }
     };
     fill(0);
-    if (head || (last && sc != nullptr)) head_covs<N, M>(sm, head, last, len, o0, fc, sc, bad);
+    if (head || (last && sc != nullptr)) head_covs<N, M>(sm, g.plan + b, head, last, len, o0, fc, sc, bad);
     if (head) head_forward<N, M>(sm, y, len, fm, bad);
     else if (last) __syncthreads();   // the tables are read, the window may take their place
     if (rows > 0) {
