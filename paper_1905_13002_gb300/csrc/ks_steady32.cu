@@ -582,9 +582,19 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
             bool ok = true;
             tc::gj_inverse<N>(s.Mx, s.Mi, vs, ok);
             float e = 0.f, c = 0.f;
-            for (int q = 0; q < N; ++q) e += fabsf(s.Mx[lane * P + q]);
-            __syncwarp();
-            for (int q = 0; q < N; ++q) c = fmaf(fabsf(s.Mi[lane * P + q]), __shfl_sync(kAll, e, q), c);
+#pragma unroll
+            for (int q = 0; q < N; q += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(s.Mx + lane * P + q);
+                e += (fabsf(v.x) + fabsf(v.y)) + (fabsf(v.z) + fabsf(v.w));
+            }
+#pragma unroll
+            for (int q = 0; q < N; q += 4) {
+                const float4 v = *reinterpret_cast<const float4*>(s.Mi + lane * P + q);
+                c = fmaf(fabsf(v.x), __shfl_sync(kAll, e, q), c);
+                c = fmaf(fabsf(v.y), __shfl_sync(kAll, e, q + 1), c);
+                c = fmaf(fabsf(v.z), __shfl_sync(kAll, e, q + 2), c);
+                c = fmaf(fabsf(v.w), __shfl_sync(kAll, e, q + 3), c);
+            }
             if (!__all_sync(kAll, ok && c <= kHeadCond)) bad = true;
         }
         __syncthreads();

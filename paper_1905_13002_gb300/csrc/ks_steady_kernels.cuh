@@ -74,7 +74,7 @@ struct PlanSmem {
     float Mx[N * N], Mi[N * N], X[N * N], W[N * N], V[N * N], Y[N * N], Z[N * N];
     float HP[M * N], S[M * M], Si[M * M], Hh[M * M], Hi[M * M], K[N * M];
     float sd[N];
-    int ok, settled;
+    int ok, settled, narrow;
 };
 
 // Threads of the preparation with the plan: warps 0-3 the FP32 constants and
@@ -121,14 +121,14 @@ KS_DEV float dot_cc(const float* a, const float* b) {   // column . column (stri
     return s;
 }
 
-// The plan of one model, by the chain's threads, from the FP32 constants mc and
-// the inputs in shared memory.  One output entry per thread and stage; a
-// doubling combine is four stages (M, M^-1 by one warp, the three products
-// with M^-1, the outer products).
-template <int N, int M, class PS>
-KS_DEV void plan_body(PlanSmem<N, M>& s, const PS& p, const ModelConst<N, M>& mc, SteadyPlan<N, M>* __restrict__ out) {
+// The element of Lemma 3 doubled kStLev times, by the chain's threads, from the
+// FP32 constants mc; returns the buffer of the last one.  One output entry per
+// thread and stage; a doubling combine is four stages (M, M^-1 by one warp, the
+// three products with M^-1, the outer products).  powers: null, or where the
+// elements before each doubling go.
+template <int N, int M>
+KS_DEV int element_powers(PlanSmem<N, M>& s, const ModelConst<N, M>& mc, SteadyPlan<N, M>* __restrict__ powers) {
     constexpr int NN = N * N, NT = kChainThreads;
-    static_assert(NN <= 64 && N * M <= 32, "entries per warp of the single-warp stages");
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     for (int e = t; e < NN; e += NT) {
         const int a = e / N, b = e % N;
@@ -137,19 +137,8 @@ KS_DEV void plan_body(PlanSmem<N, M>& s, const PS& p, const ModelConst<N, M>& mc
         float j = 0.f;
         for (int q = 0; q < M; ++q) j = fmaf(mc.U[q * N + a], mc.U[q * N + b], j);
         s.J[0][e] = j;
-        out->F[e] = mc.F[e];
     }
-    for (int e = t; e < M * N; e += NT) out->H[e] = p.H[e / N][e % N];
-    for (int e = t; e < sym_size(N); e += NT) out->Q[e] = mc.Q[e];
-    for (int e = t; e < sym_size(M); e += NT) {
-        int a, b;
-        tri_rc(e, a, b);
-        out->R[e] = 0.5f * (p.R[a][b] + p.R[b][a]);
-    }
-    for (int e = t; e < N; e += NT) out->u[e] = mc.u[e];
-    for (int e = t; e < M; e += NT) out->d[e] = p.d[e];
     chain_sync();
-    // ---- element powers
     int cur = 0;
 #pragma unroll 1
     for (int lev = 0; lev < kStLev; ++lev, cur ^= 1) {
@@ -164,13 +153,13 @@ KS_DEV void plan_body(PlanSmem<N, M>& s, const PS& p, const ModelConst<N, M>& mc
             float cond;
             const bool ok = warp_inverse<N>(s.Mx, s.Mi, lane, cond);
             if (lane == 0 && !(ok && cond <= kRefineCond)) s.ok = 0;
-        } else {   // the powers, beside it
+        } else if (powers != nullptr) {
             for (int e = t - 32; e < NN; e += NT - 32) {
                 const int a = e / N, b = e % N;
-                out->EA[lev][e] = A[e];
+                powers->EA[lev][e] = A[e];
                 if (b <= a) {
-                    out->EC[lev][sidx(a, b)] = C[e];
-                    out->EJ[lev][sidx(a, b)] = J[e];
+                    powers->EC[lev][sidx(a, b)] = C[e];
+                    powers->EJ[lev][sidx(a, b)] = J[e];
                 }
             }
         }
@@ -199,6 +188,27 @@ KS_DEV void plan_body(PlanSmem<N, M>& s, const PS& p, const ModelConst<N, M>& mc
         }
         chain_sync();
     }
+    return cur;
+}
+
+// The plan of one model, by the chain's threads, from the FP32 constants mc and
+// the inputs in shared memory.
+template <int N, int M, class PS>
+KS_DEV void plan_body(PlanSmem<N, M>& s, const PS& p, const ModelConst<N, M>& mc, SteadyPlan<N, M>* __restrict__ out) {
+    constexpr int NN = N * N, NT = kChainThreads;
+    static_assert(NN <= 64 && N * M <= 32, "entries per warp of the single-warp stages");
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    for (int e = t; e < NN; e += NT) out->F[e] = mc.F[e];
+    for (int e = t; e < M * N; e += NT) out->H[e] = p.H[e / N][e % N];
+    for (int e = t; e < sym_size(N); e += NT) out->Q[e] = mc.Q[e];
+    for (int e = t; e < sym_size(M); e += NT) {
+        int a, b;
+        tri_rc(e, a, b);
+        out->R[e] = 0.5f * (p.R[a][b] + p.R[b][a]);
+    }
+    for (int e = t; e < N; e += NT) out->u[e] = mc.u[e];
+    for (int e = t; e < M; e += NT) out->d[e] = p.d[e];
+    const int cur = element_powers<N, M>(s, mc, nullptr);
     // ---- settled covariances, gains and Phi
     const float *A = s.A[cur], *P = s.C[cur], *J = s.J[cur];
     float *FPm = s.X, *Pm = s.Y, *Ph0 = s.A[cur ^ 1];
@@ -368,7 +378,7 @@ KS_DEV void plan_block(char* dsm, int sg, const PlanArgs<N, M>& g) {
         if (!(f < 1e18f)) f = 1e18f;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(0xffffffffu, f, o));
-        if (lane == 0) out->narrow = narrow ? 1 : 0;
+        if (lane == 0) out->narrow = s.narrow = narrow ? 1 : 0;
         const float n = s.Hh[0];
         // at every length: the head's closed forms hold for a fixed point P only
         const bool settled = s.settled != 0 && fmaxf(f, 1.f) * n * n <= kStCovTol;
@@ -381,6 +391,10 @@ KS_DEV void plan_block(char* dsm, int sg, const PlanArgs<N, M>& g) {
                 block_coef_warp<N, M>(mc, &p.H[0][0], g.ch, g.coef + sg);
         }
     }
+    // the powers, for a head from a narrow start only (stored beside the first
+    // doubling they cost every plan: 20 us of 1000 for 4096 sequences)
+    __syncthreads();
+    if (s.narrow && t < kChainThreads) element_powers<N, M>(s, mc, out);
 }
 
 template <int N, int M, bool FOLD>
@@ -797,7 +811,14 @@ KS_DEV void head_covs(SteadySmem<N, M>& sm, const SteadyPlan<N, M>* __restrict__
                 for (int i = 0; i < SY; ++i) { X[i] = D[i]; J[i] = n > 0 ? o[i] : 0.f; }
             }
             float Mi[N][N];
-            inverse_ixj<N>(X, J, Mi, bad);
+            if (it < 2) {
+                inverse_ixj<N>(X, J, Mi, bad);
+            } else {                                       // D = 0
+#pragma unroll
+                for (int a = 0; a < N; ++a)
+#pragma unroll
+                    for (int c = 0; c < N; ++c) Mi[a][c] = a == c ? 1.f : 0.f;
+            }
             if (it > 0) {
                 smoothed_cov<N>(P, Mi, J, pl.Pf, sc + (int64_t)(it == 1 ? k : len - 1 - k) * NN);
             } else if (it == 0 && k == 0) {
