@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(NW * 32) gfilter_reduce_kernel(const ModelCons
 template <int N, int NWS>
 __global__ void __launch_bounds__(NWS * 32) gspine_filter_kernel(const float* __restrict__ src, float* __restrict__ dst,
                                                                  int ntiles, int s, uint32_t* status, const uint32_t* gate) {
-    if (gate_closed(gate)) return;
+    if (gate_closed<false>(gate)) return;
     using SM = GSpineSmem<N, NWS>;
     constexpr int FS = Dim<N>::FSLOT;
     constexpr int SLOT = GChain<N>::SLOT;
@@ -484,7 +484,7 @@ template <int N, int NWS>
 __global__ void __launch_bounds__(NWS * 32) gspine_smoother_kernel(const float* __restrict__ src,
                                                                    float* __restrict__ dst, int ntiles, int s,
                                                                    uint32_t* status, const uint32_t* gate) {
-    if (gate_closed(gate)) return;
+    if (gate_closed<false>(gate)) return;
     using SM = GSpineSmem<N, NWS>;
     constexpr int SS = Dim<N>::SSLOT;
     constexpr int SLOT = GChain<N>::SLOT;

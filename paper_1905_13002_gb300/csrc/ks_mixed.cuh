@@ -68,9 +68,7 @@ KS_DEV void mixed_filter_tile(const MG6& g6, const MG4& g4, const MG2& g2, const
 // refines ill-conditioned inverses at once.
 template <int CH>
 __global__ void __launch_bounds__(kMixedThreads) mixed_filter_kernel(MG6 g6, MG4 g4, MG2 g2, MixedQueue q) {
-    pdl_trigger();
-    pdl_wait();
-    if (!general_wanted(q.status)) return;   // the settled path took every sequence
+    if (gate_closed<false>(q.status)) return;   // the settled path took every sequence
     mixed_filter_tile<CH>(g6, g4, g2, q);
 }
 
@@ -138,8 +136,7 @@ __global__ void __launch_bounds__(kMixedThreads, kRevMinBlocks<4>) mixed_smoothe
                                                                                        MixedQueue q) {
     __shared__ int s_tile;
     extern __shared__ __align__(16) char dsm[];
-    pdl_wait();
-    if (!general_wanted(q.status)) return;
+    if (gate_closed<false>(q.status)) return;
     if (threadIdx.x == 0) s_tile = (int)atomicAdd(q.scounter, 1u);
     __syncthreads();
     int t = s_tile;

@@ -492,7 +492,6 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
     RowSmem32& s = *reinterpret_cast<RowSmem32*>(dsm32);
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const Plan32& p = *g.s.plan;
-    pdl_trigger();
     pdl_wait();
     bool okp, narrow;
     {   // the chain's checks, and the transient of P_1 (relative to P) after 128 steps
@@ -507,6 +506,7 @@ __global__ void __launch_bounds__(kRowNT) rows32_kernel(Args32 g) {
         if (blockIdx.x == 0 && t == 0) atomicOr(g.status + HDR_GENERAL, 1u);
         return;
     }
+    pdl_trigger();   // not before: what follows is to know whether the plan passed (gate_closed)
     const int64_t T = g.T;
     if (blockIdx.x >= kS32Head) {
         // ---- eight chunks: one pass from the guess, what it misses the next chunk's guess by
@@ -732,7 +732,7 @@ __global__ void __launch_bounds__(kFwdNT) forward32_kernel(Args32 g) {
     FwdSmem32& s = *reinterpret_cast<FwdSmem32*>(dsm32);
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const Plan32& p = *g.s.plan;
-    pdl_trigger();
+    if (!general_wanted(g.status)) pdl_trigger();
     pdl_wait();
     if (general_set(g.status)) return;
     const int64_t T = g.T, nch = (T - kS32Head + kS32Chunk - 1) / kS32Chunk;
@@ -860,7 +860,7 @@ __global__ void __launch_bounds__(256, 2) reverse32_kernel(Args32 g) {
     __shared__ RevSmem32 s;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const Plan32& p = *g.s.plan;
-    pdl_trigger();
+    if (!general_wanted(g.status)) pdl_trigger();
     pdl_wait();
     if (general_set(g.status)) return;
     const int64_t T = g.T, nch = (T - kS32Head + kS32Chunk - 1) / kS32Chunk;

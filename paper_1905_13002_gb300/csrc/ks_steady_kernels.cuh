@@ -1103,6 +1103,7 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
         cp_async_wait_all();
         return;
     }
+    pdl_trigger();   // not before: what follows is to know whether the plans passed (gate_closed)
     {   // the plan (the head's part too for a head)
         using Core = SteadyCore<N, M>;
         const int n = (int)((head || last ? sizeof(Core) : offsetof(Core, W)) / 16);
@@ -1365,7 +1366,6 @@ constexpr int kSteadyMinBlocks = N <= 2 ? 4 : N <= 4 ? 3 : N <= 6 ? 2 : 1;
 template <int N, int M>
 __global__ void __launch_bounds__(kStNT, kSteadyMinBlocks<N>) steady_kernel(SteadyArgs<N, M> g) {
     extern __shared__ __align__(16) char dsm[];
-    pdl_trigger();
     steady_block<N, M>(dsm, g, (int64_t)blockIdx.x);
 }
 

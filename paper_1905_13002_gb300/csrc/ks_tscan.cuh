@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(NW * 32) tfilter_reduce_kernel(const ModelCons
 template <int N, int NWS>
 __global__ void __launch_bounds__(NWS * 32) tspine_filter_kernel(const float* __restrict__ src, float* __restrict__ dst,
                                                                  int ntiles, int s, uint32_t* status, const uint32_t* gate) {
-    if (gate_closed(gate)) return;
+    if (gate_closed<false>(gate)) return;
     using SM = SpineSmem<N, NWS, kSpineBufF>;
     constexpr int FR = Rec<N>::F;
     extern __shared__ __align__(16) char tsm[];
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(NW * 32) tsmoother_reduce_kernel(const ModelCo
 template <int N, int NWS>
 __global__ void __launch_bounds__(NWS * 32) tspine_smoother_kernel(const float* __restrict__ src, float* __restrict__ dst,
                                                                    int ntiles, int s, uint32_t* status, const uint32_t* gate) {
-    if (gate_closed(gate)) return;
+    if (gate_closed<false>(gate)) return;
     using SM = SpineSmem<N, NWS, kSpineBufS>;
     constexpr int SR = Rec<N>::S;
     extern __shared__ __align__(16) char tsm[];
