@@ -36,7 +36,8 @@ template <int K>
 struct Dims {
     static constexpr int Q = K + 4;
     static constexpr int SLOT = K * Q + K;       // rows, then log g
-    static constexpr int FREC = K * K + K;       // global filtering record: rows, then log g
+    static constexpr int OFF = K * K + K;        // global filtering record: rows, log g relative to
+    static constexpr int FREC = OFF + 4;         // an offset, the offset in FP64 (16 bytes kept for it)
 };
 
 // A chain is K lanes of one warp (lane z = row z); 32 / K chains per warp.  The
@@ -51,11 +52,16 @@ struct Const {
     float q1[K];   // p(x_1) = pi Pi
 };
 
-// One warp's share of a filtering element: lane z holds row z and lg[z].
+// One warp's share of a filtering element: lane z holds row z and log g(z) as
+// lg + off, lg relative to the element's largest and off common to its rows.
+// Kept as one FP32 number, a long prefix's log g (-1e5 and beyond) would leave no
+// bits for the differences between states, which weigh its rows (K = 8, 2^20 steps
+// of a nearly static chain: marginals 1e-3 off).
 template <int K>
 struct FRow {
     float f[K];
     float lg;
+    double off;
 };
 
 template <int K>
@@ -79,10 +85,13 @@ KS_DEV int group_max_i(int v) {
     return v;
 }
 
-// log g relative to its largest, all that beta needs: over a long suffix the
-// sum itself would leave no bits for the differences between states.
+// The largest of lg into the offset.
 template <int K>
-KS_DEV void relative_lg(FRow<K>& r) { r.lg -= group_max<K>(r.lg); }
+KS_DEV void relative_lg(FRow<K>& r) {
+    const float m = group_max<K>(r.lg);
+    r.lg -= m;
+    r.off += (double)m;
+}
 
 // Pi (pitch K) into shared memory.
 template <int K>
@@ -104,6 +113,7 @@ KS_DEV void load_frow(const float* __restrict__ src, FRow<K>& r) {
         r.f[4 * i + 3] = q.w;
     }
     r.lg = __ldcg(src + K * K + z);
+    r.off = __ldcg(reinterpret_cast<const double*>(src + Dims<K>::OFF));
 }
 
 template <int K>
@@ -113,6 +123,7 @@ KS_DEV void store_frow(float* __restrict__ dst, const FRow<K>& r) {
 #pragma unroll
     for (int i = 0; i < K / 4; ++i) p[i] = make_float4(r.f[4 * i], r.f[4 * i + 1], r.f[4 * i + 2], r.f[4 * i + 3]);
     dst[K * K + z] = r.lg;
+    if (z == 0) *reinterpret_cast<double*>(dst + Dims<K>::OFF) = r.off;
 }
 
 // A chain's element in a shared-memory slot (pitch Q rows, then lg).
@@ -238,9 +249,10 @@ KS_DEV void fold_end(FRow<K>& r, int ex, Flags& bad) {
     r.lg = fmaf((float)ex, 0.693147180559945f, logf(s));
 }
 
-// Definition 1, (row z of a_i, in registers) (x) a_j (in shared memory).
+// Definition 1, (row z of a_i, in registers) (x) a_j (in shared memory, its
+// offset offj).
 template <int K>
-KS_DEV void combine_row(FRow<K>& r, const float* __restrict__ ej, Flags& bad) {
+KS_DEV void combine_row(FRow<K>& r, const float* __restrict__ ej, double offj, Flags& bad) {
     float mx = ej[K * Dims<K>::Q];
 #pragma unroll
     for (int y = 1; y < K; ++y) mx = fmaxf(mx, ej[K * Dims<K>::Q + y]);
@@ -262,6 +274,8 @@ KS_DEV void combine_row(FRow<K>& r, const float* __restrict__ ej, Flags& bad) {
 #pragma unroll
     for (int x = 0; x < K; ++x) r.f[x] = o[x] * rd;
     r.lg += mx + __logf(d);
+    r.off += offj;
+    relative_lg<K>(r);
 }
 
 // The prefix (all rows equal) as a state: lane x takes p(x) from row 0.
@@ -274,7 +288,7 @@ KS_DEV void row0_state(const FRow<K>& r, float& p, float& L) {
         const float v = __shfl_sync(kFull, r.f[x], 0, K);
         if (lane == x) p = v;
     }
-    L = __shfl_sync(kFull, r.lg, 0, K);
+    L = (float)(r.off + (double)__shfl_sync(kFull, r.lg, 0, K));
 }
 
 // sum_x m[x] v(x) for a vector with v(x) on lane x, through the group's buffer
@@ -438,6 +452,7 @@ __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* 
             // log g relative to the chain's largest exponent, which is kept beside it
             const int top = group_max_i<K>(ex[r]);
             fold_end(fr[r], ex[r] - top, bad);
+            fr[r].off = 0.0;   // beta needs no offset
             put_frow(sm.slot[t], fr[r]);
             if (lane == 0) sm.top[t] = top;
             if (b.chain != nullptr && t < nvalid) store_frow(b.chain + (c0 + t) * Dims<K>::FREC, fr[r]);
@@ -448,24 +463,16 @@ __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* 
         FRow<K> acc;
         smem_row<Dims<K>::Q>(sm.slot[0], lane, acc.f);
         acc.lg = sm.slot[0][K * Dims<K>::Q + lane];
-        int top = sm.top[0];
+        constexpr double kLn2 = 0.69314718055994531;
+        acc.off = sm.top[0] * kLn2;
         const bool mine = w == 0;
-        auto absolute = [&](float* dst) {   // log g itself, for the prefixes
-            FRow<K> q = acc;
-            q.lg = fmaf((float)top, 0.693147180559945f, q.lg);
-            if (mine) store_frow(dst, q);
-        };
 #pragma unroll 1
         for (int t = 1; t < nvalid; ++t) {
-            absolute(b.fexcl + (c0 + t) * Dims<K>::FREC);
-            combine_row(acc, sm.slot[t], bad);
-            top += sm.top[t];
+            if (mine) store_frow(b.fexcl + (c0 + t) * Dims<K>::FREC, acc);
+            combine_row(acc, sm.slot[t], sm.top[t] * kLn2, bad);
         }
-        absolute(b.fspine0 + (int64_t)blockIdx.x * Dims<K>::FREC);
-        if (b.chain != nullptr) {
-            relative_lg<K>(acc);
-            if (mine) store_frow(b.sspine0 + (int64_t)blockIdx.x * Dims<K>::FREC, acc);
-        }
+        if (mine) store_frow(b.fspine0 + (int64_t)blockIdx.x * Dims<K>::FREC, acc);
+        if (b.chain != nullptr && mine) store_frow(b.sspine0 + (int64_t)blockIdx.x * Dims<K>::FREC, acc);
     }
     report_flags(status, bad, kFull, (threadIdx.x & 31) == 0);
 }
@@ -493,10 +500,10 @@ __global__ void __launch_bounds__(NW * 32) spine_kernel(const float* __restrict_
     FRow<K> r;   // every group combines; one without a partner copies instead
     load_frow(src + (int64_t)(comb ? right : 0) * REC, r);
     put_frow(slot[w], r);
+    const double offj = r.off;
     __syncwarp();
     load_frow(src + (int64_t)(comb ? left : 0) * REC, r);
-    combine_row(r, slot[w], comb ? bad : none);
-    if (!prefix) relative_lg<K>(r);
+    combine_row(r, slot[w], offj, comb ? bad : none);
     if (comb) {
         store_frow(dst + (int64_t)t * REC, r);
     } else if (in) {
@@ -538,7 +545,7 @@ __global__ void __launch_bounds__(NW * 32) filter_apply_kernel(const Const<K>* _
         put_frow(slot[w], e);
         __syncwarp();
         FRow<K> both = r;
-        combine_row(both, slot[w], has_tile && has_in ? bad : none);
+        combine_row(both, slot[w], e.off, has_tile && has_in ? bad : none);
         float p1, L1, p2, L2;
         row0_state(has_tile ? r : e, p1, L1);
         row0_state(both, p2, L2);
