@@ -178,9 +178,10 @@ KS_DEV void fadvance(FS<K>& st, const FE<K>& e, Flags& bad) {
 }
 
 // 2^-e and e for the exponent e of a positive finite r (r 2^-e in [1, 2); a
-// subnormal r keeps e = -127).
+// subnormal r keeps e = -127, and e is at most 126, since 2^-127 is no normal
+// number: r 2^-e lies in [2, 4) for the topmost r).
 KS_DEV float pow2_of(float r, int& e) {
-    e = (int)(__float_as_uint(r) >> 23) - 127;
+    e = min((int)(__float_as_uint(r) >> 23) - 127, 126);
     return __uint_as_float((uint32_t)(127 - e) << 23);
 }
 

@@ -154,9 +154,10 @@ KS_DEV void smem_row(const float* __restrict__ M, int y, float (&v)[K]) {
     }
 }
 
-// 2^-e and e for the exponent e of a positive finite r.
+// 2^-e and e for the exponent e of a positive finite r, at most 126 (2^-127 is no
+// normal number: r 2^-e lies in [2, 4) for the topmost r).
 KS_DEV float pow2_of(float r, int& e) {
-    e = (int)(__float_as_uint(r) >> 23) - 127;
+    e = min((int)(__float_as_uint(r) >> 23) - 127, 126);
     return __uint_as_float((uint32_t)(127 - e) << 23);
 }
 
@@ -366,7 +367,7 @@ struct Ahead {
     }
 };
 
-// Likelihood entries scaled by a power of two to a row maximum in [1, 2); le:
+// Likelihood entries scaled by a power of two (pow2_of) to a row maximum in [1, 2); le:
 // the exponents taken out.
 template <int K>
 KS_DEV void scale_rows(float (&lx)[kAhead], int (&le)[kAhead], Flags& bad) {
