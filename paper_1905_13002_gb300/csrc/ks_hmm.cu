@@ -208,17 +208,20 @@ struct WImpl {
 
 // Chains of 32 steps for shorter sequences (more of them than lane groups the
 // chip can hold only from there on), else of `LONG` steps: fewer tiles for the
-// spine's levels.  K = 8, 2^20 steps: 341 us one element per thread, 160 us here;
-// K = 32, 131072 steps: 1163 us with 64-step chains and Definition 2 elements,
-// 440 us.
+// spine's levels.  Up to 64 steps at K = 16 and 32 are one chain, which starts from
+// p(x_1): a later chain's rows start from every state, and a state that cannot
+// give the chain's measurements (an absorbing one, say) fails it.  K = 8, 2^20
+// steps: 341 us one element per thread, 160 us here; K = 32, 131072 steps: 1163 us
+// with 64-step chains and Definition 2 elements, 440 us.
 template <int K, int LONG>
 struct WSize {
     static constexpr int64_t kLong = 128 * 1024;
     static size_t bytes(int64_t T) { return std::max(WImpl<K, 32>::layout(T).bytes, WImpl<K, LONG>::layout(T).bytes); }
     static int smooth(const ks_hmm* h, const float* lik, int64_t T, void* ws, size_t ws_bytes, float* filt,
                       float* smooth, float* loglik, cudaStream_t st, void* const* ev) {
-        return T < kLong ? WImpl<K, 32>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev)
-                         : WImpl<K, LONG>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev);
+        return T < kLong && !(LONG == 64 && T > 32 && T <= LONG)
+                   ? WImpl<K, 32>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev)
+                   : WImpl<K, LONG>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev);
     }
 };
 using W8 = WSize<8, 128>;

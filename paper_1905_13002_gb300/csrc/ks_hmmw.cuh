@@ -206,7 +206,7 @@ KS_DEV void rows_times(const float* const (&f)[R], const float* __restrict__ M, 
 // exponent; on[r] false: nothing happens to chain r.
 template <int K, int R>
 KS_DEV void fold_rows(FRow<K> (&fr)[R], int (&ex)[R], const float* __restrict__ Pi, const float* const (&l)[R],
-                      const int (&le)[R], const bool (&on)[R], Flags& bad) {
+                      const int (&le)[R], const bool (&on)[R], Flags (&bad)[R]) {
     uint64_t acc[R][K / 2];
     const float* f[R];
 #pragma unroll
@@ -229,7 +229,7 @@ KS_DEV void fold_rows(FRow<K> (&fr)[R], int (&ex)[R], const float* __restrict__ 
         int e;
         const float rs = pow2_of(s, e);
         if (on[r]) {
-            bad |= !(s > 0.f);
+            bad[r] |= !(s > 0.f);
 #pragma unroll
             for (int x = 0; x < K; ++x) fr[r].f[x] = o[x] * rs;
             ex[r] += e + le[r];
@@ -401,8 +401,10 @@ __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* 
         Ahead<K> lk[R];
         float* buf[R];
         const float* cbuf[R];
+        Flags fbad[R];   // an absent chain folds the last one's steps from another row: its flags do not count
 #pragma unroll
         for (int r = 0; r < R; ++r) {
+            fbad[r] = 0u;
             const int64_t k0 = min(c0 + w * R + r, nch - 1) * CH;
             n[r] = (int)((k0 + CH < T ? k0 + CH : T) - k0);
             nmax = max(nmax, n[r]);
@@ -418,7 +420,7 @@ __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* 
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 lk[r].take(i0, lx[r]);
-                scale_rows<K>(lx[r], le[r], bad);
+                scale_rows<K>(lx[r], le[r], fbad[r]);
             }
 #pragma unroll
             for (int j = 0; j < kAhead; ++j) {
@@ -442,7 +444,7 @@ __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* 
                         lej[r] = le[r][j];
                         on[r] = i0 + j < n[r];
                     }
-                    fold_rows<K, R>(fr, ex, sm.Pi, cbuf, lej, on, bad);
+                    fold_rows<K, R>(fr, ex, sm.Pi, cbuf, lej, on, fbad);
                 }
             }
         }
@@ -452,7 +454,8 @@ __global__ void __launch_bounds__(NW * 32) filter_reduce_kernel(const Const<K>* 
             const int t = w * R + r;
             // log g relative to the chain's largest exponent, which is kept beside it
             const int top = group_max_i<K>(ex[r]);
-            fold_end(fr[r], ex[r] - top, bad);
+            fold_end(fr[r], ex[r] - top, fbad[r]);
+            if (t < nvalid) bad |= fbad[r];
             fr[r].off = 0.0;   // beta needs no offset
             put_frow(sm.slot[t], fr[r]);
             if (lane == 0) sm.top[t] = top;
