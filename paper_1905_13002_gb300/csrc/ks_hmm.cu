@@ -206,27 +206,29 @@ struct WImpl {
     }
 };
 
-// Chains of 32 steps for shorter sequences (more of them than lane groups the
-// chip can hold only from there on), else of `LONG` steps: fewer tiles for the
-// spine's levels.  Up to 64 steps at K = 16 and 32 are one chain, which starts from
-// p(x_1): a later chain's rows start from every state, and a state that cannot
-// give the chain's measurements (an absorbing one, say) fails it.  K = 8, 2^20
-// steps: 341 us one element per thread, 160 us here; K = 32, 131072 steps: 1163 us
-// with 64-step chains and Definition 2 elements, 440 us.
-template <int K, int LONG>
+// Chains of 32 steps below `LINE` steps, where the chip still has lane groups
+// to spare (32 / K chains a warp: the fewer states, the longer), else of `LONG`:
+// fewer tiles for the spine's levels.  Chains of 32 / of LONG, either side of
+// the lines: K = 8, 650000 steps 150 / 165 us, 786432 167 / 164, 2^21 318 / 280; K =
+// 16, 200003 177 / 186, 300000 209 / 208, 400000 266 / 252; K = 32, 70000 339 / 358,
+// 80000 406 / 410, 90000 454 / 423.  Up to 64 steps at K = 16 and 32 are one chain,
+// which starts from p(x_1): a later chain's rows start from every state, and a
+// state that cannot give the chain's measurements (an absorbing one, say) fails
+// it.  K = 8, 2^20 steps: 341 us one element per thread, 160 us here; K = 32, 131072
+// steps: 1163 us with 64-step chains and Definition 2 elements, 440 us.
+template <int K, int LONG, int64_t LINE>
 struct WSize {
-    static constexpr int64_t kLong = 128 * 1024;
     static size_t bytes(int64_t T) { return std::max(WImpl<K, 32>::layout(T).bytes, WImpl<K, LONG>::layout(T).bytes); }
     static int smooth(const ks_hmm* h, const float* lik, int64_t T, void* ws, size_t ws_bytes, float* filt,
                       float* smooth, float* loglik, cudaStream_t st, void* const* ev) {
-        return T < kLong && !(LONG == 64 && T > 32 && T <= LONG)
+        return T < LINE && !(LONG == 64 && T > 32 && T <= LONG)
                    ? WImpl<K, 32>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev)
                    : WImpl<K, LONG>::smooth(h, lik, T, ws, ws_bytes, filt, smooth, loglik, st, ev);
     }
 };
-using W8 = WSize<8, 128>;
-using W16 = WSize<16, 64>;
-using W32 = WSize<32, 64>;
+using W8 = WSize<8, 128, 768 * 1024>;
+using W16 = WSize<16, 64, 256 * 1024>;
+using W32 = WSize<32, 64, 80 * 1024>;
 
 }  // namespace
 }  // namespace hmm
