@@ -332,13 +332,15 @@ def main():
 
 
 def block_length(ks, nx: int, T: int) -> dict:
-    """Steps per thread the library uses for this call, whether full blocks
-    go through the linear block fold, and where the rule came from (the
-    tuner's cache for this device, or the built-in table)."""
+    """Steps per thread of this call's general scans, whether they fold full
+    blocks linearly, and where the rule came from (the tuner's cache for this
+    device, or the built-in table).  A time-invariant model that settles does
+    not run them."""
     from paper_1905_13002_gb300 import tune
     src = os.path.relpath(tune.APPLIED, ROOT) if tune.APPLIED else "built-in table"
     return {"steps_per_thread": ks.chunk_steps(nx, T) if nx <= 6 else None,
-            "block_fold": bool(ks.chunk_fold(nx, T)) if nx <= 6 else False, "rules": src}
+            "block_fold": bool(ks.chunk_fold(nx, T)) if nx <= 6 else False, "rules": src,
+            "of": "the general scans (closed behind the settled path when the model settles)"}
 
 
 def launches_per_call(nx: int, T: int) -> int:

@@ -696,7 +696,9 @@ __global__ void __launch_bounds__(kTvThreads<N>) tv_const_kernel(TVArgs tv, int6
         for (int e = r; e < 4; e += GS) mc.pad[e] = 0.f;
         gsync<N>();
     }
-    pdl_wait();                                               // step 0's preparation clears the status word
+    // not before the end: the steps need nothing of step 0's preparation, but when
+    // this kernel is done the chained launches behind it take that one for done too
+    pdl_wait();
     report_flags(status, bad, gmask<N>(), r == 0);
 }
 

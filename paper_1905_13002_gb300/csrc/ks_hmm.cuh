@@ -90,14 +90,15 @@ KS_DEV void set_identity(FE<K>& e) {
     }
 }
 
-// Likelihood row of step k scaled to a maximum of 1; returns log of the
-// maximum (a row with no positive finite maximum is flagged).
+// Likelihood row of step k.
 template <int K>
 KS_DEV void load_raw(const float* __restrict__ src, int64_t k, float (&v)[K]) {
 #pragma unroll
     for (int x = 0; x < K; ++x) v[x] = __ldg(src + k * K + x);
 }
 
+// The row scaled to a maximum of 1; returns log of the maximum (a row with no
+// positive finite maximum is flagged).
 template <int K>
 KS_DEV float scale_lik(float (&l)[K], Flags& bad) {
     float m = 0.f;
@@ -108,12 +109,6 @@ KS_DEV float scale_lik(float (&l)[K], Flags& bad) {
 #pragma unroll
     for (int x = 0; x < K; ++x) l[x] *= r;
     return __logf(m);
-}
-
-template <int K>
-KS_DEV float load_lik(const float* __restrict__ lik, int64_t k, float (&l)[K], Flags& bad) {
-    load_raw<K>(lik, k, l);
-    return scale_lik<K>(l, bad);
 }
 
 // Definition 1, a_i (x) a_j for general elements (i earlier).  With

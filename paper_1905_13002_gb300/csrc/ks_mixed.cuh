@@ -59,7 +59,7 @@ constexpr int kMixedThreads = 128;
 // groups (nx = 6 sequences first; it also zeroes the queue counters), and the
 // settled path, one launch per state size (ks_steady_mixed.cu).
 int launch_mixed_plan(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, bool fold, cudaStream_t st);
-int launch_mixed_steady(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q, cudaStream_t st);
+int launch_mixed_steady(const MG6& g6, const MG4& g4, const MG2& g2, cudaStream_t st);
 
 template <int CH>
 KS_DEV void mixed_filter_tile(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue& q);
@@ -237,7 +237,7 @@ struct Mixed {
         if (!ok) return KS_ECUDA;
         int rc = launch_mixed_plan(g6, g4, g2, q, fold, st);
         if (rc) return rc;
-        if ((rc = launch_mixed_steady(g6, g4, g2, q, st))) return rc;
+        if ((rc = launch_mixed_steady(g6, g4, g2, st))) return rc;
         rc = launch_pdl(mixed_filter_kernel<CH>, ntiles, kMixedThreads, mixed_filter_smem(), st, g6, g4, g2, q);
         if (rc) return rc;
         return launch_pdl(mixed_smoother_kernel<CH>, ntiles, kMixedThreads, mixed_smoother_smem(), st, g6, g4, g2, q);

@@ -1125,8 +1125,7 @@ KS_DEV void steady_block(char* dsm, const SteadyArgs<N, M>& g, int64_t slot) {
     __syncthreads();
     // Issued in kFill slices between the passes, each copy by another warp: the
     // copies go out no faster than the memory takes them, and a warp that
-    // issues them all at once keeps the block waiting at its next barrier
-    // (3.2 of 7.8 stall cycles per instruction at nx = 4, T = 2^20).
+    // issues them all at once keeps the block waiting at its next barrier.
     constexpr int kFill = 6;
     const int nf = fillf ? (o1 - o0 + PR - 1) / PR : 0, ns = fills ? (s1 - o0 + PR - 1) / PR : 0;
     auto fill = [&](int slice) {

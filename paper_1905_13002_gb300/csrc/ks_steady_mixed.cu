@@ -64,7 +64,7 @@ int launch_mixed_plan(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQu
     return launch_status();
 }
 
-int launch_mixed_steady(const MG6& g6, const MG4& g4, const MG2& g2, const MixedQueue&, cudaStream_t st) {
+int launch_mixed_steady(const MG6& g6, const MG4& g4, const MG2& g2, cudaStream_t st) {
     int rc = KS_OK;
     if (g6.B && (rc = launch_steady_kernel(steady_args(g6), st))) return rc;
     if (g4.B && (rc = launch_steady_kernel(steady_args(g4), st))) return rc;
