@@ -172,15 +172,15 @@ KS_DEV void fadvance(FS<K>& st, const FE<K>& e, Flags& bad) {
     st.L += mx + __logf(d);
 }
 
-// 2^-e and e for the exponent e of a positive finite r (r 2^-e in [1, 2); a
-// subnormal r keeps e = -127, and e is at most 126, since 2^-127 is no normal
-// number: r 2^-e lies in [2, 4) for the topmost r).
+// 2^-e and e for the exponent e of a positive r < 2^127 (r 2^-e in [1, 2); a
+// subnormal r keeps e = -127; 2^-127 is no normal number).
 KS_DEV float pow2_of(float r, int& e) {
-    e = min((int)(__float_as_uint(r) >> 23) - 127, 126);
+    e = (int)(__float_as_uint(r) >> 23) - 127;
     return __uint_as_float((uint32_t)(127 - e) << 23);
 }
 
-// Likelihood row scaled by a power of two to a maximum in [1, 2); returns the
+// Likelihood row scaled by a power of two to a maximum in [1, 2), the topmost
+// (2^127 and above) to [2, 4); returns the
 // exponent taken out.
 template <int K>
 KS_DEV int scale_lik2(float (&l)[K], Flags& bad) {
@@ -190,7 +190,7 @@ KS_DEV int scale_lik2(float (&l)[K], Flags& bad) {
     const bool ok = m > 0.f && m <= 3.0e38f;
     bad |= !ok;
     int e;
-    const float s = pow2_of(ok ? m : 1.f, e);
+    const float s = pow2_of(ok ? fminf(m, 1.7e38f) : 1.f, e);
 #pragma unroll
     for (int x = 0; x < K; ++x) l[x] *= s;
     return e;

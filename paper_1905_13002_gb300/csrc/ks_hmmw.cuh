@@ -154,10 +154,9 @@ KS_DEV void smem_row(const float* __restrict__ M, int y, float (&v)[K]) {
     }
 }
 
-// 2^-e and e for the exponent e of a positive finite r, at most 126 (2^-127 is no
-// normal number: r 2^-e lies in [2, 4) for the topmost r).
+// 2^-e and e for the exponent e of a positive r < 2^127 (2^-127 is no normal number).
 KS_DEV float pow2_of(float r, int& e) {
-    e = min((int)(__float_as_uint(r) >> 23) - 127, 126);
+    e = (int)(__float_as_uint(r) >> 23) - 127;
     return __uint_as_float((uint32_t)(127 - e) << 23);
 }
 
@@ -367,7 +366,8 @@ struct Ahead {
     }
 };
 
-// Likelihood entries scaled by a power of two (pow2_of) to a row maximum in [1, 2); le:
+// Likelihood entries scaled by a power of two to a row maximum in [1, 2), the
+// topmost (2^127 and above) to [2, 4); le:
 // the exponents taken out.
 template <int K>
 KS_DEV void scale_rows(float (&lx)[kAhead], int (&le)[kAhead], Flags& bad) {
@@ -376,7 +376,7 @@ KS_DEV void scale_rows(float (&lx)[kAhead], int (&le)[kAhead], Flags& bad) {
         const float m = group_max<K>(lx[j]);
         const bool ok = m > 0.f && m <= 3.0e38f && lx[j] <= 3.0e38f;
         bad |= !ok;
-        lx[j] *= pow2_of(ok ? m : 1.f, le[j]);
+        lx[j] *= pow2_of(ok ? fminf(m, 1.7e38f) : 1.f, le[j]);
     }
 }
 
