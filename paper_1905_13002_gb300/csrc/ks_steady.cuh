@@ -40,7 +40,7 @@
 // scans before and this after: nx = 4, 2^20 steps 229 -> 70 us (2.6 TB/s of the
 // 6.8 a copy reaches; the rest is the plan's and the head's latency, 13 and 20
 // us); 1024 steps 50 -> 41 us; nx = 6, 100003 steps filtered 177 -> 59 us; 24 nx
-// = 8 sequences 1071 -> 210 us; 4096 mixed sequences 5.4 -> 1.0 ms.  Every length
+// = 8 sequences 1071 -> 217 us; 4096 mixed sequences 5.4 -> 1.0 ms.  Every length
 // takes it: at 1024 steps it is the plan and one block, still less than the
 // scans.  A head of 128 rows: one thread per row, seven doublings; 2048-row
 // windows give 16 steps per thread, a quarter of them halo.
